@@ -16,7 +16,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libwri.so")
-SOURCES = ["wri_api.cu", "wri_k32.cu", "wri_k64.cu", "wri_small.cu", "wri_k32_tma.cu"]
+SOURCES = ["wri_api.cu", "wri_k32.cu", "wri_k64.cu", "wri_small.cu", "wri_k32_tma.cu", "wri_lin.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden"]
 

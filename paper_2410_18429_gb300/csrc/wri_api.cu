@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <complex>
 #include <cstdlib>
 #include <cstring>
 #include <memory>
@@ -16,6 +17,7 @@
 
 #include "../../include/wri.h"
 #include "wri_launch.h"
+#include "wri_lin.cuh"
 #include "wri_tma.cuh"
 
 using namespace wri;
@@ -23,15 +25,19 @@ using namespace wri;
 namespace {
 
 constexpr int kRefSMs = 152;  // SMs of a GB300; sets the z-split of small batches
-// Measured defaults of the TMA phases on GB300 (128 sources x 3 frequency grids): the
-// warp-specialised kernel (a copy warp and 4 consumer warps, two nodes per thread, 32 x 8
-// tiles, 4 stages, 4 CTAs/SM); work items in blocks of 16 systems (neighbouring tiles of a
-// system run together, so their halos meet in L2); L2 fills of 64 bytes on a copy miss
-// (128-byte fills over-fetch the halo columns).  wri_autotune refines the choice per batch.
-constexpr int kDefaultTmaCfg = 9;
+// Measured defaults on GB300: the chunk kernels with x updated every fourth iteration (configuration
+// 24; 64 sources x 3 frequency grids, 24 iterations: 126 ms against 131 with an update every second
+// iteration and 169 on the TMA boxes of configuration 9); where they cannot run, the warp-specialised
+// boxes; work items in blocks of 16 systems (neighbouring tiles of a system run together, so their
+// halos meet in L2; 126 ms against 128 for blocks of 8 and 131 for all systems of a tile in a row); L2
+// fills of 64 bytes on a TMA miss (128-byte fills over-fetch the halo columns of the boxes).
+// wri_autotune refines the choice per batch.
+constexpr int kDefaultTmaCfg = 24;
+constexpr int kBoxTmaCfg = 9;   // where the chunk kernels cannot run (see plan_solve)
 constexpr int kFirstWsCfg = 9;  // configurations from here on are the warp-specialised kernels
 constexpr int kDefaultOrder = 6;
 constexpr int kDefaultPromotion = 2;
+constexpr int kGradPlanes = 16;  // planes of a z-chunk of the gradient, at most (its sums: 32 KB of shared memory)
 constexpr size_t kAlign = 256;
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
@@ -93,12 +99,34 @@ void fill_geom(GroupDev& G, const wri_grid& g) {
   G.npml = g.npml;
   G.h = g.h;
   G.omega = g.omega;
+  G.ih2 = 1.0 / (g.h * g.h);
+  G.om2 = g.omega * g.omega;
   G.ih2f = (float)(1.0 / (g.h * g.h));
   G.om2f = (float)(g.omega * g.omega);
   G.ax = axis(g.nx, g);
   G.ay = axis(g.ny, g);
   G.az = axis(g.nz, g);
   G.n = grid_n(g);
+}
+
+// Layer table of the chunk kernels (kLayerTab): entries for nodes 0 .. npml cells inside the layer, in FP64.
+// The same entries serve the three axes and both faces, since the profile depends on the distance alone.
+void layer_table(const wri_grid& g, std::vector<double>& t) {
+  typedef std::complex<double> Z;
+  t.assign((size_t)(g.npml + 1) * kLayerTab, 0.0);
+  const AxisPml a = axis(g.nx, g);
+  auto stretch = [&](double cells) -> Z {
+    const double q = std::max(cells, 0.0) * a.h * a.invL;
+    return Z(1.0, a.smax * q * q * a.inv_omega);
+  };
+  for (int d = 0; d <= g.npml; ++d) {
+    const Z s = stretch(d), ih2 = Z(1.0 / (g.h * g.h), 0.0);
+    const Z near_ = ih2 / stretch(d - 0.5), far_ = ih2 / stretch(d + 0.5);
+    const Z an = near_ / s, af = far_ / s, a0 = -(an + af);
+    const double e[kLayerTab] = {an.real(), an.imag(), af.real(), af.imag(), a0.real(), a0.imag(), s.imag(), 0.0,
+                                 near_.real(), near_.imag(), far_.real(), far_.imag()};
+    std::copy(e, e + kLayerTab, t.begin() + (size_t)d * kLayerTab);
+  }
 }
 
 // tiles_x, tiles_y, zsplit, zc of a grid for a given batch size
@@ -109,6 +137,22 @@ void decompose(const wri_grid& g, int by, int zs_req, GroupDev& G) {
   G.zc = (g.nz + zs - 1) / zs;
   G.zsplit = (g.nz + G.zc - 1) / G.zc;
   G.ntiles = G.tiles_x * G.tiles_y * G.zsplit;
+  G.rw = (g.nx + 31) / 32;
+}
+
+// The same for the chunk kernels: equal chunks of at most kLinChunk nodes of the x-y plane.
+int lin_chunks(const wri_grid& g) { return (int)(((long long)g.nx * g.ny + kLinChunk - 1) / kLinChunk); }
+
+void decompose_lin(const wri_grid& g, int zs, GroupDev& G) {
+  const int zs_req = std::max(1, std::min(zs, g.nz));
+  const int plane = g.nx * g.ny, nch = lin_chunks(g);
+  G.chunk = ((plane + nch - 1) / nch + 31) / 32 * 32;
+  G.tiles_x = (plane + G.chunk - 1) / G.chunk;
+  G.tiles_y = 1;
+  G.zc = (g.nz + zs_req - 1) / zs_req;
+  G.zsplit = (g.nz + G.zc - 1) / G.zc;
+  G.ntiles = G.tiles_x * G.zsplit;
+  G.rw = (g.nx + 31) / 32;
 }
 
 // z-chunks per tile column when the caller leaves it open: the count that minimises the modelled
@@ -124,6 +168,25 @@ int auto_zsplit(long long xy_items, int nz) {
     const int zc = (nz + zs - 1) / zs;
     const long long items = xy_items * ((nz + zc - 1) / zc);
     const double cost = (double)((items + wave - 1) / wave) * (zc + 2);
+    if (zs == 1 || cost < best_cost) {
+      best_cost = cost;
+      best = zs;
+    }
+  }
+  return best;
+}
+
+// The same for the chunk kernels, with chunks of at least one plane.  complex64: waves of 4 CTAs per SM
+// times the planes an item streams.  complex128: the FP64 pipe binds, so the planes per SM count, and a
+// little for the planes next to the chunk.
+int auto_zsplit_lin(long long xy_items, int nz, bool wide) {
+  int best = 1;
+  double best_cost = 0.0;
+  for (int zs = 1; zs <= 64 && zs <= nz; ++zs) {
+    const int zc = (nz + zs - 1) / zs;
+    const long long items = xy_items * ((nz + zc - 1) / zc);
+    const long long wave = (long long)kRefSMs * (wide ? 1 : 4);
+    const double cost = (double)((items + wave - 1) / wave) * (wide ? zc : zc + 2) + (wide ? 0.3 * (zc + 2) : 0.0);
     if (zs == 1 || cost < best_cost) {
       best_cost = cost;
       best = zs;
@@ -164,14 +227,19 @@ int validate_groups(const wri_group* groups, int ngroups, bool need_data) {
 struct Plan {
   int ngroups = 0, nsys_total = 0, nnz_total = 0, dtype = 0, ir = 0, by = 8;
   int tma_cfg = -1;  // TMA configuration of the CG phases, -1 = z-march kernels
+  bool lin = false;  // chunk kernels instead of the TMA or z-march kernels
+  int pair = 0;      // Batch::pair
+  int xsteps = 1;    // chunk kernels: iterations per iterate update
   bool host_loop = false;  // the host replays the iteration graph (no conditional node)
   int vbytes = 8;   // bytes of one complex of the iteration vectors
   int rlbytes = 8;  // bytes of one complex of lamd / r2
   long long nitems = 0;
   long long nparts = 0;
+  long long xitems = 0;
   size_t off_sys = 0, off_rec = 0, off_part = 0, off_rem = 0, off_lamd = 0, off_r2 = 0;
   size_t off_r2_64 = 0, off_r2_in = 0;  // refinement: FP64 receiver residual master, complex64 inner r2
-  size_t aux_total = 0, total = 0;
+  size_t off_ltab32[WRI_MAXG], off_ltab64[WRI_MAXG];  // layer tables of the chunk kernels
+  size_t aux_base = 0, aux_total = 0, total = 0;  // aux_base: without the layer tables
   GroupDev g[WRI_MAXG];
   size_t v_r1[WRI_MAXG][2], v_p[WRI_MAXG][4], v_s[WRI_MAXG], v_t1[WRI_MAXG];
   int pslots = 2;  // search-direction slots: 4 when the phases may update x every fourth iteration
@@ -202,6 +270,14 @@ void plan_aux(const wri_group* groups, int ngroups, Plan& P) {
     P.off_ztab64[gi] = off;
     off += align_up(sizeof(double) * 2 * 2 * 3 * (size_t)groups[gi].grid.nz);
   }
+  P.aux_base = off;
+  for (int gi = 0; gi < ngroups; ++gi) {  // layer tables of the chunk kernels
+    const size_t e = (size_t)kLayerTab * (groups[gi].grid.npml + 1);
+    P.off_ltab32[gi] = off;
+    off += align_up(sizeof(float) * e);
+    P.off_ltab64[gi] = off;
+    off += align_up(sizeof(double) * e);
+  }
   P.aux_total = off;
   P.total = off;
 }
@@ -214,6 +290,15 @@ bool host_loop_forced() {
   return forced;
 }
 
+// TMA configurations whose phases are the chunk kernels: 18 and 22 (two direction slots, x updated every
+// second iteration) and 24, the automatic choice (four slots, every fourth iteration).  Complex128 batches
+// and x extents that are not multiples of 4, which the TMA boxes cannot take, run on them too unless
+// z-march kernels or a z-march tile are asked for.  Microseconds per system and iteration against the
+// boxes of configuration 9 (and of 24): 148^3 x 32 systems 46.9 (58.6, 52.5), 116^3 x 32 22.6 (31.4, 28.7),
+// 84^3 x 64 9.0 (12.3, 11.2), one 148^3 82 (92, 86); against the z-march kernels on 81^3 x 9 with 2025
+// receivers: 13 (41) in complex64.
+bool lin_config(int cfg) { return cfg == 18 || cfg == 22 || cfg == 24; }
+
 void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, Plan& P) {
   plan_aux(groups, ngroups, P);
   P.dtype = o->dtype;
@@ -221,41 +306,70 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
   P.ir = (o->dtype == WRI_C64 && o->max_refine > 0) ? 1 : 0;
   P.by = by_of_tile(o->tile);
   P.tma_cfg = -1;
-  if (!o->plain && o->kernel != 1 && o->dtype == WRI_C64) {
-    bool ok = true;
-    // the refinement's inner iterate lives in the workspace; otherwise the TMA phases update u
-    for (int gi = 0; gi < ngroups; ++gi)
-      ok = ok && (groups[gi].grid.nx % 4 == 0) && (P.ir || (uintptr_t)groups[gi].u % 16 == 0);
-    if (ok) {
-      P.tma_cfg = o->kernel >= 2 ? o->kernel - 2 : kDefaultTmaCfg;
-      // the refinement's inner phase 2 adds S^H r64, which only the warp-specialised kernels do
-      if (P.ir && P.tma_cfg < kFirstWsCfg) P.tma_cfg = kDefaultTmaCfg;
-      P.by = tma_config_by(P.tma_cfg);
-      // a ring of four directions for the configurations that update x every fourth iteration; the
-      // automatic choice reserves it too, so that wri_autotune may pick them in the same workspace
-      P.pslots = (o->kernel == 0 || tma_config_xsteps(P.tma_cfg) == 4) ? 4 : 2;
+  P.lin = false;
+  bool boxes = !o->plain && o->kernel != 1 && o->dtype == WRI_C64;
+  // the refinement's inner iterate lives in the workspace; otherwise the TMA phases update u
+  for (int gi = 0; gi < ngroups; ++gi)
+    boxes = boxes && (groups[gi].grid.nx % 4 == 0) && (P.ir || (uintptr_t)groups[gi].u % 16 == 0);
+  const int cfg = o->kernel >= 2 ? o->kernel - 2 : kDefaultTmaCfg;
+  if (!o->plain && o->kernel != 1 && lin_config(cfg) && (boxes || o->tile == 0)) {
+    P.lin = true;
+    P.pair = o->dtype == WRI_C64 ? 1 : 0;
+    Batch probe;
+    probe.ngroups = ngroups;
+    for (int gi = 0; gi < ngroups; ++gi) {
+      const wri_grid& g = groups[gi].grid;
+      const size_t cb = o->dtype == WRI_C128 ? 16 : 8;
+      P.lin = P.lin && (long long)g.nx * g.ny < (1LL << 28) && (uintptr_t)groups[gi].m % (cb / 2) == 0 &&
+              (uintptr_t)groups[gi].u % cb == 0;
+      P.pair = P.pair && g.nx % 2 == 0 && (uintptr_t)groups[gi].m % 8 == 0 &&
+               (P.ir || (uintptr_t)groups[gi].u % 16 == 0);
+      probe.g[gi].nx = g.nx;
+      probe.g[gi].ny = g.ny;
+      probe.g[gi].zc = 0;
+      probe.g[gi].m_double = o->dtype == WRI_C128 ? 1 : 0;
     }
+    P.lin = P.lin && lin_smem(probe, (o->dtype == WRI_C128 || P.ir) ? 8 : 4, M_P1) <= (size_t)kLinMaxSmem;
+  }
+  if (P.lin) {
+    // complex128 keeps two direction slots: the same bytes per iteration as an update in every one
+    P.pslots = (o->dtype == WRI_C64 && cfg == 24) ? 4 : 2;
+    P.xsteps = P.pslots;
+  } else if (boxes) {
+    P.tma_cfg = o->kernel >= 2 ? o->kernel - 2 : kBoxTmaCfg;
+    // the refinement's inner phase 2 adds S^H r64, which only the warp-specialised kernels do
+    if (P.ir && P.tma_cfg < kFirstWsCfg) P.tma_cfg = kBoxTmaCfg;
+    P.by = tma_config_by(P.tma_cfg);
+    // a ring of four directions for the configurations that update x every fourth iteration; the
+    // automatic choice reserves it too, so that wri_autotune may pick them in the same workspace
+    P.pslots = (o->kernel == 0 || tma_config_xsteps(P.tma_cfg) == 4) ? 4 : 2;
   }
   P.vbytes = (o->dtype == WRI_C128) ? 16 : 8;
   P.rlbytes = (o->dtype == WRI_C128 || P.ir) ? 16 : 8;
   long long xy_items = 0;
   for (int gi = 0; gi < ngroups; ++gi) {
     const wri_grid& g = groups[gi].grid;
-    xy_items += (long long)groups[gi].nsys * ((g.nx + WRI_TX - 1) / WRI_TX) * ((g.ny + P.by - 1) / P.by);
+    xy_items += (long long)groups[gi].nsys *
+                (P.lin ? lin_chunks(g) : ((g.nx + WRI_TX - 1) / WRI_TX) * ((g.ny + P.by - 1) / P.by));
   }
   int nz_max = 0;
   for (int gi = 0; gi < ngroups; ++gi) nz_max = std::max(nz_max, groups[gi].grid.nz);
   const int zs = o->zsplit > 0 ? o->zsplit
+                 : P.lin       ? auto_zsplit_lin(xy_items, nz_max, o->dtype == WRI_C128)
                                : auto_zsplit(o->plain ? xy_items / std::max(1, P.nsys_total) : xy_items, nz_max);
   long long item = 0, parts = 0;
   int sys0 = 0;
+  P.xitems = 0;
   for (int gi = 0; gi < ngroups; ++gi) {
     GroupDev& G = P.g[gi];
     std::memset(&G, 0, sizeof(G));
     fill_geom(G, groups[gi].grid);
-    decompose(groups[gi].grid, P.by, zs, G);
+    if (P.lin) decompose_lin(groups[gi].grid, zs, G);
+    else decompose(groups[gi].grid, P.by, zs, G);
     G.nsys = groups[gi].nsys;
     G.sys0 = sys0;
+    G.xitem0 = P.xitems;
+    P.xitems += (long long)G.nsys * ((G.n + kXupdNodes - 1) / kXupdNodes);
     G.item0 = item;
     G.nitems = (long long)G.ntiles * G.nsys;
     item += G.nitems;
@@ -282,7 +396,7 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
   }
   for (int gi = 0; gi < ngroups; ++gi) {  // receiver bitmaps (one bit per node and system)
     const GroupDev& G = P.g[gi];
-    P.rcol_bytes[gi] = 4 * (size_t)G.nsys * G.ny * G.tiles_x;
+    P.rcol_bytes[gi] = 4 * (size_t)G.nsys * G.ny * G.rw;
     P.rmask_bytes[gi] = P.rcol_bytes[gi] * (size_t)G.nz;
     P.off_rcol[gi] = off;
     off += align_up(P.rcol_bytes[gi]);
@@ -463,6 +577,13 @@ cudaError_t march(int rbytes, int obytes, int mode, bool conj, int by, const Bat
   return launch_march_f64_to_f32(mode, by, b, 0, st);
 }
 
+// A set-up or residual pass of a solve, on the kernels of its plan.
+cudaError_t stencil_pass(const Plan& P, int rbytes, int obytes, int mode, const Batch& b, const LinWait& w,
+                         cudaStream_t st) {
+  if (P.lin) return launch_lin(rbytes, obytes, mode, mode == M_SH, b, w, nullptr, 0, st);
+  return march(rbytes, obytes, mode, mode == M_SH, P.by, b, st);
+}
+
 // Base batch for the solver: geometry, workspace pointers, per-group vector views.
 Batch solver_batch(const wri_group* groups, const Plan& P, char* ws, bool inner_view) {
   Batch b;
@@ -510,8 +631,13 @@ Batch solver_batch(const wri_group* groups, const Plan& P, char* ws, bool inner_
     G.ztab64 = (const double2*)(ws + P.off_ztab64[gi]);
     G.rmask = (const uint32_t*)(ws + P.off_rmask[gi]);
     G.rcol = (const uint32_t*)(ws + P.off_rcol[gi]);
+    G.ltab32 = (const float*)(ws + P.off_ltab32[gi]);
+    G.ltab64 = (const double*)(ws + P.off_ltab64[gi]);
     b.g[gi] = G;
   }
+  b.pair = P.pair;
+  b.xsteps = P.xsteps;
+  b.xitems = P.xitems;
   return b;
 }
 
@@ -522,6 +648,32 @@ int setup_rmask(const Plan& P, const Batch& b, char* ws, cudaStream_t st) {
     WRI_CK(cudaMemsetAsync(ws + P.off_rmask[gi], 0, P.rmask_bytes[gi], st));
   }
   WRI_CK(launch_rmask(b, P.nsys_total, st));
+  return WRI_OK;
+}
+
+// s = S^H b of the chunk kernels: flavor SH_INIT starts a solve (r1 = b1, x = 0), SH_REF only forms the
+// reference norm.  A point right-hand side needs no pass over the grid; a general one is copied into r1
+// (widened where the pass is in FP64) and goes through the stencil.
+int lin_rhs(const Plan& P, const Batch& b, int rbytes, int obytes, const LinWait& w, cudaStream_t st) {
+  const bool init = b.flavor == SH_INIT;
+  bool field = false;
+  for (int gi = 0; gi < P.ngroups; ++gi) field = field || b.g[gi].q;
+  for (int gi = 0; gi < P.ngroups; ++gi) {
+    const GroupDev& G = b.g[gi];
+    const size_t cnt = (size_t)G.nsys * (size_t)G.n;
+    if (init) WRI_CK(cudaMemsetAsync(G.x, 0, 2 * rbytes * cnt, st));
+    if (G.q && rbytes == 8 && !G.q_double) {
+      WRI_CK(launch_widen(G.q, G.r1[0], (long long)cnt, st));
+    } else if (G.q) {
+      WRI_CK(cudaMemcpyAsync(G.r1[0], G.q, 2 * rbytes * cnt, cudaMemcpyDeviceToDevice, st));
+    } else if (init || field) {
+      WRI_CK(cudaMemsetAsync(G.r1[0], 0, 2 * rbytes * cnt, st));
+      if (field && G.alpha) WRI_CK(launch_point_field(rbytes, b, gi, st));
+    }
+    if (init && !field) WRI_CK(cudaMemsetAsync(G.s, 0, 2 * obytes * cnt, st));
+  }
+  if (field) WRI_CK(launch_lin(rbytes, obytes, M_SH, true, b, w, nullptr, 0, st));
+  else WRI_CK(launch_init_point(rbytes, obytes, b, P.nsys_total, st));
   return WRI_OK;
 }
 
@@ -624,10 +776,15 @@ bool device_loop_supported() {
 
 // Captures K CG iterations (phase 1 + phase 2 launches) on c->cap into whatever capture is open.
 cudaError_t capture_iterations(const Plan& P, const Batch& b1, const Batch& b2, int mode2, int K, int rb,
-                               bool use_tma, const TmaSet* tma, cudaStream_t cap) {
+                               bool use_tma, const TmaSet* tma, const LinWait* lin, cudaStream_t cap) {
   cudaError_t err = cudaSuccess;
   for (int k = 0; k < K && err == cudaSuccess; ++k) {
-    if (use_tma) {
+    if (P.lin) {
+      const LinWait w = {b1.remaining + 1, lin->wait_ns, lin->withhold};
+      err = launch_lin(rb, rb, M_P1, false, b1, w, nullptr, 0, cap);
+      if (err == cudaSuccess) err = launch_lin(rb, rb, M_P2, true, b2, w, nullptr, 0, cap);
+      if (err == cudaSuccess && ((k + 1) % P.xsteps == 0 || k + 1 == K)) err = launch_xupdate(rb, b1, cap);
+    } else if (use_tma) {
       err = launch_phase_tma(M_P1, P.tma_cfg, b1, *tma, 0, cap);
       if (err == cudaSuccess) err = launch_phase_tma(M_P2, P.tma_cfg, b2, *tma, 0, cap);
     } else {
@@ -645,7 +802,7 @@ cudaError_t capture_iterations(const Plan& P, const Batch& b1, const Batch& b2, 
 // the counters after every replay.)  The workspace counters are: [0] systems not yet done, [1] the
 // copy-wait error flag, [2] loop bodies run.
 int run_loop(const Plan& P, const Batch& b1_in, const Batch& b2_in, int mode2, int K, int max_iter, cudaStream_t st,
-             const TmaSet* tma = nullptr) {
+             const TmaSet* tma, const LinWait* lin) {
   DevCtx* c = ctx();
   int* slot = poll_slot();
   if (!c || !slot) return WRI_ECUDA;
@@ -654,19 +811,23 @@ int run_loop(const Plan& P, const Batch& b1_in, const Batch& b2_in, int mode2, i
   // iterate updates every m-th iteration: only the grouped-update configurations' phase-1 kernel
   // does them (m = 4 needs the four direction slots)
   Batch b1 = b1_in, b2 = b2_in;
-  int xs = use_tma ? tma_config_xsteps(P.tma_cfg) : 1;
+  const int xs = P.lin ? P.xsteps : use_tma ? tma_config_xsteps(P.tma_cfg) : 1;
   if (xs == 4 && !b1.g[0].p[2]) return WRI_EINVAL;
   b1.xsteps = b2.xsteps = xs;
+  // chunk kernels: the iterate-update pass follows every xs-th iteration of a body and its last one, so a
+  // body holds a multiple of xs iterations or all of them
+  if (P.lin) K = K >= max_iter ? max_iter : (K + xs - 1) / xs * xs;
   const bool dev_loop = !P.host_loop && device_loop_supported();
   // loop bodies after which the device loop gives up: every system stops by max_iter + 1 iterations
   const int cap_bodies = (max_iter + 2 + K - 1) / K + 2;
   // graph lookup / capture
-  std::vector<unsigned char> key(sizeof(Batch) * 2 + 7 * sizeof(int) + (use_tma ? sizeof(TmaSet) : 0));
+  std::vector<unsigned char> key(sizeof(Batch) * 2 + 7 * sizeof(int) + (use_tma ? sizeof(TmaSet) : sizeof(LinWait)));
   std::memcpy(key.data(), &b1, sizeof(Batch));
   std::memcpy(key.data() + sizeof(Batch), &b2, sizeof(Batch));
-  const int extra[7] = {mode2, K, P.by, rb, use_tma ? P.tma_cfg : -1, dev_loop ? 1 : 0, cap_bodies};
+  const int extra[7] = {mode2, K, P.by, rb, P.lin ? -2 : use_tma ? P.tma_cfg : -1, dev_loop ? 1 : 0, cap_bodies};
   std::memcpy(key.data() + 2 * sizeof(Batch), extra, sizeof(extra));
   if (use_tma) std::memcpy(key.data() + 2 * sizeof(Batch) + sizeof(extra), tma, sizeof(TmaSet));
+  else std::memcpy(key.data() + 2 * sizeof(Batch) + sizeof(extra), lin, sizeof(LinWait));
   std::shared_ptr<CUgraphExec_st> exec;
   {
     std::lock_guard<std::mutex> lk(g_mu);
@@ -690,7 +851,7 @@ int run_loop(const Plan& P, const Batch& b1_in, const Batch& b2_in, int mode2, i
           cudaGraph_t body = np.conditional.phGraph_out[0];
           err = cudaStreamBeginCaptureToGraph(c->cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
           if (err == cudaSuccess) {
-            err = capture_iterations(P, b1, b2, mode2, K, rb, use_tma, tma, c->cap);
+            err = capture_iterations(P, b1, b2, mode2, K, rb, use_tma, tma, lin, c->cap);
             if (err == cudaSuccess) err = launch_loop_ctl(h, b1.remaining, cap_bodies, c->cap);
             const cudaError_t e2 = cudaStreamEndCapture(c->cap, &body);
             if (err == cudaSuccess) err = e2;
@@ -698,7 +859,7 @@ int run_loop(const Plan& P, const Batch& b1_in, const Batch& b2_in, int mode2, i
         }
       } else {
         WRI_CK(cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeRelaxed));
-        err = capture_iterations(P, b1, b2, mode2, K, rb, use_tma, tma, c->cap);
+        err = capture_iterations(P, b1, b2, mode2, K, rb, use_tma, tma, lin, c->cap);
         const cudaError_t e2 = cudaStreamEndCapture(c->cap, &graph);
         if (err == cudaSuccess) err = e2;
       }
@@ -742,12 +903,42 @@ int upload(const wri_group* groups, int ngroups, const Plan& P, char* ws, cudaSt
   build_sys(groups, ngroups, P, sys, rec);
   WRI_CK(cudaMemcpyAsync(ws + P.off_sys, sys.data(), sizeof(SysDev) * sys.size(), cudaMemcpyHostToDevice, st));
   WRI_CK(cudaMemcpyAsync(ws + P.off_rec, rec.data(), sizeof(int) * rec.size(), cudaMemcpyHostToDevice, st));
+  if (P.lin) {  // one copy: the tables of all groups are neighbours
+    std::vector<char> tabs(P.aux_total - P.off_ltab32[0]);
+    std::vector<double> t;
+    for (int gi = 0; gi < ngroups; ++gi) {
+      layer_table(groups[gi].grid, t);
+      char* p32 = tabs.data() + (P.off_ltab32[gi] - P.off_ltab32[0]);
+      for (size_t i = 0; i < t.size(); ++i) ((float*)p32)[i] = (float)t[i];
+      std::memcpy(tabs.data() + (P.off_ltab64[gi] - P.off_ltab32[0]), t.data(), sizeof(double) * t.size());
+    }
+    WRI_CK(cudaMemcpyAsync(ws + P.off_ltab32[0], tabs.data(), tabs.size(), cudaMemcpyHostToDevice, st));
+  }
   return WRI_OK;
 }
 
 int check_ws(const Plan& P, const void* ws, size_t bytes) {
   if (!ws || ((uintptr_t)ws % kAlign) != 0 || bytes < P.total) return WRI_EWORKSPACE;
   return WRI_OK;
+}
+
+// Work order of the phases (wri_solve_opts.order) as Batch::order and Batch::sblock.
+int order_of(const wri_solve_opts* o) {
+  const int ord = o->order ? o->order : kDefaultOrder;
+  return (ord == 1) ? 1 : (ord == 3) ? 2 : (ord >= 4) ? 3 : 0;
+}
+int sblock_of(const wri_solve_opts* o) {
+  const int ord = o->order ? o->order : kDefaultOrder;
+  return (ord >= 4) ? (1 << (ord - 2)) : 1;  // 4 -> 4 systems, 5 -> 8, 6 -> 16
+}
+
+LinWait lin_wait(const Batch& b, const wri_solve_opts* o) {
+  LinWait w;
+  std::memset(&w, 0, sizeof(w));
+  w.err = b.remaining + 1;
+  w.wait_ns = o->wait_limit_us > 0 ? 1000ull * (unsigned long long)o->wait_limit_us : kWaitLimitNs;
+  w.withhold = o->test_withhold > 0 ? o->test_withhold - 1 : -1;
+  return w;
 }
 
 // ---------------------------------------------------------------- fused, batched solve
@@ -757,36 +948,36 @@ int solve_fused(const wri_group* groups, int ngroups, const wri_solve_opts* o, c
   b.max_iter = o->max_iter;
   b.tol = o->tol;
   const int vb = P.vbytes / 2;
+  const LinWait w = lin_wait(b, o);
+  b.order = order_of(o);
+  b.sblock = sblock_of(o);
   if (setup_rmask(P, b, ws, st) != WRI_OK) return WRI_ECUDA;
-  WRI_CK(launch_ztable(b, st));
+  if (!P.lin) WRI_CK(launch_ztable(b, st));
   WRI_CK(launch_setup_rhs(o->dtype == WRI_C128 ? 8 : 4, vb, b, P.nsys_total, st));
   WRI_CK(cudaMemsetAsync(b.remaining, 0, 3 * sizeof(int), st));
-  if (o->warm_start) {
-    Batch r = b;
-    r.flavor = SH_REF;
-    WRI_CK(march(vb, vb, M_SH, true, P.by, r, st));
-    r.flavor = 0;
-    WRI_CK(march(vb, vb, M_RES, false, P.by, r, st));
-    r.flavor = SH_WARM;
-    WRI_CK(march(vb, vb, M_SH, true, P.by, r, st));
+  Batch r = b;
+  r.flavor = o->warm_start ? SH_REF : SH_INIT;
+  if (P.lin) {
+    if (lin_rhs(P, r, vb, vb, w, st) != WRI_OK) return WRI_ECUDA;
   } else {
-    Batch r = b;
-    r.flavor = SH_INIT;
-    WRI_CK(march(vb, vb, M_SH, true, P.by, r, st));
+    WRI_CK(stencil_pass(P, vb, vb, M_SH, r, w, st));
+  }
+  if (o->warm_start) {
+    r.flavor = 0;
+    WRI_CK(stencil_pass(P, vb, vb, M_RES, r, w, st));
+    r.flavor = SH_WARM;
+    WRI_CK(stencil_pass(P, vb, vb, M_SH, r, w, st));
   }
   Batch b1 = b, b2 = b;
   b1.flavor = b2.flavor = 0;
-  const int ord = o->order ? o->order : kDefaultOrder;
-  b1.order = b2.order = (ord == 1) ? 1 : (ord == 3) ? 2 : (ord >= 4) ? 3 : 0;
-  b1.sblock = b2.sblock = (ord >= 4) ? (1 << (ord - 2)) : 1;  // 4 -> 4 systems, 5 -> 8, 6 -> 16
   const int K = o->poll_every > 0 ? o->poll_every : poll_default(P);
   if (P.tma_cfg >= 0) {
     static thread_local TmaSet T;  // ~8 KB: kept off the stack
     if (build_tma(b, P, b.remaining + 1, o->l2_promotion ? o->l2_promotion : kDefaultPromotion, o, T))
-      return run_loop(P, b1, b2, M_P2, std::min(K, o->max_iter + 1), o->max_iter, st, &T);
+      return run_loop(P, b1, b2, M_P2, std::min(K, o->max_iter + 1), o->max_iter, st, &T, &w);
     // descriptors rejected (e.g. an unaligned model array): same decomposition, z-march kernels
   }
-  return run_loop(P, b1, b2, M_P2, std::min(K, o->max_iter + 1), o->max_iter, st);
+  return run_loop(P, b1, b2, M_P2, std::min(K, o->max_iter + 1), o->max_iter, st, nullptr, &w);
 }
 
 // ---------------------------------------------------------------- FP64 iterative refinement
@@ -802,6 +993,9 @@ int solve_refined(const wri_group* groups, int ngroups, const wri_solve_opts* o,
   if (!slot) return WRI_ECUDA;
   // FP64 views: the residual kernel reads x64 and writes q64 (nodes) and b.r2 = q2 (receivers)
   Batch outer = solver_batch(groups, P, ws, false);
+  outer.order = order_of(o);
+  outer.sblock = sblock_of(o);
+  const LinWait w = lin_wait(outer, o);
   for (int gi = 0; gi < P.ngroups; ++gi) {
     outer.g[gi].x = outer.g[gi].x64;
     outer.g[gi].r1[0] = outer.g[gi].q64;
@@ -819,7 +1013,7 @@ int solve_refined(const wri_group* groups, int ngroups, const wri_solve_opts* o,
   Batch inner = solver_batch(groups, P, ws, true);
   inner.max_iter = o->max_iter;
   if (setup_rmask(P, inner, ws, st) != WRI_OK) return WRI_ECUDA;
-  WRI_CK(launch_ztable(inner, st));  // the outer view shares the tables
+  if (!P.lin) WRI_CK(launch_ztable(inner, st));  // the outer view shares the tables
   void* u[WRI_MAXG] = {};
   for (int gi = 0; gi < P.ngroups; ++gi) u[gi] = groups[gi].u;
   // lambda d in FP64 (lamd and q2), x64 = warm ? u : 0, r64 = 0, dx = 0
@@ -828,7 +1022,11 @@ int solve_refined(const wri_group* groups, int ngroups, const wri_solve_opts* o,
   if (o->warm_start) {  // ||S^H b|| with the FP64 stencil (q2 still holds lambda d)
     Batch r = outer;
     r.flavor = SH_REF;
-    WRI_CK(launch_march_f64_to_f32(M_SH, P.by, r, 0, st));
+    if (P.lin) {
+      if (lin_rhs(P, r, 8, 4, w, st) != WRI_OK) return WRI_ECUDA;
+    } else {
+      WRI_CK(stencil_pass(P, 8, 4, M_SH, r, w, st));
+    }
   }
   // g' = S^H r64 (FP64 stencil on r64 and r2_64, rounded into the inner gvec)
   Batch gb = outer;
@@ -842,10 +1040,9 @@ int solve_refined(const wri_group* groups, int ngroups, const wri_solve_opts* o,
   // inner solves on the warp-specialised TMA phases when the batch allows them
   const TmaSet* tma = nullptr;
   static thread_local TmaSet T;
+  inner.order = order_of(o);
+  inner.sblock = sblock_of(o);
   if (P.tma_cfg >= 0) {
-    const int ord = o->order ? o->order : kDefaultOrder;
-    inner.order = (ord == 1) ? 1 : (ord == 3) ? 2 : (ord >= 4) ? 3 : 0;
-    inner.sblock = (ord >= 4) ? (1 << (ord - 2)) : 1;
     if (build_tma(inner, P, inner.remaining + 1, o->l2_promotion ? o->l2_promotion : kDefaultPromotion, o, T))
       tma = &T;
   }
@@ -859,13 +1056,17 @@ int solve_refined(const wri_group* groups, int ngroups, const wri_solve_opts* o,
     Batch r = inner;
     r.flavor = SH_INIT;
     r.tol = std::max(o->inner_tol, 0.95 * o->refine_tol);
-    WRI_CK(march(4, 4, M_SH, true, P.by, r, st));                  // s = S^H b, r1 = b1, dx = 0
+    if (P.lin) {                                                   // s = S^H b, r1 = b1, dx = 0
+      if (lin_rhs(P, r, 4, 4, w, st) != WRI_OK) return WRI_ECUDA;
+    } else {
+      WRI_CK(stencil_pass(P, 4, 4, M_SH, r, w, st));
+    }
     WRI_CK(cudaMemcpyAsync(slot, inner.remaining, sizeof(int), cudaMemcpyDeviceToHost, st));
     WRI_CK(cudaStreamSynchronize(st));
     if (*slot > 0) {
       Batch in = inner;
       for (int gi = 0; gi < P.ngroups; ++gi) in.g[gi].gvec = nullptr;  // r64 = 0: no g'
-      const int rc = run_loop(P, in, in, M_P2, std::min(K, o->max_iter + 1), o->max_iter, st, tma);
+      const int rc = run_loop(P, in, in, M_P2, std::min(K, o->max_iter + 1), o->max_iter, st, tma, &w);
       if (rc != WRI_OK) return rc;
       WRI_CK(launch_ir_update(inner, st));                         // x64 = dx, r64 = dr
     }
@@ -876,11 +1077,12 @@ int solve_refined(const wri_group* groups, int ngroups, const wri_solve_opts* o,
     Batch r = outer;
     r.outer = outer_k;
     r.flavor = SH_REFINE;
-    WRI_CK(march(8, 8, M_RES, false, P.by, r, st));                // q = b - S x64
+    WRI_CK(stencil_pass(P, 8, 8, M_RES, r, w, st));                // q = b - S x64
     WRI_CK(launch_ir_forcing(inner, outer.r2, st));                // f = q - r64 (complex64)
-    WRI_CK(launch_march_f64_to_f32(M_SH, P.by, r, 0, st));         // c = S^H q, outer test
-    WRI_CK(cudaMemcpyAsync(slot, outer.remaining, sizeof(int), cudaMemcpyDeviceToHost, st));
+    WRI_CK(stencil_pass(P, 8, 4, M_SH, r, w, st));                 // c = S^H q, outer test
+    WRI_CK(cudaMemcpyAsync(slot, outer.remaining, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
     WRI_CK(cudaStreamSynchronize(st));
+    if (slot[1] != 0) return WRI_ECUDA;                            // a bounded copy wait timed out
     if (*slot <= 0) break;
     Batch in = inner;
     if (outer_k == 0) {
@@ -888,9 +1090,9 @@ int solve_refined(const wri_group* groups, int ngroups, const wri_solve_opts* o,
       // phase 2 reads no g'
       for (int gi = 0; gi < P.ngroups; ++gi) in.g[gi].gvec = nullptr;
     } else {
-      WRI_CK(launch_march_f64_to_f32(M_SH, P.by, gb, 0, st));      // g' = S^H r64
+      WRI_CK(stencil_pass(P, 8, 4, M_SH, gb, w, st));              // g' = S^H r64
     }
-    const int rc = run_loop(P, in, in, M_P2, std::min(K, o->max_iter + 1), o->max_iter, st, tma);
+    const int rc = run_loop(P, in, in, M_P2, std::min(K, o->max_iter + 1), o->max_iter, st, tma, &w);
     if (rc != WRI_OK) return rc;
     WRI_CK(launch_ir_update(inner, st));                           // x64 += dx, r64 += dr
     if (outer_k > o->max_refine + 1) return WRI_ECUDA;
@@ -1058,6 +1260,23 @@ int apply_common(const wri_grid* grid, int dtype, const void* m, int nsys, const
   G.s = y;
   b.nitems = G.nitems;
   const int rb = dtype == WRI_C128 ? 8 : 4;
+  // The chunk kernel, where the layer table fits its arguments and the arrays have their natural alignment
+  // (complex128, A^H on 81^3 x 9: 336 us against the z-march kernel's 1387; a single complex64 36^3 is bound
+  // by the call).
+  if (grid->npml < kLinInlineTab && (long long)grid->nx * grid->ny < (1LL << 28) && (uintptr_t)m % rb == 0 &&
+      ((uintptr_t)x | (uintptr_t)y) % vb == 0 && lin_smem(b, rb, M_APPLY) <= (size_t)kLinMaxSmem) {
+    b.pair = rb == 4 && grid->nx % 2 == 0 && ((uintptr_t)x | (uintptr_t)y) % 16 == 0 && (uintptr_t)m % 8 == 0;
+    b.order = 3;
+    b.sblock = 16;
+    decompose_lin(*grid, auto_zsplit_lin((long long)nsys * lin_chunks(*grid), grid->nz, rb == 8), G);
+    G.nitems = (long long)G.ntiles * nsys;
+    b.nitems = G.nitems;
+    std::vector<double> tab;
+    layer_table(*grid, tab);
+    const LinWait w = {nullptr, kWaitLimitNs, -1};
+    WRI_CK(launch_lin(rb, rb, M_APPLY, conj, b, w, tab.data(), grid->npml + 1, st));
+    return WRI_OK;
+  }
   WRI_CK(march(rb, rb, M_APPLY, conj, 8, b, st));
   return WRI_OK;
 }
@@ -1121,11 +1340,75 @@ Batch aux_batch(const wri_group* groups, int ngroups, const Plan& P, char* ws, i
   return b;
 }
 
+// Whether the gradient can run on the chunk kernel: FP64 stencils (where the FP64 pipe binds and the chunk
+// kernel takes half the instructions; the complex64 gradient stays on the z-march kernel), planes that fit,
+// natural alignment of the arrays.
+bool grad_lin_ok(const wri_group* groups, int ngroups, int dtype, bool wide) {
+  const size_t rb = dtype == WRI_C128 ? 8 : 4;
+  if (rb == 4 && !wide) return false;
+  Batch probe;
+  probe.ngroups = ngroups;
+  for (int gi = 0; gi < ngroups; ++gi) {
+    const wri_grid& g = groups[gi].grid;
+    const uintptr_t u = (uintptr_t)(wide ? groups[gi].u64 : groups[gi].u);
+    if ((long long)g.nx * g.ny >= (1LL << 28) || u % 16 || (uintptr_t)groups[gi].m % rb) return false;
+    probe.g[gi].nx = g.nx;
+    probe.g[gi].ny = g.ny;
+    probe.g[gi].zc = kGradPlanes;
+    probe.g[gi].m_double = dtype == WRI_C128 ? 1 : 0;
+  }
+  return lin_smem(probe, 8, M_GRAD) <= (size_t)kLinMaxSmem;
+}
+
+// The gradient pass and the data term of aux_batch's view.  The chunk kernel streams a z-chunk of one system
+// after the other and keeps the sums in shared memory; its z-chunks (at most kGradPlanes planes) are as long
+// as the waves of resident CTAs (2 per SM) allow.
+int gradient_pass(const wri_group* groups, const Plan& P, Batch& b, const char* ws, int rb, int db, cudaStream_t st) {
+  if (!P.lin) {
+    WRI_CK(launch_ztable(b, st));
+    WRI_CK(march(rb, rb, M_GRAD, false, 8, b, st));
+  } else {
+    long long chunks = 0;
+    int nz = 0;
+    for (int gi = 0; gi < b.ngroups; ++gi) {
+      chunks += lin_chunks(groups[gi].grid);
+      nz = std::max(nz, b.g[gi].nz);
+    }
+    const long long wave = (long long)kRefSMs * 2;
+    int zc = kGradPlanes;
+    double best = 0.0;
+    for (int c = kGradPlanes; c >= 1; --c) {
+      const long long items = chunks * ((nz + c - 1) / c);
+      const double cost = (double)((items + wave - 1) / wave) * (c + 0.3);
+      if (c == kGradPlanes || cost < best) {
+        best = cost;
+        zc = c;
+      }
+    }
+    long long item = 0;
+    for (int gi = 0; gi < b.ngroups; ++gi) {
+      GroupDev& G = b.g[gi];
+      decompose_lin(groups[gi].grid, (G.nz + zc - 1) / zc, G);
+      G.item0 = item;
+      G.nitems = G.ntiles;
+      item += G.nitems;
+      G.ltab64 = (const double*)(ws + P.off_ltab64[gi]);
+    }
+    b.nitems = item;
+    const LinWait w = {nullptr, kWaitLimitNs, -1};
+    WRI_CK(launch_lin(rb, rb, M_GRAD, false, b, w, nullptr, 0, st));
+  }
+  WRI_CK(launch_data_term(rb, db, b, P.nsys_total, st));
+  return WRI_OK;
+}
+
 // ---------------------------------------------------------------- allocation-free gradient
 // Scratch of wri_gradient_noalloc: the device copy of the geometry (per-system
 // descriptors and receiver list).  Host code must not hand the symbol itself to a
 // kernel; it looks up the device address once per device (noalloc_scratch).
-static __device__ __align__(256) unsigned char g_noalloc_scratch[WRI_NOALLOC_SCRATCH_BYTES];
+// The extra room is for the layer tables, which the limit of the entry point does not count.
+constexpr size_t kNoallocTables = 256u << 10;
+static __device__ __align__(256) unsigned char g_noalloc_scratch[WRI_NOALLOC_SCRATCH_BYTES + kNoallocTables];
 std::mutex g_noalloc_mu;
 void* g_noalloc_ptr[64];
 
@@ -1159,7 +1442,9 @@ int wri_gradient_noalloc(const wri_group* groups, int ngroups, int dtype, const 
   if (rc != WRI_OK) return rc;
   Plan P;
   plan_aux(groups, ngroups, P);
-  if (P.aux_total > (size_t)WRI_NOALLOC_SCRATCH_BYTES) return WRI_ESCRATCH;
+  if (P.aux_base > (size_t)WRI_NOALLOC_SCRATCH_BYTES) return WRI_ESCRATCH;
+  P.lin = grad_lin_ok(groups, ngroups, dtype, wide) &&
+          P.aux_total <= (size_t)WRI_NOALLOC_SCRATCH_BYTES + kNoallocTables;
   char* ws = nullptr;
   rc = noalloc_scratch(&ws);
   if (rc != WRI_OK) return rc;
@@ -1173,10 +1458,7 @@ int wri_gradient_noalloc(const wri_group* groups, int ngroups, int dtype, const 
     b.g[gi].grad = grad[gi];
   }
   const int rb = (dtype == WRI_C128 || wide) ? 8 : 4;
-  WRI_CK(launch_ztable(b, st));
-  WRI_CK(march(rb, rb, M_GRAD, false, 8, b, st));
-  WRI_CK(launch_data_term(rb, dtype == WRI_C128 ? 8 : 4, b, P.nsys_total, st));
-  return WRI_OK;
+  return gradient_pass(groups, P, b, ws, rb, dtype == WRI_C128 ? 8 : 4, st);
 }
 
 
@@ -1285,6 +1567,7 @@ int wri_gradient(const wri_group* groups, int ngroups, int dtype, const double* 
   if (rc != WRI_OK) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   char* ws = (char*)workspace;
+  P.lin = grad_lin_ok(groups, ngroups, dtype, wide);
   rc = upload(groups, ngroups, P, ws, st);
   if (rc != WRI_OK) return rc;
   Batch b = aux_batch(groups, ngroups, P, ws, dtype, wide);
@@ -1294,10 +1577,7 @@ int wri_gradient(const wri_group* groups, int ngroups, int dtype, const double* 
     b.g[gi].grad = grad[gi];
   }
   const int rb = (dtype == WRI_C128 || wide) ? 8 : 4;
-  WRI_CK(launch_ztable(b, st));
-  WRI_CK(march(rb, rb, M_GRAD, false, 8, b, st));
-  WRI_CK(launch_data_term(rb, dtype == WRI_C128 ? 8 : 4, b, P.nsys_total, st));
-  return WRI_OK;
+  return gradient_pass(groups, P, b, ws, rb, dtype == WRI_C128 ? 8 : 4, st);
 }
 
 int wri_gradient_refined(const wri_group* groups, int ngroups, const wri_solve_opts* opts, double* const* grad,
@@ -1424,7 +1704,7 @@ int wri_autotune(const wri_group* groups, int ngroups, wri_solve_opts* opts, int
       o.test_withhold = 0;
       Plan P;
       plan_solve(groups, ngroups, &o, P);
-      if (P.tma_cfg != cfg || check_ws(P, workspace, ws_bytes) != WRI_OK) continue;
+      if ((P.lin ? !lin_config(cfg) : P.tma_cfg != cfg) || check_ws(P, workspace, ws_bytes) != WRI_OK) continue;
       char* ws = (char*)workspace;
       float ms = 0.f;
       for (int rep = 0; rep < 2 && rc == WRI_OK; ++rep) {  // the first run captures the graph

@@ -11,6 +11,12 @@
 
 namespace wri {
 
+// Layer table of the chunk kernels: entry d (0 .. npml) of a node d cells inside the layer holds, in
+// R[kLayerTab]: alpha of the half point nearer the interior (0, 1) and farther from it (2, 3), minus their
+// sum (4, 5), Im s (6), a pad (7), and 1 / (s(half) h^2) of the nearer (8, 9) and farther (10, 11) half point.
+constexpr int kLayerTab = 12;
+constexpr int kXupdNodes = 4096;  // nodes of a work item of the iterate-update pass
+
 // z-chunk of the gradient kernel (its FP64 accumulator tile lives in shared memory)
 __host__ __device__ constexpr int grad_zc(int by) { return by >= 16 ? 8 : 16; }
 
@@ -131,10 +137,14 @@ struct SysDev {
 struct GroupDev {
   int nx, ny, nz, npml;
   double h, omega, lambda;
+  double ih2, om2;            // 1/h^2, omega^2
   float ih2f, om2f, lambdaf;  // 1/h^2, omega^2, lambda in FP32
   AxisPml ax, ay, az;
   int nsys, sys0;          // systems of the group and global index of the first
   int tiles_x, tiles_y, zsplit, zc, ntiles;
+  int chunk;               // chunk kernels: nodes of a chunk of the x-y plane (tiles_x chunks, tiles_y = 1)
+  int rw;                  // words of a row of the receiver bitmaps
+  long long xitem0;        // chunk kernels: first work item of the group in the iterate-update pass
   long long item0, nitems;  // work items (tile x system) of the group in the batched launch
   int masked;               // 1 = source-free (Z applied), 0 = known weight or general right-hand side
   long long n;              // nodes
@@ -156,19 +166,22 @@ struct GroupDev {
   const void* gvec;         // [nsys][n] complex64 S^H r64, added to s in phase 2 (or null)
   const int* rmap;          // [nsys][n] receiver entry of a node (-1: none): the FP64 S^H kernels of
                             // the refinement add lambda P^T r2 in the stencil pass (or null)
-  const uint32_t* rmask;    // [nsys][nz][ny][tiles_x] receiver bits of the normal-residual norms
+  const uint32_t* rmask;    // [nsys][nz][ny][rw] receiver bits of the normal-residual norms
                             // (bit b of word (k, j, t): node (32 t + b, j, k) is a receiver), or null
-  const uint32_t* rcol;     // [nsys][ny][tiles_x] OR of rmask over k (columns holding a receiver)
+  const uint32_t* rcol;     // [nsys][ny][rw] OR of rmask over k (columns holding a receiver)
   double* grad;             // [n] gradient accumulator (gradient kernel only)
   const float2* ztab;       // [2][nz][3] z-axis coefficients (s_z, 1/(s_z(k-1/2) h^2), 1/(s_z(k+1/2) h^2)),
                             // [0] for A, [1] conjugated for A^H; FP32, built once per call (or null)
   const double2* ztab64;    // the same table in FP64 (the z-march FP64 kernels), or null
+  const float* ltab32;      // layer table of the chunk kernels (kLayerTab), FP32 and FP64
+  const double* ltab64;
 };
 
 struct Batch {
   int ngroups;
   int bx, by;           // thread block shape (bx = WRI_TX)
   long long nitems;     // total work items
+  long long xitems;     // work items of the iterate-update pass (chunk kernels)
   SysDev* sys;
   double* partial;      // per (system, tile) FP64 partial sums
   const int* rec_idx;   // batch-wide receiver nodes
@@ -184,6 +197,7 @@ struct Batch {
                         // consecutive, 2 = z-chunk slowest (the resident wave shares z-slabs),
                         // 3 = blocks of sblock systems, tiles in order, systems fastest in a block
   int sblock;           // systems per block of order 3
+  int pair;             // chunk kernels, complex64: a thread's two nodes are adjacent (nx even, arrays aligned)
   int xsteps;           // m: phase 1 adds the steps of m iterations to x every m-th iteration (m = 2, 4:
                         // the warp-specialised grouped-update configurations; 0 or 1: every iteration)
   double tol;           // tolerance of a cold-start solve

@@ -63,4 +63,22 @@ int tma_config_count();
 int tma_config_by(int cfg);
 int tma_config_xsteps(int cfg);  // iterations per iterate update of phase 1 (1, 2 or 4)
 cudaError_t launch_phase_tma(int mode, int cfg, const Batch& b, const TmaSet& T, int grid, cudaStream_t st);
+
+// Chunk kernels (wri_lin.cu): stencil passes over linear chunks of the x-y plane.
+constexpr int kLinStages = 3;
+constexpr int kLinMaxSmem = 220 * 1024;
+struct LinWait {  // bounded waits of the copy pipelines (TmaSet)
+  int* err;
+  unsigned long long wait_ns;
+  int withhold;
+};
+size_t lin_smem(const Batch& b, int rbytes, int mode);  // shared memory of a CTA
+// mode M_APPLY, M_SH, M_RES, M_P1, M_P2 or M_GRAD; tab (tab_n entries): the layer table of M_APPLY
+cudaError_t launch_lin(int rbytes, int obytes, int mode, bool conj, const Batch& b, const LinWait& w,
+                       const double* tab, int tab_n, cudaStream_t st);
+// s = S^H b of point right-hand sides (flavors SH_INIT, SH_REF) without a pass over the grid
+cudaError_t launch_init_point(int rbytes, int obytes, const Batch& b, int nsys_total, cudaStream_t st);
+cudaError_t launch_point_field(int rbytes, const Batch& b, int gi, cudaStream_t st);  // r1[src] = alpha
+// x += the steps of the last b.xsteps iterations; closes systems that have stopped
+cudaError_t launch_xupdate(int rbytes, const Batch& b, cudaStream_t st);
 }  // namespace wri

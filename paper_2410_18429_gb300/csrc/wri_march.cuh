@@ -136,11 +136,11 @@ __device__ __forceinline__ ZCoef<R> z_lookup(const GroupDev& G, int k) {
 // Bits of the thread's 32-node row segment (x0 .. x0+31, row j) that hold a receiver at any z ...
 __device__ __forceinline__ uint32_t rec_col_bits(const GroupDev& G, int sl, int j, int x0) {
   if (!G.rmask) return 0u;
-  return __ldg(G.rcol + ((long long)sl * G.ny + j) * G.tiles_x + (x0 >> 5));
+  return __ldg(G.rcol + ((long long)sl * G.ny + j) * G.rw + (x0 >> 5));
 }
 // ... and at plane k
 __device__ __forceinline__ uint32_t rec_plane_bits(const GroupDev& G, int sl, int k, int j, int x0) {
-  return __ldg(G.rmask + (((long long)sl * G.nz + k) * G.ny + j) * G.tiles_x + (x0 >> 5));
+  return __ldg(G.rmask + (((long long)sl * G.nz + k) * G.ny + j) * G.rw + (x0 >> 5));
 }
 
 // First/last node index of an axis whose own stretch and both half-point stretches are 1.

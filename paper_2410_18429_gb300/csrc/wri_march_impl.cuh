@@ -15,6 +15,74 @@ __device__ __forceinline__ cx<R> ldg_c(const cx<R>* p) {
 }
 
 // ------------------------------------------------------------------ finalizers
+// Scalars of a system after s = S^H r, with g = ||s||^2 (one thread).
+__device__ inline void sh_scalars(const Batch& b, SysDev* sd, double g) {
+  const double rn = sqrt(g);
+  if (b.flavor == SH_PLAIN) {
+    // S^H r64 of the refinement: output vector only, no scalar changes
+  } else if (b.flavor == SH_REF) {
+    sd->snorm_b = rn;
+  } else if (b.flavor == SH_INIT || b.flavor == SH_WARM) {
+    if (b.flavor == SH_INIT) sd->snorm_b = rn;
+    sd->snorm_ref = sd->snorm_b;
+    sd->gamma = g;
+    sd->beta = 0.0;
+    sd->alpha = 0.0;
+    sd->alpha_hist[0] = sd->alpha_hist[1] = sd->alpha_hist[2] = 0.0;
+    sd->iter = 0;
+    sd->iter_total = 0;
+    sd->tol = b.tol;
+    sd->relres = sd->snorm_b > 0.0 ? rn / sd->snorm_b : 0.0;
+    if (!isfinite(g)) {
+      sd->status = WRI_SYS_NONFINITE;
+      sd->state = ST_DONE;
+    } else if (g == 0.0 || rn <= b.tol * sd->snorm_b) {
+      sd->status = WRI_SYS_OK;
+      sd->state = ST_DONE;
+    } else {
+      sd->status = WRI_SYS_OK;
+      sd->state = ST_ACTIVE;
+      atomicAdd(b.remaining, 1);
+    }
+  } else {  // SH_REFINE: outer step of the FP64 refinement
+    if (b.outer == 0 && !b.warm) {
+      sd->snorm_b = rn;
+      sd->iter_total = 0;
+    }
+    const double rr = sd->snorm_b > 0.0 ? rn / sd->snorm_b : 0.0;
+    sd->relres = rr;
+    const bool bad = !isfinite(g) || sd->status == WRI_SYS_NONFINITE;
+    if (bad) {
+      sd->status = WRI_SYS_NONFINITE;
+      sd->outer_done = 1;
+      sd->state = ST_DONE;
+    } else if (g == 0.0 || rr <= b.refine_tol) {
+      sd->status = WRI_SYS_OK;
+      sd->outer_done = 1;
+      sd->state = ST_DONE;
+    } else if (b.outer >= b.max_refine) {
+      sd->status = WRI_SYS_MAXITER;
+      sd->outer_done = 1;
+      sd->state = ST_DONE;
+    } else {
+      sd->status = WRI_SYS_OK;
+      sd->gamma = g;
+      sd->snorm_ref = rn;
+      // the correction needs no more accuracy than the outer target asks for, with 5 % of
+      // margin for the drift between the FP32 recurrence and the FP64 residual (measured about
+      // 0.5 % at 1e-2): a tighter inner tolerance would only add iterations, and CGLS's normal
+      // residual can stall for thousands of iterations just below a target
+      sd->tol = fmax(b.inner_tol, 0.95 * b.refine_tol * sd->snorm_b / rn);
+      sd->beta = 0.0;
+      sd->alpha = 0.0;
+      sd->alpha_hist[0] = sd->alpha_hist[1] = sd->alpha_hist[2] = 0.0;
+      sd->iter = 0;
+      sd->state = ST_ACTIVE;
+      atomicAdd(b.remaining, 1);
+    }
+  }
+}
+
 // Run by every thread of the CTA that completed the last tile of system `sd`.
 // NT is the number of threads that run it (the whole CTA, any 2-D shape, or the first NT
 // threads of a 1-D CTA with SYNC = FirstThreadsSync<NT>).
@@ -119,71 +187,7 @@ __device__ void finalize(const Batch& b, const GroupDev& G, SysDev* sd, int sl, 
       }
       sd->gamma = g;
     } else if (MODE == M_SH) {
-      const double g = tot;
-      const double rn = sqrt(g);
-      if (b.flavor == SH_PLAIN) {
-        // S^H r64 of the refinement: output vector only, no scalar changes
-      } else if (b.flavor == SH_REF) {
-        sd->snorm_b = rn;
-      } else if (b.flavor == SH_INIT || b.flavor == SH_WARM) {
-        if (b.flavor == SH_INIT) sd->snorm_b = rn;
-        sd->snorm_ref = sd->snorm_b;
-        sd->gamma = g;
-        sd->beta = 0.0;
-        sd->alpha = 0.0;
-        sd->alpha_hist[0] = sd->alpha_hist[1] = sd->alpha_hist[2] = 0.0;
-        sd->iter = 0;
-        sd->iter_total = 0;
-        sd->tol = b.tol;
-        sd->relres = sd->snorm_b > 0.0 ? rn / sd->snorm_b : 0.0;
-        if (!isfinite(g)) {
-          sd->status = WRI_SYS_NONFINITE;
-          sd->state = ST_DONE;
-        } else if (g == 0.0 || rn <= b.tol * sd->snorm_b) {
-          sd->status = WRI_SYS_OK;
-          sd->state = ST_DONE;
-        } else {
-          sd->status = WRI_SYS_OK;
-          sd->state = ST_ACTIVE;
-          atomicAdd(b.remaining, 1);
-        }
-      } else {  // SH_REFINE: outer step of the FP64 refinement
-        if (b.outer == 0 && !b.warm) {
-          sd->snorm_b = rn;
-          sd->iter_total = 0;
-        }
-        const double rr = sd->snorm_b > 0.0 ? rn / sd->snorm_b : 0.0;
-        sd->relres = rr;
-        const bool bad = !isfinite(g) || sd->status == WRI_SYS_NONFINITE;
-        if (bad) {
-          sd->status = WRI_SYS_NONFINITE;
-          sd->outer_done = 1;
-          sd->state = ST_DONE;
-        } else if (g == 0.0 || rr <= b.refine_tol) {
-          sd->status = WRI_SYS_OK;
-          sd->outer_done = 1;
-          sd->state = ST_DONE;
-        } else if (b.outer >= b.max_refine) {
-          sd->status = WRI_SYS_MAXITER;
-          sd->outer_done = 1;
-          sd->state = ST_DONE;
-        } else {
-          sd->status = WRI_SYS_OK;
-          sd->gamma = g;
-          sd->snorm_ref = rn;
-          // the correction needs no more accuracy than the outer target asks for, with 5 % of
-          // margin for the drift between the FP32 recurrence and the FP64 residual (measured about
-          // 0.5 % at 1e-2): a tighter inner tolerance would only add iterations, and CGLS's normal
-          // residual can stall for thousands of iterations just below a target
-          sd->tol = fmax(b.inner_tol, 0.95 * b.refine_tol * sd->snorm_b / rn);
-          sd->beta = 0.0;
-          sd->alpha = 0.0;
-          sd->alpha_hist[0] = sd->alpha_hist[1] = sd->alpha_hist[2] = 0.0;
-          sd->iter = 0;
-          sd->state = ST_ACTIVE;
-          atomicAdd(b.remaining, 1);
-        }
-      }
+      sh_scalars(b, sd, tot);
     }
     sd->ticket = 0u;
   }
