@@ -122,8 +122,13 @@ cudaError_t launch_data_term(int rbytes, int dbytes, const Batch& b, int nsys_to
 
 cudaError_t launch_tv(const double* m, int nx, int ny, int nz, double beta, double gamma, double* tv, double* grad,
                       cudaStream_t st) {
-  const long long n = (long long)nx * ny * nz;
-  k_tv<<<grid_for(n, 256, 4096), 256, 0, st>>>(m, nx, ny, nz, beta, gamma, tv, grad);
+  const int bx = (nx + kTvX - 2) / (kTvX - 1), by = (ny + kTvY - 2) / (kTvY - 1);
+  // z-chunks: about eight blocks per SM, chunks of at least 8 planes (one more is evaluated below each)
+  int zs = (int)((8LL * 152 + (long long)bx * by - 1) / ((long long)bx * by));
+  zs = zs > nz / 8 ? nz / 8 : zs;
+  zs = zs < 1 ? 1 : zs;
+  const int zc = (nz + zs - 1) / zs;
+  k_tv<<<dim3(bx, by, (nz + zc - 1) / zc), dim3(kTvX, kTvY), 0, st>>>(m, nx, ny, nz, zc, beta, gamma, tv, grad);
   return cudaGetLastError();
 }
 
