@@ -239,6 +239,26 @@ __device__ __forceinline__ void item_coords(const Batch& b, const GroupDev& G, l
   }
 }
 
+// The same for the chunk kernels (order 0, 1 or 3 of a group with fewer than 2^31 items: 32-bit divisions).
+__device__ __forceinline__ void item_coords32(const Batch& b, const GroupDev& G, long long local, int& sl, int& tile) {
+  if (b.order == 2 || G.nitems >= (1LL << 31)) {
+    item_coords(b, G, local, sl, tile);
+    return;
+  }
+  const unsigned l = (unsigned)local, nt = (unsigned)G.ntiles, ns = (unsigned)G.nsys;
+  if (b.order == 1) {
+    sl = (int)(l / nt);
+    tile = (int)(l - (unsigned)sl * nt);
+    return;
+  }
+  const unsigned sb = b.order == 3 ? min((unsigned)b.sblock, ns) : ns;
+  const unsigned nb = (ns + sb - 1) / sb;
+  const unsigned blk = nb == 1 ? 0u : min(l / (sb * nt), nb - 1);
+  const unsigned rem = l - blk * sb * nt, cnt = min(sb, ns - blk * sb);
+  tile = (int)(rem / cnt);
+  sl = (int)(blk * sb + (rem - (unsigned)tile * cnt));
+}
+
 __device__ __forceinline__ int find_group(const Batch& b, long long item) {
   int g = 0;
 #pragma unroll 1

@@ -65,6 +65,7 @@ int tma_config_xsteps(int cfg);  // iterations per iterate update of phase 1 (1,
 cudaError_t launch_phase_tma(int mode, int cfg, const Batch& b, const TmaSet& T, int grid, cudaStream_t st);
 
 // Chunk kernels (wri_lin.cu): stencil passes over linear chunks of the x-y plane.
+constexpr int kLinChunk = 256;  // nodes of a chunk, at most
 constexpr int kLinStages = 3;
 constexpr int kLinMaxSmem = 220 * 1024;
 struct LinWait {  // bounded waits of the copy pipelines (TmaSet)

@@ -4,7 +4,7 @@
 
 namespace wri {
 
-// Stage layout of a batch: the two fields' regions (256 nodes and nx on either side, one more element
+// Stage layout of a batch: the two fields' regions (a chunk and nx nodes on either side, one more element
 // for the 16-byte boundary at each end) and the model's.
 static size_t lin_layout(const Batch& b, int rbytes, int mode, LinSet& T) {
   const bool two = mode == M_P1 || mode == M_P2;

@@ -29,7 +29,10 @@
 //
 // What binds: complex64 phases move 32 bytes per node and reach 5.4 TB/s in phase 1 (148^3 x 16, ncu) at 50 %
 // issue utilisation, 270 warp instructions per 64 nodes and plane (320 in the boxes, 374 before the warps
-// without stretched nodes and the z layers got loops of their own).  Stages beyond three are slower (the
+// without stretched nodes and the z layers got loops of their own).  Running addresses in the copy warp, no
+// plane or lane checks in the main loop and one set of y coefficients per pair: 148^3 x 32 46.8 -> 45.8 us
+// per system and iteration, 84^3 x 64 9.0 -> 8.7.  Chunks of 512 nodes (half the halo) are slower: 47.8
+// and 9.4, 276 x 276 x 180 x 4 181 against 173.  Stages beyond three are slower (the
 // plane streams alone: 749 against 550 us with six).  complex128 passes are bound by the FP64 pipe (86-90 %
 // busy).
 //
@@ -39,12 +42,12 @@
 
 #include <type_traits>
 
+#include "wri_launch.h"
 #include "wri_march_impl.cuh"
 #include "wri_tma.cuh"
 
 namespace wri {
 
-constexpr int kLinChunk = 256;     // nodes of a chunk, at most
 constexpr int kLinInlineTab = 33;  // entries of the table that travels with the kernel arguments (APPLY)
 
 struct LinSet {
@@ -131,9 +134,11 @@ __device__ __forceinline__ AxisCoef<R> axis_coef(const R* tab, int i, int n, int
   return c;
 }
 
+// element e of a staged model chunk (complex64 passes have a float model, FP64 passes either)
 template <typename R>
 __device__ __forceinline__ R model_smem(const unsigned char* p, int m_double, int e) {
-  return m_double ? R(reinterpret_cast<const double*>(p)[e]) : R(reinterpret_cast<const float*>(p)[e]);
+  if (sizeof(R) == 8 && m_double) return R(reinterpret_cast<const double*>(p)[e]);
+  return R(reinterpret_cast<const float*>(p)[e]);
 }
 
 // R: arithmetic; OR: type of the stencil's output vector; MODE: M_APPLY, M_SH, M_RES, M_P1, M_P2 or M_GRAD; NC
@@ -145,7 +150,8 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
   typedef cx<R> C;
   typedef cx<OR> OC;
   static_assert(!PAIR || (NPT == 2 && sizeof(R) == 4), "pairs of complex64");
-  static_assert(NC * NPT == kLinChunk, "the threads cover a chunk");
+  constexpr int L = NC * NPT;
+  static_assert(L == kLinChunk, "the threads cover a chunk");
   constexpr bool HASB = (MODE == M_P1 || MODE == M_P2);
   constexpr bool NORM = (MODE == M_P1 || MODE == M_P2 || MODE == M_SH);
   constexpr int NCW = NC / 32;
@@ -166,20 +172,18 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
   const int SB = T.stage;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)S * SB);
   uint64_t* empty = full + S;
-  double* gacc = reinterpret_cast<double*>(empty + S);  // gradient: [planes of the z-chunk][kLinChunk]
+  double* gacc = reinterpret_cast<double*>(empty + S);  // gradient: [planes of the z-chunk][L]
   const int tid = threadIdx.x;
   if (tid == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], NCW);
     }
-    // a copy wait of an earlier launch of this solve timed out: this launch does nothing
-    s_abort = (T.err && *(volatile const int*)T.err != 0) ? 1 : 0;
+    s_abort = 0;
   }
   if constexpr (MODE == M_APPLY)
     for (int e = tid; e < tab_in.n * kLayerTab; e += NC + 32) s_tab[e] = R(tab_in.v[e]);
   __syncthreads();  // the only CTA-wide barrier: the copy warp leaves the consumers' barriers after it
-  if (s_abort) return;
 
   // what the item does; the same decision in both roles
   auto skip_item = [&](const SysDev* sd) -> bool {
@@ -198,6 +202,12 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
   // ================================================================ copy warp
   if (tid >= NC) {
     if (tid != NC) return;
+    // a copy wait of an earlier launch of this solve timed out: this launch copies nothing, and its consumers
+    // find the flag in their first wait
+    if (T.err && *(volatile const int*)T.err != 0) {
+      s_abort = 1;
+      return;
+    }
     unsigned fills = 0;
     int st = 0;
     uint32_t par = 1;  // parity of the stage's previous release (first use: none)
@@ -206,7 +216,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
       const int gi = find_group(b, item);
       const GroupDev& G = b.g[gi];
       int sl = 0, tile = (int)(item - G.item0);
-      if (!GRAD) item_coords(b, G, item - G.item0, sl, tile);
+      if (!GRAD) item_coords32(b, G, item - G.item0, sl, tile);
       const SysDev* sd = (MODE == M_APPLY) ? nullptr : b.sys + (G.sys0 + sl);
       if (MODE != M_APPLY && skip_item(sd)) continue;
       const int plane = G.nx * G.ny;
@@ -219,43 +229,55 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
       const int em = G.m_double ? 8 : 4;
       // the gradient streams its z-chunk of one system after the other
       const int passes = GRAD ? G.nsys : 1;
-      // copies nodes [e0, e1) of plane k so that node c0 - nx lands `virt & 15` bytes into the region
-      auto field = [&](uint32_t dst, const char* f, int k, int e0, int e1, uint64_t* bar, bool issue) -> uint32_t {
-        const uintptr_t first = (uintptr_t)f + ((long long)k * plane + e0) * CB;
-        const uintptr_t virt = (uintptr_t)f + ((long long)k * plane + c0 - G.nx) * CB;
-        const uint32_t pre = (uint32_t)(first & 15), bytes = (pre + (uint32_t)(e1 - e0) * CB + 15) & ~15u;
+      // Running addresses of the chunk's first node (plane k), and what an inner plane adds on either side.  A
+      // copy starts at the 16-byte boundary below its first node and ends at the one above its last; node
+      // c0 - nx lands (its address & 15) bytes into the region (always 0 where rows are whole 16-byte units).
+      constexpr bool ALIGNED = PAIR || CB == 16;
+      const int k0 = max(z0 - 1, 0);
+      const long long fstep = (long long)plane * CB, mstep = (long long)plane * em;
+      const uint32_t below = (uint32_t)(c0 - lo) * CB, above = (uint32_t)(hi - c1) * CB, mid = (uint32_t)(c1 - c0) * CB;
+      const uint32_t halo = (uint32_t)G.nx * CB;  // bytes between the region's start and the chunk's
+      uint64_t* const bars = full;
+      auto copy = [&](uint32_t region, uintptr_t at, bool inner, int stage, bool issue) -> uint32_t {
+        const uint32_t back = inner ? below : 0u;
+        const uintptr_t first = at - back;
+        const uint32_t pre = ALIGNED ? 0u : (uint32_t)(first & 15);
+        const uint32_t len = mid + (inner ? below + above : 0u);
+        const uint32_t bytes = ALIGNED ? len : (pre + len + 15) & ~15u;
         if (issue)
-          bulk_load(dst + (uint32_t)(e0 - c0 + G.nx) * CB + (uint32_t)(virt & 15) - pre, (const void*)(first - pre), bytes,
-                    bar);
+          bulk_load(region + (halo - back) + (ALIGNED ? 0u : (uint32_t)((at - halo) & 15) - pre), (const void*)(first - pre),
+                    bytes, &bars[stage]);
         return bytes;
       };
-      for (int pass = 0; pass < passes && !stop; ++pass, fa += (long long)G.n * CB)
-      for (int k = max(z0 - 1, 0); k <= min(z1, G.nz - 1); ++k, ++fills) {
-        if (fills >= (unsigned)S && !mbar_wait_or_abort(&empty[st], par, &s_abort, T.wait_ns)) {
-          s_abort = 1;
-          if (T.err) atomicExch(T.err, 1);
-          stop = true;
-          break;
-        }
-        // test hook (off unless the caller asks): this fill is never issued, so its "full" barrier
-        // never completes and the consumers' bounded wait for it runs out
-        if (!(blockIdx.x == 0 && (int)fills == T.withhold)) {
-          const uint32_t base = smem_addr(smem) + (uint32_t)st * SB;
-          const bool inner = k >= z0 && k < z1;  // the planes next to the z-chunk give z neighbours only
-          const int e0 = inner ? lo : c0, e1 = inner ? hi : c1;
-          uint32_t bytes = field(base, fa, k, e0, e1, nullptr, false);
-          if (HASB) bytes += field(base, fb, k, e0, e1, nullptr, false);
-          const uintptr_t mfirst = (uintptr_t)G.m + ((long long)k * plane + c0) * em;
-          const uint32_t mpre = (uint32_t)(mfirst & 15), mbytes = (mpre + (uint32_t)(c1 - c0) * em + 15) & ~15u;
-          if (inner) bytes += mbytes;
-          mbar_expect_tx(&full[st], bytes);
-          field(base, fa, k, e0, e1, &full[st], true);
-          if (HASB) field(base + T.off_b, fb, k, e0, e1, &full[st], true);
-          if (inner) bulk_load(base + T.off_m, (const void*)(mfirst - mpre), mbytes, &full[st]);
-        }
-        if (++st == S) {
-          st = 0;
-          par ^= 1;
+      for (int pass = 0; pass < passes && !stop; ++pass) {
+        uintptr_t pa = (uintptr_t)fa + ((long long)(GRAD ? pass : 0) * G.n + (long long)k0 * plane + c0) * CB;
+        uintptr_t pb = HASB ? (uintptr_t)fb + ((long long)k0 * plane + c0) * CB : 0;
+        uintptr_t pm = (uintptr_t)G.m + ((long long)k0 * plane + c0) * em;
+        for (int k = k0; k <= min(z1, G.nz - 1); ++k, ++fills, pa += fstep, pb += fstep, pm += mstep) {
+          if (fills >= (unsigned)S && !mbar_try_wait(&empty[st], par) &&
+              !mbar_wait_or_abort(&empty[st], par, &s_abort, T.wait_ns)) {
+            s_abort = 1;
+            if (T.err) atomicExch(T.err, 1);
+            stop = true;
+            break;
+          }
+          // test hook (off unless the caller asks): this fill is never issued, so its "full" barrier
+          // never completes and the consumers' bounded wait for it runs out
+          if (!(blockIdx.x == 0 && (int)fills == T.withhold)) {
+            const uint32_t base = smem_addr(smem) + (uint32_t)st * SB;
+            const bool inner = k >= z0 && k < z1;  // the planes next to the z-chunk give z neighbours only
+            const uint32_t mpre = (uint32_t)(pm & 15), mbytes = (mpre + (uint32_t)(c1 - c0) * em + 15) & ~15u;
+            const uint32_t ba = copy(base, pa, inner, st, false);
+            const uint32_t bb = !HASB ? 0u : ALIGNED ? ba : copy(base, pb, inner, st, false);
+            mbar_expect_tx(&full[st], ba + bb + (inner ? mbytes : 0u));
+            copy(base, pa, inner, st, true);
+            if (HASB) copy(base + T.off_b, pb, inner, st, true);
+            if (inner) bulk_load(base + T.off_m, (const void*)(pm - mpre), mbytes, &full[st]);
+          }
+          if (++st == S) {
+            st = 0;
+            par ^= 1;
+          }
         }
       }
     }
@@ -277,7 +299,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
     const int gi = find_group(b, item);
     const GroupDev& G = b.g[gi];
     int sl = 0, tile = (int)(item - G.item0);
-    if (!GRAD) item_coords(b, G, item - G.item0, sl, tile);
+    if (!GRAD) item_coords32(b, G, item - G.item0, sl, tile);
     SysDev* sd = (MODE == M_APPLY) ? nullptr : b.sys + (G.sys0 + sl);
     if (MODE != M_APPLY && skip_item(sd)) continue;
 
@@ -314,6 +336,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
       }
     }
     gen = __any_sync(0xffffffffu, gen);
+    const bool idle = !__any_sync(0xffffffffu, own[0]);  // the warp lies past the chunk's end
 
     const R coef = MODE == M_P1 ? (iter > 0 ? R(sd->beta) : R(0)) : MODE == M_P2 ? -R(sd->alpha) : R(0);
     int src_k = -1, src_r = -1;  // plane of the source, and which of the thread's nodes it is
@@ -330,7 +353,8 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
     C* pF = nullptr;
     if (MODE == M_P1) pF = (C*)G.p[pslot(b, iter)] + off + (long long)z0 * plane + e0;
     if (MODE == M_P2) pF = (C*)G.r1[(iter & 1) ^ 1] + off + (long long)z0 * plane + e0;
-    OC* pO = (OC*)(MODE == M_P1 ? G.t1 : MODE == M_RES ? G.r1[0] : G.s) + off + (long long)(z0 - 1) * plane + e0;
+    // (the first step's "plane z0 - 1" is nobody's: it goes to plane z0, which the next step writes)
+    OC* pO = (OC*)(MODE == M_P1 ? G.t1 : MODE == M_RES ? G.r1[0] : G.s) + off + (long long)z0 * plane + e0;
     // bytes from the region's start to its first node (c0 - nx) and to the model's (c0): the copies start at
     // 16-byte boundaries, so these change with the plane when its bytes are not a multiple of 16
     constexpr bool SHIFT = !PAIR && CB == 8;
@@ -343,11 +367,13 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
     const int o = nx + (PAIR ? 2 * tid : tid);  // own (first) node in the region
 
     // coefficients of the thread's nodes (only warps with a stretched or boundary node)
-    C am[NPT], ap[NPT], bm[NPT], bp[NPT], cc[NPT];
-    R sx_[NPT], sy_[NPT];
+    constexpr int NY = PAIR ? 1 : NPT;  // rows of the thread's nodes (a pair lies in one row)
+    C am[NPT], ap[NPT], bm[NY], bp[NY], cc[NPT];
+    R sx_[NPT], sy_[NY];
     R cc0[NPT];  // Re cc with the z axis unstretched
 
     double accd = 0.0;
+    // sum of |output|^2: FP32 over 4 planes, then FP64 (pairs past the chunk's end are left out at the end)
     R accf = R(0);
     C fc[NPT], q[NPT];
 #pragma unroll
@@ -357,7 +383,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
     if constexpr (GRAD)
       for (int k = 0; k < z1 - z0; ++k)
 #pragma unroll
-        for (int r = 0; r < NPT; ++r) gacc[k * kLinChunk + tid + r * NC] = 0.0;
+        for (int r = 0; r < NPT; ++r) gacc[k * L + tid + r * NC] = 0.0;
 
     auto wait = [&]() -> bool {
       if (mbar_try_wait(&full[st], par)) return true;
@@ -408,14 +434,14 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         if (G.q) rr = rr - q_at<R>(G, sl, (long long)kp * plane + e0 + r * RS);
         else if (kp == src_k && r == src_r) rr = rr - a_src;
         C u = fc[r];
-        if (g) u = smul(sy_[r], smul(sx_[r], u));
+        if (g) u = smul(sy_[PAIR ? 0 : r], smul(sx_[r], u));
         if (z) u = smul(hs, u);
-        gacc[(kp - z0) * kLinChunk + tid + r * NC] += (double)(om2 * (u.x * rr.x + u.y * rr.y));
+        gacc[(kp - z0) * L + tid + r * NC] += (double)(om2 * (u.x * rr.x + u.y * rr.y));
         accd += 0.5 * (double)abs2(rr);
       }
     };
-    // the finished stencil t of plane kp: mask, right-hand side, store, norm (ok: the plane is the item's)
-    auto emit = [&](int kp, C (&t)[NPT], bool ok) {
+    // the finished stencil t of plane kp: mask, right-hand side, store, norm
+    auto emit = [&](int kp, C (&t)[NPT]) {
       if (MODE == M_P1 && kp == src_k) {
 #pragma unroll
         for (int r = 0; r < NPT; ++r)
@@ -426,7 +452,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         for (int r = 0; r < NPT; ++r) {
           C rr = czero<R>() - t[r];
           if (G.q) {
-            if (own[r] && ok) rr = q_at<R>(G, sl, (long long)kp * plane + e0 + r * RS) - t[r];
+            if (own[r] && kp >= z0) rr = q_at<R>(G, sl, (long long)kp * plane + e0 + r * RS) - t[r];
           } else if (kp == src_k && r == src_r) {
             rr = G.masked ? czero<R>() : a_src - t[r];
           }
@@ -437,7 +463,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         // refinement inner solve: s = S^H r + S^H r64
         const float2* pG = (const float2*)G.gvec + (pO - (OC*)G.s);
         if constexpr (PAIR) {
-          if (own[0] && ok) {
+          if (own[0]) {
             const float4 gv = __ldg(reinterpret_cast<const float4*>(pG));
             t[0] = t[0] + lo2(gv);
             t[1] = t[1] + hi2(gv);
@@ -445,14 +471,14 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         } else {
 #pragma unroll
           for (int r = 0; r < NPT; ++r)
-            if (own[r] && ok) t[r] = t[r] + to_c(__ldg(pG + r * RS), R(0));
+            if (own[r]) t[r] = t[r] + to_c(__ldg(pG + r * RS), R(0));
         }
       }
       uint32_t skip = 0;
       if ((MODE == M_P2 || MODE == M_SH) && rcb) {
         // receivers of this plane: left to the finalizer (rec_col_bits), or (FP64 normal residual of the
         // refinement, where A^H F and lambda P^T r2 nearly cancel) added here before the one rounding
-        if (ok) {
+        if (kp >= z0) {
           const uint32_t* pm = G.rmask + ((long long)sl * nz + kp) * ny * G.rw;
 #pragma unroll
           for (int r = 0; r < NPT; ++r)
@@ -467,18 +493,21 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         }
       }
       if constexpr (PAIR && sizeof(OR) == 4) {
-        if (own[0] && ok) st4(pO, t[0], t[1]);
+        if (own[0]) st4(pO, t[0], t[1]);
       } else {
 #pragma unroll
         for (int r = 0; r < NPT; ++r)
-          if (own[r] && ok) pO[r * RS] = to_c(t[r], OR(0));
+          if (own[r]) pO[r * RS] = to_c(t[r], OR(0));
       }
       pO += plane;
       if (NORM) {
-        // per-thread partial sum: FP32 over 4 planes, then FP64
+        R s2 = R(0);
 #pragma unroll
-        for (int r = 0; r < NPT; ++r)
-          if (own[r] && ok && !((skip >> r) & 1u)) accf += fma_r(t[r].x, t[r].x, t[r].y * t[r].y);
+        for (int r = 0; r < NPT; ++r) {
+          const R a2 = fma_r(t[r].x, t[r].x, t[r].y * t[r].y);
+          s2 += (((skip >> r) & 1u) || !(PAIR || own[r])) ? R(0) : a2;
+        }
+        accf += s2;
         if (sizeof(R) == 8 || (kp & 3) == 3) {
           accd += (double)accf;
           accf = R(0);
@@ -492,12 +521,14 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         const AxisCoef<R> cy_ = axis_coef<R, CONJ>(tab, nj[r], ny, npml, ih2);
         am[r] = cx_.am;
         ap[r] = cx_.ap;
-        bm[r] = cy_.am;
-        bp[r] = cy_.ap;
+        if (r < NY) {
+          bm[r] = cy_.am;
+          bp[r] = cy_.ap;
+          sy_[r] = cy_.im;
+        }
         cc[r] = cx_.a0 + cy_.a0;
         cc0[r] = cc[r].x - R(2) * ih2;
         sx_[r] = cx_.im;
-        sy_[r] = cy_.im;
       }
     }
     // One plane of the item: its F, the z + 1 term of plane k - 1, and its own stencil without that term.
@@ -570,12 +601,12 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         for (int r = 0; r < NPT; ++r) {
           const C d = DIFF ? v[r] - fc[r] : v[r];
           t[r] = ZG ? cfma(hz, d, q[r]) : rfma(ih2, d, q[r]);
-          if (GEN) t[r] = smul(sy_[r], smul(sx_[r], t[r]));
+          if (GEN) t[r] = smul(sy_[PAIR ? 0 : r], smul(sx_[r], t[r]));
         }
         if constexpr (GRAD) {
           if (k > z0) accum(k - 1, t, GEN, ZG);
         } else {
-          emit(k - 1, t, k > z0);
+          emit(k - 1, t);
         }
       }
       AxisCoef<R> cz;
@@ -587,11 +618,12 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
       for (int r = 0; r < NPT; ++r) {
         if (GEN) {
           // outside the grid: zero (the stage holds other rows or nothing there)
-          if (ni[r] == 0) l[r] = czero<R>();
-          if (ni[r] == nx - 1) rgt[r] = czero<R>();
+          // (of a pair in a row of even length only the first node can lie at its start, the second at its end)
+          if (!(PAIR && r == 1) && ni[r] == 0) l[r] = czero<R>();
+          if (!(PAIR && r == 0) && ni[r] == nx - 1) rgt[r] = czero<R>();
           if (edge) {
-            if (nj[r] == 0) ym[r] = czero<R>();
-            if (nj[r] == ny - 1) yp[r] = czero<R>();
+            if (nj[PAIR ? 0 : r] == 0) ym[r] = czero<R>();
+            if (nj[PAIR ? 0 : r] == ny - 1) yp[r] = czero<R>();
           }
         }
         if (DIFF) {
@@ -619,8 +651,8 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         if (GEN) {
           acc = cfma(am[r], l[r], acc);
           acc = cfma(ap[r], rgt[r], acc);
-          acc = cfma(bm[r], ym[r], acc);
-          acc = cfma(bp[r], yp[r], acc);
+          acc = cfma(bm[PAIR ? 0 : r], ym[r], acc);
+          acc = cfma(bp[PAIR ? 0 : r], yp[r], acc);
           acc = ZG ? cfma(cz.am, zm, acc) : rfma(ih2, zm, acc);
         } else {
           C sum = (l[r] + rgt[r]) + (ym[r] + yp[r]);
@@ -631,6 +663,11 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         q[r] = ZG ? smul(cz.im, acc) : acc;
         fc[r] = v[r];
       }
+      if (!GRAD && k == z0) {  // what this step finished was no plane of the item
+        pO -= plane;
+        accf = R(0);
+        accd = 0.0;
+      }
       release();
       return true;
     };
@@ -640,9 +677,10 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
       int k = z0;
       for (; k < za; ++k)
         if (!step(gen_c, std::true_type(), k)) return false;
+      const int kl = k;
       for (; k < zb; ++k)
         if (!step(gen_c, std::false_type(), k)) return false;
-      if (k > za || za == z0) {
+      if (k > kl) {  // the pending plane is an interior one
         hz = mkc(ih2, R(0));
         hs = R(0);
       }
@@ -678,7 +716,12 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         da = (da + pstep) & 15;
         db = (db + pstep) & 15;
       }
-      if (!dead) dead = gen ? !planes(std::true_type()) : !planes(std::false_type());
+      if (idle) {
+        for (int k = z0; k < z1 && !dead; ++k) {
+          dead = !wait();
+          if (!dead) release();
+        }
+      } else if (!dead) dead = gen ? !planes(std::true_type()) : !planes(std::false_type());
       if (!dead) {
         // the plane above completes the last one
         C v[NPT];
@@ -698,14 +741,15 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
 #pragma unroll
           for (int r = 0; r < NPT; ++r) {
             t[r] = cfma(hz, DIFF ? v[r] - fc[r] : v[r], q[r]);
-            if (gen) t[r] = smul(sy_[r], smul(sx_[r], t[r]));
+            if (gen) t[r] = smul(sy_[PAIR ? 0 : r], smul(sx_[r], t[r]));
           }
           if constexpr (GRAD) accum(z1 - 1, t, gen, true);
-          else emit(z1 - 1, t, true);
+          else emit(z1 - 1, t);
         }
       }
     }
-    accd += (double)accf;
+    accd = PAIR && !own[0] ? 0.0 : accd + (double)accf;
+
 
     if (MODE == M_APPLY) {
       if (!dead) continue;
@@ -727,7 +771,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
       for (int k = z0; k < z1; ++k)
 #pragma unroll
         for (int r = 0; r < NPT; ++r)
-          if (own[r]) G.grad[(long long)k * plane + e0 + r * RS] += gacc[(k - z0) * kLinChunk + tid + r * NC];
+          if (own[r]) G.grad[(long long)k * plane + e0 + r * RS] += gacc[(k - z0) * L + tid + r * NC];
       if (tid == 0 && tsum != 0.0) atomicAdd(b.f, tsum);
       continue;
     }
