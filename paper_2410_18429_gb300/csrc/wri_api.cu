@@ -153,6 +153,7 @@ void decompose_lin(const wri_grid& g, int zs, GroupDev& G) {
   G.zsplit = (g.nz + G.zc - 1) / G.zc;
   G.ntiles = G.tiles_x * G.zsplit;
   G.rw = (g.nx + 31) / 32;
+  G.zw = (g.nz + 31) / 32;
 }
 
 // z-chunks per tile column when the caller leaves it open: the count that minimises the modelled
@@ -397,7 +398,7 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
   for (int gi = 0; gi < ngroups; ++gi) {  // receiver bitmaps (one bit per node and system)
     const GroupDev& G = P.g[gi];
     P.rcol_bytes[gi] = 4 * (size_t)G.nsys * G.ny * G.rw;
-    P.rmask_bytes[gi] = P.rcol_bytes[gi] * (size_t)G.nz;
+    P.rmask_bytes[gi] = G.zw ? 4 * (size_t)G.nsys * G.nx * G.ny * G.zw : P.rcol_bytes[gi] * (size_t)G.nz;
     P.off_rcol[gi] = off;
     off += align_up(P.rcol_bytes[gi]);
     P.off_rmask[gi] = off;

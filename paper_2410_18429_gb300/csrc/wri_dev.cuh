@@ -144,6 +144,7 @@ struct GroupDev {
   int tiles_x, tiles_y, zsplit, zc, ntiles;
   int chunk;               // chunk kernels: nodes of a chunk of the x-y plane (tiles_x chunks, tiles_y = 1)
   int rw;                  // words of a row of the receiver bitmaps
+  int zw;                  // chunk kernels: words of a column of rmask, which runs along z (0: along x)
   long long xitem0;        // chunk kernels: first work item of the group in the iterate-update pass
   long long item0, nitems;  // work items (tile x system) of the group in the batched launch
   int masked;               // 1 = source-free (Z applied), 0 = known weight or general right-hand side
@@ -167,7 +168,9 @@ struct GroupDev {
   const int* rmap;          // [nsys][n] receiver entry of a node (-1: none): the FP64 S^H kernels of
                             // the refinement add lambda P^T r2 in the stencil pass (or null)
   const uint32_t* rmask;    // [nsys][nz][ny][rw] receiver bits of the normal-residual norms
-                            // (bit b of word (k, j, t): node (32 t + b, j, k) is a receiver), or null
+                            // (bit b of word (k, j, t): node (32 t + b, j, k) is a receiver), or null;
+                            // chunk kernels: [nsys][ny][nx][zw], bit b of word (j, i, t): node (i, j, 32 t + b),
+                            // so that a thread reads its column's receivers once per 32 planes
   const uint32_t* rcol;     // [nsys][ny][rw] OR of rmask over k (columns holding a receiver)
   double* grad;             // [n] gradient accumulator (gradient kernel only)
   const float2* ztab;       // [2][nz][3] z-axis coefficients (s_z, 1/(s_z(k-1/2) h^2), 1/(s_z(k+1/2) h^2)),

@@ -141,6 +141,54 @@ __device__ __forceinline__ R model_smem(const unsigned char* p, int m_double, in
   return R(reinterpret_cast<const float*>(p)[e]);
 }
 
+// The system's scalars, run by the NT consumer threads of the CTA that finished its last item.  Phase 1 adds
+// lambda^2 |p|^2 of the receivers; phase 2 moves the receiver residual (r2 -= alpha lambda p, with the p that
+// phase 1 stored) and adds lambda P^T r2 to s.
+// One reduction, no vector that this launch wrote but at the receivers: with the fences that leaves
+// (148^3 x 1 system 79.7 -> 71.9 us per iteration, x 64 sources x 3 grids 2331 -> 2266; half of it from the
+// receivers' bits, which cost the borehole's CTAs a global load per plane when rows of x held them).
+template <typename R, typename OR, int MODE, int NT, typename SYNC>
+__device__ void finalize_lin(const Batch& b, const GroupDev& G, SysDev* sd, int sl, double* red) {
+  typedef cx<R> C;
+  typedef cx<OR> OC;
+  const int tid = threadIdx.x;
+  const long long off = (long long)sl * G.n;
+  double part = 0.0;  // sums of the items, in item order per thread
+  if (MODE != M_RES) {
+    const double* pp = b.partial + sd->part_off;
+    for (int t = tid; t < G.ntiles; t += NT) part += __ldcg(pp + t);
+  }
+  const R lam = R(G.lambda);
+  C* r2 = (C*)b.r2;
+  const R step = MODE == M_P2 ? R(sd->alpha * (double)lam) : R(0);
+  const C* p = (MODE == M_P1 || MODE == M_P2) ? (const C*)G.p[pslot(b, sd->iter)] + off : nullptr;
+  if (!(MODE == M_SH && G.rmap)) {
+    for (int k = sd->rec_begin + tid; k < sd->rec_end; k += NT) {
+      const int node = b.rec_idx[k];
+      if (MODE == M_P1) {
+        part += (double)lam * (double)lam * (double)abs2(ldcg_c(p + node));
+      } else if (MODE == M_RES) {
+        r2[k] = ((const C*)b.lamd)[k] - lam * ldcg_c((const C*)G.x + off + node);
+      } else {
+        C r = r2[k];
+        if (MODE == M_P2) r2[k] = r = r - step * ldcg_c(p + node);
+        OC* S = (OC*)G.s + off + node;
+        // the stencil pass left receiver nodes out of its partial sums
+        const OC sn = to_c(to_c(ldcg_c(S), R(0)) + lam * r, OR(0));
+        *S = sn;
+        part += (double)abs2(sn);
+      }
+    }
+  }
+  const double tot = block_sum<NT, SYNC>(part, red);
+  if (tid == 0) {
+    if (MODE == M_P1) p1_scalars(b, sd, tot);
+    if (MODE == M_P2) p2_scalars(b, sd, tot);
+    if (MODE == M_SH) sh_scalars(b, sd, tot);
+    sd->ticket = 0u;
+  }
+}
+
 // R: arithmetic; OR: type of the stencil's output vector; MODE: M_APPLY, M_SH, M_RES, M_P1, M_P2 or M_GRAD; NC
 // consumer threads of NPT nodes each; GV: phase 2 adds S^H r64 (gvec); PAIR: a thread's two nodes are adjacent (16-byte accesses: nx even
 // and every pointer aligned), otherwise they lie NC apart; S stages.
@@ -164,7 +212,6 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
   typedef FirstThreadsSync<NC> CSync;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ double red[NCW];
-  __shared__ double bcast;
   __shared__ int s_last;
   __shared__ volatile int s_abort;
   __shared__ R s_tab[MODE == M_APPLY ? kLinInlineTab * kLayerTab : 1];
@@ -318,8 +365,8 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
     const int e0 = c0 + (PAIR ? 2 * tid : tid);
     bool own[NPT];
     int ni[NPT], nj[NPT];
-    uint32_t rcb = 0;  // receivers of this system in the thread's columns
-    int ri[NPT];
+    uint32_t rcb = 0;      // the thread's columns that hold receivers of this system
+    uint32_t rz[NPT] = {};  // their receivers at the current 32 planes
     bool gen = false;  // a stretched axis or a neighbour outside the grid
 #pragma unroll
     for (int r = 0; r < NPT; ++r) {
@@ -329,10 +376,8 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
       ni[r] = ee - nj[r] * nx;
       const int w = npml > 0 ? npml + 1 : 1;
       gen = gen || (own[r] && !(ni[r] >= w && ni[r] < nx - w && nj[r] >= w && nj[r] < ny - w));
-      ri[r] = 0;
-      if ((MODE == M_P2 || MODE == M_SH) && G.rmask && own[r]) {
-        ri[r] = nj[r] * G.rw + (ni[r] >> 5);
-        if ((__ldg(G.rcol + (long long)sl * ny * G.rw + ri[r]) >> (ni[r] & 31)) & 1u) rcb |= 1u << r;
+      if (NORM && G.rmask && own[r]) {
+        if ((__ldg(G.rcol + ((long long)sl * ny + nj[r]) * G.rw + (ni[r] >> 5)) >> (ni[r] & 31)) & 1u) rcb |= 1u << r;
       }
     }
     gen = __any_sync(0xffffffffu, gen);
@@ -478,19 +523,21 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
       if ((MODE == M_P2 || MODE == M_SH) && rcb) {
         // receivers of this plane: left to the finalizer (rec_col_bits), or (FP64 normal residual of the
         // refinement, where A^H F and lambda P^T r2 nearly cancel) added here before the one rounding
-        if (kp >= z0) {
-          const uint32_t* pm = G.rmask + ((long long)sl * nz + kp) * ny * G.rw;
+        if (kp == z0 || (kp > z0 && (kp & 31) == 0)) {
 #pragma unroll
           for (int r = 0; r < NPT; ++r)
-            if (((rcb >> r) & 1u) && ((__ldg(pm + ri[r]) >> (ni[r] & 31)) & 1u)) {
-              if (MODE == M_SH && G.rmap) {
-                const int rk = G.rmap[off + (long long)kp * plane + e0 + r * RS];
-                t[r] = t[r] + R(G.lambda) * ((const C*)b.r2)[rk];
-              } else {
-                skip |= 1u << r;
-              }
-            }
+            rz[r] = ((rcb >> r) & 1u) ? __ldg(G.rmask + ((long long)sl * plane + e0 + r * RS) * G.zw + (kp >> 5)) : 0u;
         }
+#pragma unroll
+        for (int r = 0; r < NPT; ++r)
+          if (kp >= z0 && ((rz[r] >> (kp & 31)) & 1u)) {
+            if (MODE == M_SH && G.rmap) {
+              const int rk = G.rmap[off + (long long)kp * plane + e0 + r * RS];
+              t[r] = t[r] + R(G.lambda) * ((const C*)b.r2)[rk];
+            } else {
+              skip |= 1u << r;
+            }
+          }
       }
       if constexpr (PAIR && sizeof(OR) == 4) {
         if (own[0]) st4(pO, t[0], t[1]);
@@ -778,14 +825,16 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
     // the copy warp may raise the flag at any time: decide on one reduced value
     if (first_threads_any<NC>(s_abort != 0)) break;
     if (tid == 0 && NORM) b.partial[sd->part_off + tile] = tsum;
-    __threadfence();
+    // what the finalizing CTA reads of this one: the partial sum, and p or s at the receivers
+    if (tid == 0 || rcb) __threadfence();
     CSync::sync();
     if (tid == 0) {
       const unsigned t = atomicAdd(&sd->ticket, 1u);
       s_last = (t == (unsigned)(G.ntiles - 1));
+      __threadfence();
     }
     CSync::sync();
-    if (s_last) finalize<R, OR, MODE, NC, CSync>(b, G, sd, sl, false, red, &bcast);
+    if (s_last) finalize_lin<R, OR, MODE, NC, CSync>(b, G, sd, sl, red);
   }
 }
 

@@ -15,6 +15,54 @@ __device__ __forceinline__ cx<R> ldg_c(const cx<R>* p) {
 }
 
 // ------------------------------------------------------------------ finalizers
+// Scalars of a system after phase 1, with delta = ||S p||^2 (one thread); returns the step, 0 on breakdown.
+__device__ inline double p1_scalars(const Batch& b, SysDev* sd, double delta) {
+  double alpha = 0.0;
+  sd->delta = delta;
+  if (!(delta > 0.0) || !isfinite(delta)) {
+    sd->status = isfinite(delta) ? WRI_SYS_BREAKDOWN : WRI_SYS_NONFINITE;
+    if (sd->iter % xsteps_of(b) != 0) {
+      // grouped updates: steps of earlier iterations are still pending (this pass added none);
+      // the step history is left as it is, newest = the previous iteration's, and the x-only
+      // pass adds them
+      sd->state = ST_FINISHING;
+    } else {
+      sd->state = ST_DONE;
+      sd->alpha = 0.0;
+      atomicSub(b.remaining, 1);
+    }
+  } else {
+    alpha = sd->gamma / delta;
+    sd->alpha_hist[2] = sd->alpha_hist[1];
+    sd->alpha_hist[1] = sd->alpha_hist[0];
+    sd->alpha_hist[0] = sd->alpha;
+    sd->alpha = alpha;
+  }
+  return alpha;
+}
+
+// ... and after phase 2, with g = ||s||^2.
+__device__ inline void p2_scalars(const Batch& b, SysDev* sd, double g) {
+  const int it = sd->iter + 1;
+  sd->iter = it;
+  sd->iter_total += 1;
+  const double rn = sqrt(g);
+  sd->relres = sd->snorm_ref > 0.0 ? rn / sd->snorm_ref : 0.0;
+  if (!isfinite(g)) {
+    sd->status = WRI_SYS_NONFINITE;
+    sd->state = ST_FINISHING;
+  } else if (rn <= sd->tol * sd->snorm_ref) {
+    sd->status = WRI_SYS_OK;
+    sd->state = ST_FINISHING;
+  } else if (it >= b.max_iter) {
+    sd->status = WRI_SYS_MAXITER;
+    sd->state = ST_FINISHING;
+  } else {
+    sd->beta = g / sd->gamma;
+  }
+  sd->gamma = g;
+}
+
 // Scalars of a system after s = S^H r, with g = ||s||^2 (one thread).
 __device__ inline void sh_scalars(const Batch& b, SysDev* sd, double g) {
   const double rn = sqrt(g);
@@ -143,49 +191,9 @@ __device__ void finalize(const Batch& b, const GroupDev& G, SysDev* sd, int sl, 
   if (tid == 0) {
     const double tot = part + rec;
     if (MODE == M_P1) {
-      const double delta = tot;
-      double alpha = 0.0;
-      sd->delta = delta;
-      if (!(delta > 0.0) || !isfinite(delta)) {
-        sd->status = isfinite(delta) ? WRI_SYS_BREAKDOWN : WRI_SYS_NONFINITE;
-        if (sd->iter % xsteps_of(b) != 0) {
-          // grouped updates: steps of earlier iterations are still pending (this pass added none);
-          // the step history is left as it is, newest = the previous iteration's, and the x-only
-          // pass adds them
-          sd->state = ST_FINISHING;
-        } else {
-          sd->state = ST_DONE;
-          sd->alpha = 0.0;
-          atomicSub(b.remaining, 1);
-        }
-      } else {
-        alpha = sd->gamma / delta;
-        sd->alpha_hist[2] = sd->alpha_hist[1];
-        sd->alpha_hist[1] = sd->alpha_hist[0];
-        sd->alpha_hist[0] = sd->alpha;
-        sd->alpha = alpha;
-      }
-      *bcast = alpha;  // step of the receiver residual (none on breakdown)
+      *bcast = p1_scalars(b, sd, tot);  // step of the receiver residual (none on breakdown)
     } else if (MODE == M_P2) {
-      const double g = tot;
-      const int it = sd->iter + 1;
-      sd->iter = it;
-      sd->iter_total += 1;
-      const double rn = sqrt(g);
-      sd->relres = sd->snorm_ref > 0.0 ? rn / sd->snorm_ref : 0.0;
-      if (!isfinite(g)) {
-        sd->status = WRI_SYS_NONFINITE;
-        sd->state = ST_FINISHING;
-      } else if (rn <= sd->tol * sd->snorm_ref) {
-        sd->status = WRI_SYS_OK;
-        sd->state = ST_FINISHING;
-      } else if (it >= b.max_iter) {
-        sd->status = WRI_SYS_MAXITER;
-        sd->state = ST_FINISHING;
-      } else {
-        sd->beta = g / sd->gamma;
-      }
-      sd->gamma = g;
+      p2_scalars(b, sd, tot);
     } else if (MODE == M_SH) {
       sh_scalars(b, sd, tot);
     }

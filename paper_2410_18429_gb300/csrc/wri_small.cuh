@@ -45,7 +45,8 @@ __global__ void k_rmask(const __grid_constant__ Batch b, int nsys_total) {
     const int y = (int)(rem / G.nx);
     const int x = (int)(rem - (long long)y * G.nx);
     const uint32_t bit = 1u << (x & 31);
-    atomicOr(mask + (((long long)sd.local * G.nz + z) * G.ny + y) * G.rw + (x >> 5), bit);
+    if (G.zw) atomicOr(mask + ((long long)sd.local * plane + rem) * G.zw + (z >> 5), 1u << (z & 31));
+    else atomicOr(mask + (((long long)sd.local * G.nz + z) * G.ny + y) * G.rw + (x >> 5), bit);
     atomicOr(col + ((long long)sd.local * G.ny + y) * G.rw + (x >> 5), bit);
   }
 }
