@@ -140,12 +140,12 @@ void decompose(const wri_grid& g, int by, int zs_req, GroupDev& G) {
   G.rw = (g.nx + 31) / 32;
 }
 
-// The same for the chunk kernels: equal chunks of at most kLinChunk nodes of the x-y plane.
-int lin_chunks(const wri_grid& g) { return (int)(((long long)g.nx * g.ny + kLinChunk - 1) / kLinChunk); }
+// The same for the chunk kernels: equal chunks of at most `most` nodes of the x-y plane.
+int lin_chunks(const wri_grid& g, int most = kLinChunk) { return (int)(((long long)g.nx * g.ny + most - 1) / most); }
 
-void decompose_lin(const wri_grid& g, int zs, GroupDev& G) {
+void decompose_lin(const wri_grid& g, int most, int zs, GroupDev& G) {
   const int zs_req = std::max(1, std::min(zs, g.nz));
-  const int plane = g.nx * g.ny, nch = lin_chunks(g);
+  const int plane = g.nx * g.ny, nch = lin_chunks(g, most);
   G.chunk = ((plane + nch - 1) / nch + 31) / 32 * 32;
   G.tiles_x = (plane + G.chunk - 1) / G.chunk;
   G.tiles_y = 1;
@@ -177,23 +177,54 @@ int auto_zsplit(long long xy_items, int nz) {
   return best;
 }
 
-// The same for the chunk kernels, with chunks of at least one plane.  complex64: waves of 4 CTAs per SM
-// times the planes an item streams.  complex128: the FP64 pipe binds, so the planes per SM count, and a
-// little for the planes next to the chunk.
-int auto_zsplit_lin(long long xy_items, int nz, bool wide) {
+// The same for the chunk kernels, with chunks of at least one plane: waves of 4 CTAs per SM times the planes an
+// item streams.
+int auto_zsplit_lin(long long xy_items, int nz) {
   int best = 1;
   double best_cost = 0.0;
   for (int zs = 1; zs <= 64 && zs <= nz; ++zs) {
     const int zc = (nz + zs - 1) / zs;
     const long long items = xy_items * ((nz + zc - 1) / zc);
-    const long long wave = (long long)kRefSMs * (wide ? 1 : 4);
-    const double cost = (double)((items + wave - 1) / wave) * (wide ? zc : zc + 2) + (wide ? 0.3 * (zc + 2) : 0.0);
+    const long long wave = (long long)kRefSMs * 4;
+    const double cost = (double)((items + wave - 1) / wave) * (zc + 2);
     if (zs == 1 || cost < best_cost) {
       best_cost = cost;
       best = zs;
     }
   }
   return best;
+}
+
+// Chunk length and z-chunks of the chunk kernels in complex128, where the FP64 pipe binds.  Modelled time of the
+// fullest SM: two items at a time, a plane of one item takes 1.3 us and 0.0063 us per node on its own, two items
+// the FP64 pipe's 0.0245 us per node, and an item 0.7 planes more than it has.  Chunks below 256 nodes only while
+// an SM has at most two items (with more, the fuller CTAs win: 81^3 x 9 883 us per iteration against 890-1010).
+// A sweep over both gave, in us per iteration: 36^3 x 1 39 (whole columns of 256 nodes: 228), 48^3 x 4 118 (337),
+// 81^3 x 9 883 (1057), 116^3 x 4 1031 (1358).
+void wide_shape(const wri_grid* grids, const int* nsys, int ngroups, int* most, int* zsplit) {
+  double best_cost = 0.0;
+  int nz = 0;
+  for (int gi = 0; gi < ngroups; ++gi) nz = std::max(nz, grids[gi].nz);
+  for (int c = kLinChunk; c >= 128; c -= 32)
+    for (int zs = 1; zs <= 64 && zs <= nz; ++zs) {
+      const int zc = (nz + zs - 1) / zs;
+      long long items = 0;
+      int chunk = 0;
+      for (int gi = 0; gi < ngroups; ++gi) {
+        const int nch = lin_chunks(grids[gi], c);
+        items += (long long)nsys[gi] * nch * ((grids[gi].nz + zc - 1) / zc);
+        chunk = std::max(chunk, (int)(((long long)grids[gi].nx * grids[gi].ny + nch - 1) / nch));
+      }
+      const long long n = (items + kRefSMs - 1) / kRefSMs;
+      if (c < kLinChunk && n > 2) continue;
+      const double one = 1.3 + 0.0063 * chunk, two = std::max(one, 0.0245 * chunk);
+      const double cost = ((double)(n / 2) * two + (double)(n % 2) * one) * (zc + 0.7);
+      if (best_cost == 0.0 || cost < best_cost) {
+        best_cost = cost;
+        *most = c;
+        *zsplit = zs;
+      }
+    }
 }
 
 int validate_groups(const wri_group* groups, int ngroups, bool need_data) {
@@ -355,8 +386,19 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
   }
   int nz_max = 0;
   for (int gi = 0; gi < ngroups; ++gi) nz_max = std::max(nz_max, groups[gi].grid.nz);
+  int most = kLinChunk, wide_zs = 0;
+  if (P.lin && o->dtype == WRI_C128 && o->zsplit == 0) {
+    std::vector<wri_grid> grids(ngroups);
+    std::vector<int> ns(ngroups);
+    for (int gi = 0; gi < ngroups; ++gi) {
+      grids[gi] = groups[gi].grid;
+      ns[gi] = groups[gi].nsys;
+    }
+    wide_shape(grids.data(), ns.data(), ngroups, &most, &wide_zs);
+  }
   const int zs = o->zsplit > 0 ? o->zsplit
-                 : P.lin       ? auto_zsplit_lin(xy_items, nz_max, o->dtype == WRI_C128)
+                 : wide_zs > 0 ? wide_zs
+                 : P.lin       ? auto_zsplit_lin(xy_items, nz_max)
                                : auto_zsplit(o->plain ? xy_items / std::max(1, P.nsys_total) : xy_items, nz_max);
   long long item = 0, parts = 0;
   int sys0 = 0;
@@ -365,7 +407,7 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
     GroupDev& G = P.g[gi];
     std::memset(&G, 0, sizeof(G));
     fill_geom(G, groups[gi].grid);
-    if (P.lin) decompose_lin(groups[gi].grid, zs, G);
+    if (P.lin) decompose_lin(groups[gi].grid, most, zs, G);
     else decompose(groups[gi].grid, P.by, zs, G);
     G.nsys = groups[gi].nsys;
     G.sys0 = sys0;
@@ -1269,7 +1311,10 @@ int apply_common(const wri_grid* grid, int dtype, const void* m, int nsys, const
     b.pair = rb == 4 && grid->nx % 2 == 0 && ((uintptr_t)x | (uintptr_t)y) % 16 == 0 && (uintptr_t)m % 8 == 0;
     b.order = 3;
     b.sblock = 16;
-    decompose_lin(*grid, auto_zsplit_lin((long long)nsys * lin_chunks(*grid), grid->nz, rb == 8), G);
+    int most = kLinChunk, zs = 1;
+    if (rb == 8) wide_shape(grid, &nsys, 1, &most, &zs);
+    else zs = auto_zsplit_lin((long long)nsys * lin_chunks(*grid), grid->nz);
+    decompose_lin(*grid, most, zs, G);
     G.nitems = (long long)G.ntiles * nsys;
     b.nitems = G.nitems;
     std::vector<double> tab;
@@ -1389,7 +1434,7 @@ int gradient_pass(const wri_group* groups, const Plan& P, Batch& b, const char* 
     long long item = 0;
     for (int gi = 0; gi < b.ngroups; ++gi) {
       GroupDev& G = b.g[gi];
-      decompose_lin(groups[gi].grid, (G.nz + zc - 1) / zc, G);
+      decompose_lin(groups[gi].grid, kLinChunk, (G.nz + zc - 1) / zc, G);
       G.item0 = item;
       G.nitems = G.ntiles;
       item += G.nitems;

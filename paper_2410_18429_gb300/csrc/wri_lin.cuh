@@ -207,6 +207,9 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
   // complex64 forms the stencil from differences to the node, which are exact or nearly so for a resolved
   // field; complex128 from the values, with the diagonal in one coefficient (up to 12 FP64 instructions less)
   constexpr bool DIFF = sizeof(R) == 4;
+  // complex64: the first step of an item finishes a plane below it all the same (no check in the loop) and
+  // its result is overwritten; complex128 saves the FP64 instructions
+  constexpr bool DUMMY = sizeof(R) == 4;
   constexpr int CB = sizeof(C);
   constexpr int RS = PAIR ? 1 : NC;  // distance of a thread's nodes
   typedef FirstThreadsSync<NC> CSync;
@@ -642,7 +645,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
           }
         }
       }
-      {
+      if (DUMMY || k > z0) {
         C t[NPT];
 #pragma unroll
         for (int r = 0; r < NPT; ++r) {
@@ -651,7 +654,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
           if (GEN) t[r] = smul(sy_[PAIR ? 0 : r], smul(sx_[r], t[r]));
         }
         if constexpr (GRAD) {
-          if (k > z0) accum(k - 1, t, GEN, ZG);
+          accum(k - 1, t, GEN, ZG);
         } else {
           emit(k - 1, t);
         }
@@ -710,7 +713,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         q[r] = ZG ? smul(cz.im, acc) : acc;
         fc[r] = v[r];
       }
-      if (!GRAD && k == z0) {  // what this step finished was no plane of the item
+      if (DUMMY && k == z0) {  // what this step finished was no plane of the item
         pO -= plane;
         accf = R(0);
         accd = 0.0;
