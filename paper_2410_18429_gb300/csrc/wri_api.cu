@@ -386,18 +386,28 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
   }
   int nz_max = 0;
   for (int gi = 0; gi < ngroups; ++gi) nz_max = std::max(nz_max, groups[gi].grid.nz);
-  int most = kLinChunk, wide_zs = 0;
+  // complex128: the shape of each group's single system while the batch stays small in it, so that a batched
+  // solve sums in the same order as an unbatched one (bit for bit the same iterates); large batches get their own
+  std::vector<int> most(ngroups, kLinChunk), wide_zs(ngroups, 0);
   if (P.lin && o->dtype == WRI_C128 && o->zsplit == 0) {
     std::vector<wri_grid> grids(ngroups);
     std::vector<int> ns(ngroups);
+    const int single = 1;
+    long long items = 0;
     for (int gi = 0; gi < ngroups; ++gi) {
-      grids[gi] = groups[gi].grid;
+      const wri_grid& g = grids[gi] = groups[gi].grid;
       ns[gi] = groups[gi].nsys;
+      wide_shape(&g, &single, 1, &most[gi], &wide_zs[gi]);
+      const int zc = (g.nz + wide_zs[gi] - 1) / wide_zs[gi];
+      items += (long long)ns[gi] * lin_chunks(g, most[gi]) * ((g.nz + zc - 1) / zc);
     }
-    wide_shape(grids.data(), ns.data(), ngroups, &most, &wide_zs);
+    if (items > 8 * kRefSMs) {
+      wide_shape(grids.data(), ns.data(), ngroups, &most[0], &wide_zs[0]);
+      most.assign(ngroups, most[0]);
+      wide_zs.assign(ngroups, wide_zs[0]);
+    }
   }
   const int zs = o->zsplit > 0 ? o->zsplit
-                 : wide_zs > 0 ? wide_zs
                  : P.lin       ? auto_zsplit_lin(xy_items, nz_max)
                                : auto_zsplit(o->plain ? xy_items / std::max(1, P.nsys_total) : xy_items, nz_max);
   long long item = 0, parts = 0;
@@ -407,7 +417,7 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
     GroupDev& G = P.g[gi];
     std::memset(&G, 0, sizeof(G));
     fill_geom(G, groups[gi].grid);
-    if (P.lin) decompose_lin(groups[gi].grid, most, zs, G);
+    if (P.lin) decompose_lin(groups[gi].grid, most[gi], wide_zs[gi] > 0 ? wide_zs[gi] : zs, G);
     else decompose(groups[gi].grid, P.by, zs, G);
     G.nsys = groups[gi].nsys;
     G.sys0 = sys0;
