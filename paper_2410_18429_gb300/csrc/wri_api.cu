@@ -676,7 +676,8 @@ Batch solver_batch(const wri_group* groups, const Plan& P, char* ws, bool inner_
     G.s = ws + P.v_s[gi];
     G.t1 = ws + P.v_t1[gi];
     G.x = (P.ir && inner_view) ? (void*)(ws + P.v_x32[gi]) : U.u;
-    G.x64 = P.ir ? ws + P.v_x64[gi] : nullptr;
+    // the refinement's FP64 solution is built in the caller's array where there is one
+    G.x64 = !P.ir ? nullptr : U.u64 ? U.u64 : (void*)(ws + P.v_x64[gi]);
     G.r64 = P.ir ? ws + P.v_r64[gi] : nullptr;
     G.q64 = P.ir ? ws + P.v_q64[gi] : nullptr;
     G.gvec = (P.ir && inner_view) ? ws + P.v_g32[gi] : nullptr;
@@ -1053,7 +1054,9 @@ int solve_refined(const wri_group* groups, int ngroups, const wri_solve_opts* o,
     outer.g[gi].x = outer.g[gi].x64;
     outer.g[gi].r1[0] = outer.g[gi].q64;
     outer.g[gi].rmap = (const int*)(ws + P.v_rmap[gi]);
-    WRI_CK(cudaMemsetAsync(ws + P.v_rmap[gi], 0xff, 4 * (size_t)P.g[gi].nsys * (size_t)P.g[gi].n, st));
+    // the chunk kernels read the map at receivers only
+    if (!P.lin)
+      WRI_CK(cudaMemsetAsync(ws + P.v_rmap[gi], 0xff, 4 * (size_t)P.g[gi].nsys * (size_t)P.g[gi].n, st));
   }
   WRI_CK(launch_ir_rmap(outer, P.nsys_total, st));
   outer.max_iter = o->max_iter;
@@ -1069,10 +1072,10 @@ int solve_refined(const wri_group* groups, int ngroups, const wri_solve_opts* o,
   if (!P.lin) WRI_CK(launch_ztable(inner, st));  // the outer view shares the tables
   void* u[WRI_MAXG] = {};
   for (int gi = 0; gi < P.ngroups; ++gi) u[gi] = groups[gi].u;
-  // lambda d in FP64 (lamd and q2), x64 = warm ? u : 0, r64 = 0, dx = 0
+  // lambda d in FP64 (lamd and q2)
   WRI_CK(launch_setup_rhs(4, 8, outer, P.nsys_total, st));
-  WRI_CK(launch_ir_init(inner, u, o->warm_start ? 1 : 0, st));
-  if (o->warm_start) {  // ||S^H b|| with the FP64 stencil (q2 still holds lambda d)
+  if (o->warm_start) {  // x64 = u, r64 = 0, dx = 0; ||S^H b|| with the FP64 stencil (q2 still holds lambda d)
+    WRI_CK(launch_ir_init(inner, u, 1, st));
     Batch r = outer;
     r.flavor = SH_REF;
     if (P.lin) {
@@ -1121,7 +1124,11 @@ int solve_refined(const wri_group* groups, int ngroups, const wri_solve_opts* o,
       for (int gi = 0; gi < P.ngroups; ++gi) in.g[gi].gvec = nullptr;  // r64 = 0: no g'
       const int rc = run_loop(P, in, in, M_P2, std::min(K, o->max_iter + 1), o->max_iter, st, tma, &w);
       if (rc != WRI_OK) return rc;
-      WRI_CK(launch_ir_update(inner, st));                         // x64 = dx, r64 = dr
+      WRI_CK(launch_ir_update(inner, true, st));                   // x64 = dx, r64 = dr
+      WRI_CK(cudaMemsetAsync(ws + P.off_r2_64, 0, 16 * (size_t)P.nnz_total, st));
+      WRI_CK(launch_ir_update_rec(inner, P.nsys_total, st));
+    } else {
+      WRI_CK(launch_ir_init(inner, u, 0, st));                     // x64 = r64 = 0
     }
     first_outer = 1;
   }
@@ -1131,12 +1138,12 @@ int solve_refined(const wri_group* groups, int ngroups, const wri_solve_opts* o,
     r.outer = outer_k;
     r.flavor = SH_REFINE;
     WRI_CK(stencil_pass(P, 8, 8, M_RES, r, w, st));                // q = b - S x64
-    WRI_CK(launch_ir_forcing(inner, outer.r2, st));                // f = q - r64 (complex64)
     WRI_CK(stencil_pass(P, 8, 4, M_SH, r, w, st));                 // c = S^H q, outer test
     WRI_CK(cudaMemcpyAsync(slot, outer.remaining, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
     WRI_CK(cudaStreamSynchronize(st));
     if (slot[1] != 0) return WRI_ECUDA;                            // a bounded copy wait timed out
     if (*slot <= 0) break;
+    WRI_CK(launch_ir_forcing(inner, outer.r2, st));                // f = q - r64 (complex64), dx = 0
     Batch in = inner;
     if (outer_k == 0) {
       // r64 = 0 (k_ir_init), so g' = S^H r64 = 0: the first inner solve is plain CGLS, and its
@@ -1147,7 +1154,8 @@ int solve_refined(const wri_group* groups, int ngroups, const wri_solve_opts* o,
     }
     const int rc = run_loop(P, in, in, M_P2, std::min(K, o->max_iter + 1), o->max_iter, st, tma, &w);
     if (rc != WRI_OK) return rc;
-    WRI_CK(launch_ir_update(inner, st));                           // x64 += dx, r64 += dr
+    WRI_CK(launch_ir_update(inner, false, st));                    // x64 += dx, r64 += dr
+    WRI_CK(launch_ir_update_rec(inner, P.nsys_total, st));
     if (outer_k > o->max_refine + 1) return WRI_ECUDA;
   }
   WRI_CK(launch_ir_final(inner, u, st));
@@ -1572,9 +1580,7 @@ int wri_solve_batch(const wri_group* groups, int ngroups, const wri_solve_opts* 
     for (int gi = 0; gi < ngroups; ++gi) {
       if (!groups[gi].u64) continue;
       const long long cnt = (long long)groups[gi].nsys * grid_n(groups[gi].grid);
-      if (P.ir)
-        WRI_CK(cudaMemcpyAsync(groups[gi].u64, ws + P.v_x64[gi], 16 * (size_t)cnt, cudaMemcpyDeviceToDevice, st));
-      else
+      if (!P.ir)
         WRI_CK(launch_widen(groups[gi].u, groups[gi].u64, cnt, st));
     }
   if (P.ir) {  // the workspace now holds b - S u64 in FP64 (the last residual step of every system)

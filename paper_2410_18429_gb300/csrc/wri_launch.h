@@ -28,7 +28,8 @@ cudaError_t launch_ir_init(const Batch& b, void* const* u, int warm, cudaStream_
 cudaError_t launch_ir_rmap(const Batch& b, int nsys_total, cudaStream_t st);  // b: outer view, map filled with -1
 cudaError_t launch_ir_cold(const Batch& b, int nsys_total, cudaStream_t st);  // b: inner view
 cudaError_t launch_ir_forcing(const Batch& b, const void* q2, cudaStream_t st);
-cudaError_t launch_ir_update(const Batch& b, cudaStream_t st);
+cudaError_t launch_ir_update(const Batch& b, bool first, cudaStream_t st);  // first: x64 = dx, r64 = dr
+cudaError_t launch_ir_update_rec(const Batch& b, int nsys_total, cudaStream_t st);
 cudaError_t launch_ir_final(const Batch& b, void* const* u, cudaStream_t st);
 cudaError_t launch_source_estimate(int rbytes, const Batch& b, int nsys_total, double* alpha_out, cudaStream_t st);
 cudaError_t launch_data_term(int rbytes, int dbytes, const Batch& b, int nsys_total, cudaStream_t st);

@@ -1,5 +1,7 @@
 // Launchers of the small kernels (setup, export, refinement, source estimate,
 // data term) and of the unfused baseline path.
+#include <algorithm>
+
 #include "wri_launch.h"
 #include "wri_small.cuh"
 
@@ -73,6 +75,13 @@ static IrU ir_u(void* const* u, int ngroups) {
   return U;
 }
 
+// blocks per group of the refinement's elementwise kernels: 8 per SM, fewer when the groups are small
+static int ir_blocks(const Batch& b) {
+  long long most = 1;
+  for (int g = 0; g < b.ngroups; ++g) most = std::max(most, (long long)b.g[g].nsys * b.g[g].n);
+  return grid_for(most, 256, 8 * 152);
+}
+
 cudaError_t launch_ir_init(const Batch& b, void* const* u, int warm, cudaStream_t st) {
   k_ir_init<<<1024, 256, 0, st>>>(b, ir_u(u, b.ngroups), warm);
   return cudaGetLastError();
@@ -91,17 +100,24 @@ cudaError_t launch_ir_cold(const Batch& b, int nsys_total, cudaStream_t st) {
 }
 
 cudaError_t launch_ir_forcing(const Batch& b, const void* q2, cudaStream_t st) {
-  k_ir_forcing<<<1024, 256, 0, st>>>(b, (const double2*)q2);
+  k_ir_forcing<<<dim3(ir_blocks(b), b.ngroups), 256, 0, st>>>(b, (const double2*)q2);
   return cudaGetLastError();
 }
 
-cudaError_t launch_ir_update(const Batch& b, cudaStream_t st) {
-  k_ir_update<<<1024, 256, 0, st>>>(b);
+cudaError_t launch_ir_update(const Batch& b, bool first, cudaStream_t st) {
+  if (first) k_ir_update<true><<<dim3(ir_blocks(b), b.ngroups), 256, 0, st>>>(b);
+  else k_ir_update<false><<<dim3(ir_blocks(b), b.ngroups), 256, 0, st>>>(b);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_ir_update_rec(const Batch& b, int nsys_total, cudaStream_t st) {
+  if (nsys_total <= 0) return cudaSuccess;
+  k_ir_update_rec<<<nsys_total, 128, 0, st>>>(b, nsys_total);
   return cudaGetLastError();
 }
 
 cudaError_t launch_ir_final(const Batch& b, void* const* u, cudaStream_t st) {
-  k_ir_final<<<1024, 256, 0, st>>>(b, ir_u(u, b.ngroups));
+  k_ir_final<<<dim3(ir_blocks(b), b.ngroups), 256, 0, st>>>(b, ir_u(u, b.ngroups));
   return cudaGetLastError();
 }
 

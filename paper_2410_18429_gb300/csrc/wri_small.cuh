@@ -67,7 +67,7 @@ __global__ void k_loop_ctl(cudaGraphConditionalHandle h, int* counters, int cap)
 //   grad[node] += -omega^2 sum over the group's systems of Re(conj(w u) q1),
 //   f          += 1/2 ||q1||^2 + 1/2 ||q2||^2.
 // One thread per node of group gi (all its systems); b: the outer view (x64 = u, q64 = q1,
-// r2 = q2 in FP64).
+// r2 = q2 in FP64).  FP64 pipe and HBM about even: 116^3 x 32 in 607 us (1017 with the product w u per system).
 __global__ void k_grad_residual(const __grid_constant__ Batch b, int gi, double* grad, double* f) {
   __shared__ double red[8];
   const GroupDev& G = b.g[gi];
@@ -84,20 +84,26 @@ __global__ void k_grad_residual(const __grid_constant__ Batch b, int gi, double*
     const int i = (int)(rem - (long long)j * G.nx);
     const double2 w = stretch_at<double, false>(G.ax, double(i)) * stretch_at<double, false>(G.ay, double(j)) *
                       stretch_at<double, false>(G.az, double(k));
-    double acc = 0.0;
+    // Re(conj(w u) q) = Re(conj(w) conj(u) q): w is taken out of the sum, and where it is 1 only the real
+    // part of conj(u) q is needed (4 FP64 instructions per node and system with the norm, 6 in the layer)
+    const bool layer = w.y != 0.0 || w.x != 1.0;
+    double acc = 0.0, aim = 0.0;
+    const double2* un = u + node;
+    const double2* qn = q + node;
+#pragma unroll 4
     for (int sl = 0; sl < G.nsys; ++sl) {
-      const double2 wu = w * u[(long long)sl * G.n + node];
-      const double2 r = q[(long long)sl * G.n + node];
-      acc += wu.x * r.x + wu.y * r.y;
-      facc += 0.5 * abs2(r);
+      const double2 uv = un[(long long)sl * G.n], r = qn[(long long)sl * G.n];
+      acc = fma(uv.x, r.x, fma(uv.y, r.y, acc));
+      if (layer) aim = fma(uv.x, r.y, fma(-uv.y, r.x, aim));
+      facc = fma(r.x, r.x, fma(r.y, r.y, facc));
     }
-    grad[node] += -om2 * acc;
+    grad[node] += -om2 * (layer ? w.x * acc + w.y * aim : acc);
   }
   const double2* q2 = (const double2*)b.r2;
   const int r0 = b.sys[G.sys0].rec_begin, r1 = b.sys[G.sys0 + G.nsys - 1].rec_end;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < r1 - r0; e += stride)
-    facc += 0.5 * abs2(q2[r0 + e]);
-  const double fs = block_sum<256>(facc, red);
+    facc += abs2(q2[r0 + e]);
+  const double fs = 0.5 * block_sum<256>(facc, red);
   if (threadIdx.x == 0 && fs != 0.0) atomicAdd(f, fs);
 }
 
@@ -285,23 +291,26 @@ __global__ void k_ir_cold(const __grid_constant__ Batch b, int nsys_total) {
     r2[k] = make_float2((float)lamd[k].x, (float)lamd[k].y);
 }
 
-// Forcing of an outer step: inner r1[0] = q64 - r64 (= f on the nodes) and inner receiver
-// residual r2_in = q2 - r2_64, both rounded to complex64.  q = b - S x64 comes from the FP64
+// Forcing of an outer step that goes on: inner r1[0] = q64 - r64 (= f on the nodes) and inner receiver
+// residual r2_in = q2 - r2_64, both rounded to complex64, and dx = 0.  q = b - S x64 comes from the FP64
 // residual kernel (q2: its receiver part).
 __global__ void k_ir_forcing(const __grid_constant__ Batch b, const double2* q2) {
   const long long stride = (long long)gridDim.x * blockDim.x;
-  for (int g = 0; g < b.ngroups; ++g) {
-    const GroupDev& G = b.g[g];
+  {
+    const GroupDev& G = b.g[blockIdx.y];
     const long long tot = (long long)G.nsys * G.n;
     const double2* q = (const double2*)G.q64;
     const double2* r64 = (const double2*)G.r64;
     float2* f = (float2*)G.r1[0];
+    float2* x32 = (float2*)G.x;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += stride) {
       if (b.sys[G.sys0 + (int)(e / G.n)].outer_done) continue;
       const double2 a = q[e], r = r64[e];
       f[e] = make_float2((float)(a.x - r.x), (float)(a.y - r.y));
+      x32[e] = make_float2(0.f, 0.f);
     }
   }
+  if (blockIdx.y > 0) return;
   const int ns = nsys_of(b);
   const double2* r2 = (const double2*)b.r2_64;
   float2* f2 = (float2*)b.r2_in;
@@ -312,57 +321,56 @@ __global__ void k_ir_forcing(const __grid_constant__ Batch b, const double2* q2)
   }
 }
 
-// Update after an inner solve: x64 += dx (then dx = 0), r64 += dr on the nodes (the inner
-// residual of the system's last iteration sits in r1[iter & 1]) and r2_64 += r2_in.
+// Update after an inner solve: x64 += dx, r64 += dr on the nodes (the inner residual of the system's last
+// iteration sits in r1[iter & 1]).  FIRST: x64 and r64 were zero and have not been written (cold start): the
+// pass writes them without reading, 48 bytes per node instead of 40 to zero them and 80 to update.
+template <bool FIRST>
 __global__ void k_ir_update(const __grid_constant__ Batch b) {
   const long long stride = (long long)gridDim.x * blockDim.x;
-  for (int g = 0; g < b.ngroups; ++g) {
-    const GroupDev& G = b.g[g];
-    const long long tot = (long long)G.nsys * G.n;
-    double2* x64 = (double2*)G.x64;
-    double2* r64 = (double2*)G.r64;
-    float2* x32 = (float2*)G.x;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += stride) {
-      const SysDev& sd = b.sys[G.sys0 + (int)(e / G.n)];
-      if (sd.outer_done) continue;
-      const float2 dx = x32[e];
-      const float2 dr = ((const float2*)G.r1[sd.iter & 1])[e];
-      double2 v = x64[e];
-      v.x += dx.x;
-      v.y += dx.y;
-      x64[e] = v;
-      x32[e] = make_float2(0.f, 0.f);
-      double2 r = r64[e];
-      r.x += dr.x;
-      r.y += dr.y;
-      r64[e] = r;
-    }
+  const GroupDev& G = b.g[blockIdx.y];
+  const long long tot = (long long)G.nsys * G.n;
+  double2* x64 = (double2*)G.x64;
+  double2* r64 = (double2*)G.r64;
+  const float2* x32 = (const float2*)G.x;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += stride) {
+    const SysDev& sd = b.sys[G.sys0 + (int)(e / G.n)];
+    if (!FIRST && sd.outer_done) continue;
+    const float2 dx = x32[e];
+    const float2 dr = ((const float2*)G.r1[sd.iter & 1])[e];
+    double2 v = FIRST ? make_double2(0.0, 0.0) : x64[e];
+    double2 r = FIRST ? make_double2(0.0, 0.0) : r64[e];
+    v.x += dx.x;
+    v.y += dx.y;
+    x64[e] = v;
+    r.x += dr.x;
+    r.y += dr.y;
+    r64[e] = r;
   }
-  const int ns = nsys_of(b);
+}
+
+// The same for the receiver part: r2_64 += r2_in, one block per system.
+__global__ void k_ir_update_rec(const __grid_constant__ Batch b, int nsys_total) {
+  const int s = blockIdx.x;
+  if (s >= nsys_total || b.sys[s].outer_done) return;
   double2* r2 = (double2*)b.r2_64;
   const float2* d2 = (const float2*)b.r2_in;
-  for (int s = blockIdx.x; s < ns; s += gridDim.x) {
-    if (b.sys[s].outer_done) continue;
-    for (int k = b.sys[s].rec_begin + threadIdx.x; k < b.sys[s].rec_end; k += blockDim.x) {
-      double2 r = r2[k];
-      r.x += d2[k].x;
-      r.y += d2[k].y;
-      r2[k] = r;
-    }
+  for (int k = b.sys[s].rec_begin + threadIdx.x; k < b.sys[s].rec_end; k += blockDim.x) {
+    double2 r = r2[k];
+    r.x += d2[k].x;
+    r.y += d2[k].y;
+    r2[k] = r;
   }
 }
 
 // u = x64 rounded to complex64.
 __global__ void k_ir_final(const __grid_constant__ Batch b, IrU U) {
   const long long stride = (long long)gridDim.x * blockDim.x;
-  for (int g = 0; g < b.ngroups; ++g) {
-    const GroupDev& G = b.g[g];
-    const long long tot = (long long)G.nsys * G.n;
-    const double2* x64 = (const double2*)G.x64;
-    float2* u = U.u[g];
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += stride)
-      u[e] = make_float2((float)x64[e].x, (float)x64[e].y);
-  }
+  const GroupDev& G = b.g[blockIdx.y];
+  const long long tot = (long long)G.nsys * G.n;
+  const double2* x64 = (const double2*)G.x64;
+  float2* u = U.u[blockIdx.y];
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += stride)
+    u[e] = make_float2((float)x64[e].x, (float)x64[e].y);
 }
 
 // alpha_out[s] = (A u_s)[src_s]; one thread per system.

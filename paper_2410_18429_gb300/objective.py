@@ -79,11 +79,13 @@ def _evaluate(m: torch.Tensor, prob: Problem, want_grad: bool):
     wide = dtype == wri.C64 and int(opts.max_refine) > 0
     for grp in prob.groups:
         step = min(prob.max_resident, grp.nsys)
-        u = torch.zeros(step, grp.n, dtype=cdt, device=dev)
-        u64 = torch.zeros(step, grp.n, dtype=torch.complex128, device=dev) if wide else None
+        # written whole by every cold-started solve; a warm start reads u
+        u = torch.empty(step, grp.n, dtype=cdt, device=dev)
+        u64 = torch.empty(step, grp.n, dtype=torch.complex128, device=dev) if wide else None
         for b, e in chunks(grp.nsys, prob.max_resident):
             spec = _sub(grp, b, e, mm, u[:e - b], None if u64 is None else u64[:e - b])
-            spec.u.zero_()
+            if int(opts.warm_start):
+                spec.u.zero_()
             work = torch.empty(wri.workspace_size([spec], opts), dtype=torch.uint8, device=dev)
             it, rr, st = wri.solve([spec], opts, workspace=work)
             if bool((st == wri.SYS_NONFINITE).any()):
