@@ -17,13 +17,15 @@ namespace wri {
 constexpr int kLayerTab = 12;
 constexpr int kXupdNodes = 4096;  // nodes of a work item of the iterate-update pass
 
-// z-chunk of the gradient kernel (its FP64 accumulator tile lives in shared memory)
-__host__ __device__ constexpr int grad_zc(int by) { return by >= 16 ? 8 : 16; }
+// z-chunk of the gradient kernel (its FP64 accumulator tile lives in shared memory: 16 KB at 8 rows, so that
+// registers and not shared memory decide how many CTAs an SM holds)
+__host__ __device__ constexpr int grad_zc(int by) { return by >= 16 ? 8 : 8; }
 
-// squared slowness at a node, in the precision of the caller's model array
+// squared slowness at a node, in the precision of the caller's model array (double only under FP64 stencils)
 template <typename R>
 __device__ __forceinline__ R model_at(const void* m, int m_double, long long node) {
-  return m_double ? R(((const double*)m)[node]) : R(((const float*)m)[node]);
+  if (sizeof(R) == 8 && m_double) return R(((const double*)m)[node]);
+  return R(((const float*)m)[node]);
 }
 
 // ------------------------------------------------------------------ complex helpers

@@ -106,7 +106,7 @@ __device__ __forceinline__ ZCoef<R> z_coef(const GroupDev& G, int k) {
 template <typename R>
 __device__ __forceinline__ cx<R> q_at(const GroupDev& G, int sl, long long node) {
   const long long e = (long long)sl * G.n + node;
-  if (G.q_double) return to_c(((const double2*)G.q)[e], R(0));
+  if (sizeof(R) == 8 && G.q_double) return to_c(((const double2*)G.q)[e], R(0));
   return to_c(((const float2*)G.q)[e], R(0));
 }
 

@@ -212,9 +212,36 @@ __device__ void finalize(const Batch& b, const GroupDev& G, SysDev* sd, int sl, 
   }
 }
 
+// Not inlined: predicated off beside the common path, the conversion would still take its slots.
+static __device__ __noinline__ double widen_cvt(float v) { return (double)v; }
+
+// float to double, exactly, by rebiasing the exponent in integer arithmetic: a conversion instruction runs on
+// the narrow FP64 pipe.  Zeros too; subnormals, infinities and NaN take the instruction.
+__device__ __forceinline__ double widen(float v) {
+  const uint32_t b = __float_as_uint(v), a = b & 0x7fffffffu;
+  if (a - 0x00800000u >= 0x7f000000u && a != 0u) return widen_cvt(v);
+  const uint32_t hi = (a >> 3) + (a ? 0x38000000u : 0u);
+  return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double v) { return v; }
+
+// Re(conj(a) b), its rounding spelled out: the gradient must not depend on how an instantiation contracts it.
+__device__ __forceinline__ float re_dot(float2 a, float2 b) { return __fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)); }
+__device__ __forceinline__ double re_dot(double2 a, double2 b) { return __fma_rn(a.x, b.x, __dmul_rn(a.y, b.y)); }
+
 // ------------------------------------------------------------------ the kernel
+// CTAs per SM the register allocation aims at: three of 256 threads for the complex64 gradient, else left to the
+// compiler.  That gradient was bound by exposed loads (the halo ring of plane k + 1 was read between two
+// barriers), by 304 CTAs holding 16-plane sums, and by six FP64-pipe instructions per node, four of them
+// conversions: 116^3 x 32 in 1657 us; ring read a plane ahead 1286, 8-plane sums 951, three CTAs 803, conversions
+// in integer arithmetic 670 (7- and 10-plane sums 930).
+template <typename R, int MODE, int BY>
+constexpr int march_min_ctas() {
+  return MODE == M_GRAD && sizeof(R) == 4 && BY == 8 ? 3 : 1;
+}
+
 template <typename R, typename OR, int MODE, bool CONJ, int BY>
-__global__ void __launch_bounds__(WRI_TX * BY) k_march(const __grid_constant__ Batch b) {
+__global__ void __launch_bounds__(WRI_TX * BY, march_min_ctas<R, MODE, BY>()) k_march(const __grid_constant__ Batch b) {
   typedef cx<R> C;
   typedef cx<OR> OC;
   constexpr int NT = WRI_TX * BY;
@@ -340,8 +367,10 @@ __global__ void __launch_bounds__(WRI_TX * BY) k_march(const __grid_constant__ B
           coef = -R(sd->alpha);
           Fst = (C*)G.r1[cur ^ 1] + off;
         }
-        C a_src = czero<R>();
-        if ((MODE == M_RES || MODE == M_GRAD) && G.alpha) a_src = mkc(R(G.alpha[2 * sl]), R(G.alpha[2 * sl + 1]));
+        // the source's weight, read where it is used (its conversions run on the FP64 pipe)
+        auto a_src = [&]() -> C {
+          return G.alpha ? mkc(R(G.alpha[2 * sl]), R(G.alpha[2 * sl + 1])) : czero<R>();
+        };
 
         // F at any node (no side effects)
         auto fieldF = [&](long long node) -> C {
@@ -378,15 +407,13 @@ __global__ void __launch_bounds__(WRI_TX * BY) k_march(const __grid_constant__ B
           else if (e < 2 * WRI_TX + BY) { rx = x0 - 1; ry = y0 + e - 2 * WRI_TX; si = 0; sj = ry - y0 + 1; }
           else { rx = x0 + WRI_TX; ry = y0 + e - 2 * WRI_TX - BY; si = WRI_TX + 1; sj = ry - y0 + 1; }
         };
-        auto load_ring = [&](int kk, int slot) {
-          for (int e = tid; e < RING; e += NT) {
-            int rx, ry, si, sj;
-            ring_node(e, rx, ry, si, sj);
-            C v = czero<R>();
-            if (kk >= 0 && kk < nz && rx >= 0 && rx < nx && ry >= 0 && ry < ny)
-              v = fieldF(kk * plane + (long long)ry * nx + rx);
-            buf[slot][sj][si] = v;
-          }
+        // the thread's element of the halo ring (one at most), if any, and its value at a plane
+        static_assert(RING <= NT, "one ring element per thread");
+        int rx = 0, ry = 0, rsi = 0, rsj = 0;
+        if (tid < RING) ring_node(tid, rx, ry, rsi, rsj);
+        const bool ring_in = tid < RING && rx >= 0 && rx < nx && ry >= 0 && ry < ny;
+        auto ring_value = [&](int kk) -> C {
+          return ring_in && kk >= 0 && kk < nz ? fieldF(kk * plane + (long long)ry * nx + rx) : czero<R>();
         };
 
         // ---- prologue
@@ -395,7 +422,7 @@ __global__ void __launch_bounds__(WRI_TX * BY) k_march(const __grid_constant__ B
         C Fc = ownF(z0);
         C Fp = (z0 + 1 <= z1) ? ownF(z0 + 1) : czero<R>();
         buf[0][ty + 1][tx + 1] = Fc;
-        load_ring(z0, 0);
+        if (tid < RING) buf[0][rsj][rsi] = ring_value(z0);
         float accf = 0.f;
 
         for (int k = z0; k < z1; ++k) {
@@ -403,6 +430,7 @@ __global__ void __launch_bounds__(WRI_TX * BY) k_march(const __grid_constant__ B
           __syncthreads();
           // issue the loads of the next planes early
           const C Fn = (k + 2 <= z1) ? ownF(k + 2) : czero<R>();
+          const C Rn = (k + 1 < z1) ? ring_value(k + 1) : czero<R>();
           // stencil at (i, j, k)
           const C u = Fc;
           const C uxm = buf[cb][ty + 1][tx];
@@ -442,7 +470,7 @@ __global__ void __launch_bounds__(WRI_TX * BY) k_march(const __grid_constant__ B
             } else if (MODE == M_RES) {
               C r = czero<R>() - AF;
               if (G.q) r = q_at<R>(G, sl, node) - AF;
-              else if (node == src) r = G.masked ? czero<R>() : a_src - AF;
+              else if (node == src) r = G.masked ? czero<R>() : a_src() - AF;
               ((C*)G.r1[0])[gnode] = r;
             } else if (MODE == M_P1) {
               const C t = (G.masked && node == src) ? czero<R>() : AF;
@@ -461,29 +489,29 @@ __global__ void __launch_bounds__(WRI_TX * BY) k_march(const __grid_constant__ B
             } else if (MODE == M_GRAD) {
               C r = AF;
               if (G.q) r = r - q_at<R>(G, sl, node);
-              else if (node == src) r = r - a_src;
+              else if (node == src) r = r - a_src();
               if (fast) {
-                gacc[k - z0][ty][tx] += (double)(om2 * (u.x * r.x + u.y * r.y));
+                gacc[k - z0][ty][tx] += widen(om2 * re_dot(u, r));
               } else {
                 const C w = cxy.sxy * zc.sz;
                 const C wu = w * u;
-                gacc[k - z0][ty][tx] += (double)(om2 * (wu.x * r.x + wu.y * r.y));
+                gacc[k - z0][ty][tx] += widen(om2 * re_dot(wu, r));
               }
-              facc += 0.5 * (double)abs2(r);
+              facc += 0.5 * widen(abs2(r));
             }
           }
-          if (sizeof(R) == 4 && ((k - z0) & 7) == 7) {
+          if (MODE != M_GRAD && sizeof(R) == 4 && ((k - z0) & 7) == 7) {
             accd += (double)accf;
             accf = 0.f;
           }
           // next plane into the other buffer
           buf[cb ^ 1][ty + 1][tx + 1] = Fp;
-          if (k + 1 < z1) load_ring(k + 1, cb ^ 1);
+          if (k + 1 < z1 && tid < RING) buf[cb ^ 1][rsj][rsi] = Rn;
           Fm = Fc;
           Fc = Fp;
           Fp = Fn;
         }
-        accd += (double)accf;
+        if (MODE != M_GRAD) accd += (double)accf;
       }  // systems (gradient) / single system
 
       if (MODE == M_GRAD) {

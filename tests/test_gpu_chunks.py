@@ -136,3 +136,33 @@ def test_one_systems_nan_stays_its_own(W):
     assert st[1] == W.SYS_NONFINITE and st[0] == st[2] == W.SYS_MAXITER
     for s in (0, 2):
         assert np.array_equal(spec.u[s].cpu().numpy(), clean.u[s].cpu().numpy())
+
+
+def test_complex64_gradient_scales_exactly_and_keeps_nan_at_its_nodes(W):
+    """The complex64 gradient widens its float terms in integer arithmetic: scaling u by 2^-30 scales every
+    term, so the gradient, by exactly 2^-60; a NaN (which takes the conversion instruction, as subnormals and
+    infinities do) stays at its node's and its neighbours' terms."""
+    from paper_2410_18429_gb300.problem import to_device
+    G = _case(((37, 23, 19), 5), "free")
+    G.d[:] = 0
+    n = G.spec.n
+    u0 = (synth.random_complex((3, n), 41) * 1e-3).astype(np.complex64)
+
+    def grad(scale, bad=None):
+        u = (u0 * np.float32(scale)).astype(np.complex64)
+        if bad is not None:
+            u[1, bad] = np.nan
+        spec = to_device(G, 0, "cuda", u=u)
+        a = torch.zeros(3, dtype=torch.complex128, device="cuda")
+        (g,), _ = W.gradient([spec], 0, a)
+        return g.cpu().numpy().ravel()
+
+    g1 = grad(1.0)
+    assert np.array_equal(grad(2.0 ** -30), g1 * 2.0 ** -60)
+    bad = n // 2 + 5
+    gn = grad(1.0, bad)
+    nx, pl = G.spec.nx, G.spec.nx * G.spec.ny
+    touched = {bad, bad - 1, bad + 1, bad - nx, bad + nx, bad - pl, bad + pl}
+    assert set(np.flatnonzero(np.isnan(gn))) == touched
+    keep = np.setdiff1d(np.arange(n), sorted(touched))
+    assert np.array_equal(gn[keep], g1[keep])
