@@ -418,7 +418,8 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
     constexpr int NY = PAIR ? 1 : NPT;  // rows of the thread's nodes (a pair lies in one row)
     C am[NPT], ap[NPT], bm[NY], bp[NY], cc[NPT];
     R sx_[NPT], sy_[NY];
-    R cc0[NPT];  // Re cc with the z axis unstretched
+    R cc0[NPT];   // Re cc with the z axis unstretched
+    R w2xy[NPT];  // gradient: |s_x s_y|^2
 
     double accd = 0.0;
     // sum of |output|^2: FP32 over 4 planes, then FP64 (pairs past the chunk's end are left out at the end)
@@ -473,19 +474,31 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         }
       }
     };
-    // gradient: residual of the finished stencil t of plane kp, accumulated over the systems
+    // gradient: the finished plane kp, accumulated over the systems.  t is the stencil without the node factor
+    // w = s_x s_y s_z, which leaves the sums: with A u - c = w t', t' = t - c / w,
+    //   Re(conj(w u) w t') = |w|^2 Re(conj(u) t'),  |w t'|^2 = |w|^2 |t'|^2,
+    // and |w|^2 enters the gradient once, after the last system (9 to 12 FP64 instructions less per node and
+    // system in the layer: 148^3 x 16 3.82 -> 2.99 ms).
     auto accum = [&](int kp, C (&t)[NPT], bool g, bool z) {
 #pragma unroll
       for (int r = 0; r < NPT; ++r) {
         if (!own[r]) continue;
-        C rr = t[r];
-        if (G.q) rr = rr - q_at<R>(G, sl, (long long)kp * plane + e0 + r * RS);
-        else if (kp == src_k && r == src_r) rr = rr - a_src;
-        C u = fc[r];
-        if (g) u = smul(sy_[PAIR ? 0 : r], smul(sx_[r], u));
-        if (z) u = smul(hs, u);
-        gacc[(kp - z0) * L + tid + r * NC] += (double)(om2 * (u.x * rr.x + u.y * rr.y));
-        accd += 0.5 * (double)abs2(rr);
+        if (G.q || (kp == src_k && r == src_r)) {
+          const C c = G.q ? q_at<R>(G, sl, (long long)kp * plane + e0 + r * RS) : a_src;
+          C w = mkc(R(1), g ? sx_[r] : R(0));
+          if (g) w = smul(sy_[r], w);
+          if (z) w = smul(hs, w);
+          const R d = R(1) / abs2(w);
+          t[r] = t[r] - mkc((c.x * w.x + c.y * w.y) * d, (c.y * w.x - c.x * w.y) * d);
+        }
+        double* ga = gacc + (kp - z0) * L + tid + r * NC;
+        *ga = fma_r(fc[r].x, t[r].x, fma_r(fc[r].y, t[r].y, *ga));
+        if (g || z) {
+          const R w2 = (g ? w2xy[r] : R(1)) * (z ? fma_r(hs, hs, R(1)) : R(1));
+          accd = fma_r(w2, fma_r(t[r].x, t[r].x, t[r].y * t[r].y), accd);
+        } else {
+          accd = fma_r(t[r].x, t[r].x, fma_r(t[r].y, t[r].y, accd));
+        }
       }
     };
     // the finished stencil t of plane kp: mask, right-hand side, store, norm
@@ -578,6 +591,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         }
         cc[r] = cx_.a0 + cy_.a0;
         cc0[r] = cc[r].x - R(2) * ih2;
+        w2xy[r] = fma_r(cx_.im, cx_.im, R(1)) * fma_r(cy_.im, cy_.im, R(1));
         sx_[r] = cx_.im;
       }
     }
@@ -651,7 +665,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         for (int r = 0; r < NPT; ++r) {
           const C d = DIFF ? v[r] - fc[r] : v[r];
           t[r] = ZG ? cfma(hz, d, q[r]) : rfma(ih2, d, q[r]);
-          if (GEN) t[r] = smul(sy_[PAIR ? 0 : r], smul(sx_[r], t[r]));
+          if (GEN && !GRAD) t[r] = smul(sy_[PAIR ? 0 : r], smul(sx_[r], t[r]));
         }
         if constexpr (GRAD) {
           accum(k - 1, t, GEN, ZG);
@@ -662,7 +676,10 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
       AxisCoef<R> cz;
       if (ZG) {
         cz = axis_coef<R, CONJ>(tab, k, nz, npml, ih2, &hz);
-        if (GRAD) hs = cz.im;
+        if (GRAD) {
+          hz = cz.ap;
+          hs = cz.im;
+        }
       }
 #pragma unroll
       for (int r = 0; r < NPT; ++r) {
@@ -710,7 +727,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
           acc = rfma(ih2, sum, acc);
           if (ZG) acc = cfma(cz.am, zm, acc);
         }
-        q[r] = ZG ? smul(cz.im, acc) : acc;
+        q[r] = ZG && !GRAD ? smul(cz.im, acc) : acc;
         fc[r] = v[r];
       }
       if (DUMMY && k == z0) {  // what this step finished was no plane of the item
@@ -791,7 +808,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
 #pragma unroll
           for (int r = 0; r < NPT; ++r) {
             t[r] = cfma(hz, DIFF ? v[r] - fc[r] : v[r], q[r]);
-            if (gen) t[r] = smul(sy_[PAIR ? 0 : r], smul(sx_[r], t[r]));
+            if (gen && !GRAD) t[r] = smul(sy_[PAIR ? 0 : r], smul(sx_[r], t[r]));
           }
           if constexpr (GRAD) accum(z1 - 1, t, gen, true);
           else emit(z1 - 1, t);
@@ -818,11 +835,15 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         if (tid == 0) atomicAdd(b.f, (double)NAN);
         break;
       }
-      for (int k = z0; k < z1; ++k)
+      for (int k = z0; k < z1; ++k) {
+        const R im = axis_coef<R, false>(tab, k, nz, npml, ih2).im;
+        const R w2z = om2 * fma_r(im, im, R(1));
 #pragma unroll
         for (int r = 0; r < NPT; ++r)
-          if (own[r]) G.grad[(long long)k * plane + e0 + r * RS] += gacc[(k - z0) * L + tid + r * NC];
-      if (tid == 0 && tsum != 0.0) atomicAdd(b.f, tsum);
+          if (own[r])
+            G.grad[(long long)k * plane + e0 + r * RS] += (gen ? w2xy[r] : R(1)) * w2z * gacc[(k - z0) * L + tid + r * NC];
+      }
+      if (tid == 0 && tsum != 0.0) atomicAdd(b.f, 0.5 * tsum);
       continue;
     }
     // the copy warp may raise the flag at any time: decide on one reduced value
