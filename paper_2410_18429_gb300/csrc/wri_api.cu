@@ -17,7 +17,6 @@
 
 #include "../../include/wri.h"
 #include "wri_launch.h"
-#include "wri_lin.cuh"
 #include "wri_tma.cuh"
 
 using namespace wri;
@@ -271,6 +270,8 @@ struct Plan {
   size_t off_sys = 0, off_rec = 0, off_part = 0, off_rem = 0, off_lamd = 0, off_r2 = 0;
   size_t off_r2_64 = 0, off_r2_in = 0;  // refinement: FP64 receiver residual master, complex64 inner r2
   size_t off_ltab32[WRI_MAXG], off_ltab64[WRI_MAXG];  // layer tables of the chunk kernels
+  size_t zero_total = 0;  // bytes from off_rem that a solve starts with zeroed
+  size_t up_total = 0;  // bytes the host uploads: systems, receivers, layer tables
   size_t aux_base = 0, aux_total = 0, total = 0;  // aux_base: without the layer tables
   GroupDev g[WRI_MAXG];
   size_t v_r1[WRI_MAXG][2], v_p[WRI_MAXG][4], v_s[WRI_MAXG], v_t1[WRI_MAXG];
@@ -296,20 +297,22 @@ void plan_aux(const wri_group* groups, int ngroups, Plan& P) {
   off += align_up(sizeof(SysDev) * (size_t)P.nsys_total);
   P.off_rec = off;
   off += align_up(sizeof(int) * (size_t)std::max(P.nnz_total, 1));
-  for (int gi = 0; gi < ngroups; ++gi) {  // [2][nz][3] complex coefficients in FP32 and FP64
-    P.off_ztab[gi] = off;
-    off += align_up(sizeof(float) * 2 * 2 * 3 * (size_t)groups[gi].grid.nz);
-    P.off_ztab64[gi] = off;
-    off += align_up(sizeof(double) * 2 * 2 * 3 * (size_t)groups[gi].grid.nz);
-  }
-  P.aux_base = off;
-  for (int gi = 0; gi < ngroups; ++gi) {  // layer tables of the chunk kernels
+  const size_t tabs = off;
+  for (int gi = 0; gi < ngroups; ++gi) {  // layer tables of the chunk kernels (one upload with the above)
     const size_t e = (size_t)kLayerTab * (groups[gi].grid.npml + 1);
     P.off_ltab32[gi] = off;
     off += align_up(sizeof(float) * e);
     P.off_ltab64[gi] = off;
     off += align_up(sizeof(double) * e);
   }
+  P.up_total = off;
+  for (int gi = 0; gi < ngroups; ++gi) {  // [2][nz][3] complex coefficients in FP32 and FP64
+    P.off_ztab[gi] = off;
+    off += align_up(sizeof(float) * 2 * 2 * 3 * (size_t)groups[gi].grid.nz);
+    P.off_ztab64[gi] = off;
+    off += align_up(sizeof(double) * 2 * 2 * 3 * (size_t)groups[gi].grid.nz);
+  }
+  P.aux_base = off - (P.up_total - tabs);
   P.aux_total = off;
   P.total = off;
 }
@@ -434,8 +437,6 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
   size_t off = P.total;
   P.off_part = off;
   off += align_up(sizeof(double) * (size_t)std::max<long long>(parts, 4096));
-  P.off_rem = off;
-  off += kAlign;
   P.off_lamd = off;
   off += align_up((size_t)P.rlbytes * std::max(P.nnz_total, 1));
   P.off_r2 = off;
@@ -447,7 +448,9 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
     P.off_r2_in = off;
     off += align_up(8 * (size_t)std::max(P.nnz_total, 1));
   }
-  for (int gi = 0; gi < ngroups; ++gi) {  // receiver bitmaps (one bit per node and system)
+  P.off_rem = off;  // counters, and next to them the receiver bitmaps (one bit per node and system): one memset
+  off += kAlign;
+  for (int gi = 0; gi < ngroups; ++gi) {
     const GroupDev& G = P.g[gi];
     P.rcol_bytes[gi] = 4 * (size_t)G.nsys * G.ny * G.rw;
     P.rmask_bytes[gi] = G.zw ? 4 * (size_t)G.nsys * G.nx * G.ny * G.zw : P.rcol_bytes[gi] * (size_t)G.nz;
@@ -456,6 +459,7 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
     P.off_rmask[gi] = off;
     off += align_up(P.rmask_bytes[gi]);
   }
+  P.zero_total = off - P.off_rem;
   for (int gi = 0; gi < ngroups; ++gi) {
     const size_t vb = align_up((size_t)P.vbytes * (size_t)P.g[gi].nsys * (size_t)P.g[gi].n);
     P.v_r1[gi][0] = off; off += vb;
@@ -695,13 +699,11 @@ Batch solver_batch(const wri_group* groups, const Plan& P, char* ws, bool inner_
   return b;
 }
 
-// Receiver bitmaps of every group (the normal-residual norms leave receiver nodes to the finalizer)
-int setup_rmask(const Plan& P, const Batch& b, char* ws, cudaStream_t st) {
-  for (int gi = 0; gi < P.ngroups; ++gi) {
-    WRI_CK(cudaMemsetAsync(ws + P.off_rcol[gi], 0, P.rcol_bytes[gi], st));
-    WRI_CK(cudaMemsetAsync(ws + P.off_rmask[gi], 0, P.rmask_bytes[gi], st));
-  }
-  WRI_CK(launch_rmask(b, P.nsys_total, st));
+// Zeroed counters and bitmaps, then lambda d, the receiver residual, the receiver bitmaps (the normal-residual
+// norms leave receiver nodes to the finalizer) and the refinement's receiver map of every system.
+int setup_systems(const Plan& P, const Batch& b, int dbytes, int rlbytes, char* ws, cudaStream_t st) {
+  WRI_CK(cudaMemsetAsync(ws + P.off_rem, 0, P.zero_total, st));
+  WRI_CK(launch_setup_rhs(dbytes, rlbytes, b, P.nsys_total, st));
   return WRI_OK;
 }
 
@@ -712,19 +714,29 @@ int lin_rhs(const Plan& P, const Batch& b, int rbytes, int obytes, const LinWait
   const bool init = b.flavor == SH_INIT;
   bool field = false;
   for (int gi = 0; gi < P.ngroups; ++gi) field = field || b.g[gi].q;
-  for (int gi = 0; gi < P.ngroups; ++gi) {
+  if (init) {  // x = 0; r1 = 0 and s = 0 where they are not written whole below
+    ZeroSet z;
+    z.count = 0;
+    for (int gi = 0; gi < P.ngroups; ++gi) {
+      const GroupDev& G = b.g[gi];
+      const long long cnt = 2LL * G.nsys * G.n;
+      z.add(G.x, rbytes * cnt);
+      if (!G.q) z.add(G.r1[0], rbytes * cnt);
+      if (!field) z.add(G.s, obytes * cnt);
+    }
+    WRI_CK(launch_zero(z, st));
+  }
+  for (int gi = 0; gi < P.ngroups && field; ++gi) {
     const GroupDev& G = b.g[gi];
     const size_t cnt = (size_t)G.nsys * (size_t)G.n;
-    if (init) WRI_CK(cudaMemsetAsync(G.x, 0, 2 * rbytes * cnt, st));
     if (G.q && rbytes == 8 && !G.q_double) {
       WRI_CK(launch_widen(G.q, G.r1[0], (long long)cnt, st));
     } else if (G.q) {
       WRI_CK(cudaMemcpyAsync(G.r1[0], G.q, 2 * rbytes * cnt, cudaMemcpyDeviceToDevice, st));
-    } else if (init || field) {
-      WRI_CK(cudaMemsetAsync(G.r1[0], 0, 2 * rbytes * cnt, st));
-      if (field && G.alpha) WRI_CK(launch_point_field(rbytes, b, gi, st));
+    } else {
+      if (!init) WRI_CK(cudaMemsetAsync(G.r1[0], 0, 2 * rbytes * cnt, st));
+      if (G.alpha) WRI_CK(launch_point_field(rbytes, b, gi, st));
     }
-    if (init && !field) WRI_CK(cudaMemsetAsync(G.s, 0, 2 * obytes * cnt, st));
   }
   if (field) WRI_CK(launch_lin(rbytes, obytes, M_SH, true, b, w, nullptr, 0, st));
   else WRI_CK(launch_init_point(rbytes, obytes, b, P.nsys_total, st));
@@ -930,7 +942,6 @@ int run_loop(const Plan& P, const Batch& b1_in, const Batch& b2_in, int mode2, i
     }
   }
   if (dev_loop) {
-    WRI_CK(cudaMemsetAsync(b1.remaining + 2, 0, sizeof(int), st));
     WRI_CK(cudaGraphLaunch(exec.get(), st));
     WRI_CK(cudaMemcpyAsync(slot, b1.remaining, 3 * sizeof(int), cudaMemcpyDeviceToHost, st));
     WRI_CK(cudaStreamSynchronize(st));
@@ -955,19 +966,19 @@ int upload(const wri_group* groups, int ngroups, const Plan& P, char* ws, cudaSt
   std::vector<SysDev> sys;
   std::vector<int> rec;
   build_sys(groups, ngroups, P, sys, rec);
-  WRI_CK(cudaMemcpyAsync(ws + P.off_sys, sys.data(), sizeof(SysDev) * sys.size(), cudaMemcpyHostToDevice, st));
-  WRI_CK(cudaMemcpyAsync(ws + P.off_rec, rec.data(), sizeof(int) * rec.size(), cudaMemcpyHostToDevice, st));
-  if (P.lin) {  // one copy: the tables of all groups are neighbours
-    std::vector<char> tabs(P.aux_total - P.off_ltab32[0]);
+  std::vector<char> up(P.lin ? P.up_total : P.off_rec + sizeof(int) * rec.size());  // one copy
+  std::memcpy(up.data() + P.off_sys, sys.data(), sizeof(SysDev) * sys.size());
+  std::memcpy(up.data() + P.off_rec, rec.data(), sizeof(int) * rec.size());
+  if (P.lin) {
     std::vector<double> t;
     for (int gi = 0; gi < ngroups; ++gi) {
       layer_table(groups[gi].grid, t);
-      char* p32 = tabs.data() + (P.off_ltab32[gi] - P.off_ltab32[0]);
-      for (size_t i = 0; i < t.size(); ++i) ((float*)p32)[i] = (float)t[i];
-      std::memcpy(tabs.data() + (P.off_ltab64[gi] - P.off_ltab32[0]), t.data(), sizeof(double) * t.size());
+      float* p32 = (float*)(up.data() + P.off_ltab32[gi]);
+      for (size_t i = 0; i < t.size(); ++i) p32[i] = (float)t[i];
+      std::memcpy(up.data() + P.off_ltab64[gi], t.data(), sizeof(double) * t.size());
     }
-    WRI_CK(cudaMemcpyAsync(ws + P.off_ltab32[0], tabs.data(), tabs.size(), cudaMemcpyHostToDevice, st));
   }
+  WRI_CK(cudaMemcpyAsync(ws + P.off_sys, up.data(), up.size(), cudaMemcpyHostToDevice, st));
   return WRI_OK;
 }
 
@@ -1005,10 +1016,8 @@ int solve_fused(const wri_group* groups, int ngroups, const wri_solve_opts* o, c
   const LinWait w = lin_wait(b, o);
   b.order = order_of(o);
   b.sblock = sblock_of(o);
-  if (setup_rmask(P, b, ws, st) != WRI_OK) return WRI_ECUDA;
+  if (setup_systems(P, b, o->dtype == WRI_C128 ? 8 : 4, vb, ws, st) != WRI_OK) return WRI_ECUDA;
   if (!P.lin) WRI_CK(launch_ztable(b, st));
-  WRI_CK(launch_setup_rhs(o->dtype == WRI_C128 ? 8 : 4, vb, b, P.nsys_total, st));
-  WRI_CK(cudaMemsetAsync(b.remaining, 0, 3 * sizeof(int), st));
   Batch r = b;
   r.flavor = o->warm_start ? SH_REF : SH_INIT;
   if (P.lin) {
@@ -1058,7 +1067,6 @@ int solve_refined(const wri_group* groups, int ngroups, const wri_solve_opts* o,
     if (!P.lin)
       WRI_CK(cudaMemsetAsync(ws + P.v_rmap[gi], 0xff, 4 * (size_t)P.g[gi].nsys * (size_t)P.g[gi].n, st));
   }
-  WRI_CK(launch_ir_rmap(outer, P.nsys_total, st));
   outer.max_iter = o->max_iter;
   outer.tol = o->tol;
   outer.refine_tol = o->refine_tol;
@@ -1068,12 +1076,11 @@ int solve_refined(const wri_group* groups, int ngroups, const wri_solve_opts* o,
   // complex64 views: x = dx, r2 = r2_in, gvec = g'
   Batch inner = solver_batch(groups, P, ws, true);
   inner.max_iter = o->max_iter;
-  if (setup_rmask(P, inner, ws, st) != WRI_OK) return WRI_ECUDA;
   if (!P.lin) WRI_CK(launch_ztable(inner, st));  // the outer view shares the tables
   void* u[WRI_MAXG] = {};
   for (int gi = 0; gi < P.ngroups; ++gi) u[gi] = groups[gi].u;
   // lambda d in FP64 (lamd and q2)
-  WRI_CK(launch_setup_rhs(4, 8, outer, P.nsys_total, st));
+  if (setup_systems(P, outer, 4, 8, ws, st) != WRI_OK) return WRI_ECUDA;
   if (o->warm_start) {  // x64 = u, r64 = 0, dx = 0; ||S^H b|| with the FP64 stencil (q2 still holds lambda d)
     WRI_CK(launch_ir_init(inner, u, 1, st));
     Batch r = outer;
@@ -1108,7 +1115,6 @@ int solve_refined(const wri_group* groups, int ngroups, const wri_solve_opts* o,
     // FP64 pass.  The first inner solve starts like an unrefined solve, from r = b (the point field
     // b1 and lambda d) and s = S^H b formed in FP32; ||S^H b|| is the reference of every outer test.
     WRI_CK(launch_ir_cold(inner, P.nsys_total, st));               // r2_in = lambda d (complex64)
-    WRI_CK(cudaMemsetAsync(inner.remaining, 0, 3 * sizeof(int), st));
     Batch r = inner;
     r.flavor = SH_INIT;
     r.tol = std::max(o->inner_tol, 0.95 * o->refine_tol);

@@ -15,17 +15,15 @@ cudaError_t launch_march_f64(int mode, bool conj, int by, const Batch& b, int gr
 cudaError_t launch_march_f64_to_f32(int mode, int by, const Batch& b, int grid, cudaStream_t st);
 
 // small kernels (wri_small.cu)
+// lambda d, receiver residual, receiver bitmaps (zeroed before) and, where b has one, receiver map
 cudaError_t launch_setup_rhs(int dtype_bytes, int rl_bytes, const Batch& b, int nsys_total, cudaStream_t st);
 cudaError_t launch_ztable(const Batch& b, cudaStream_t st);
-// receiver bitmaps of every group (b: solver view with rmask / rcol set and zeroed)
-cudaError_t launch_rmask(const Batch& b, int nsys_total, cudaStream_t st);
 // control kernel of the device-side CG loop (one thread; sets the WHILE node's condition)
 cudaError_t launch_loop_ctl(cudaGraphConditionalHandle h, int* counters, int cap, cudaStream_t st);
 cudaError_t launch_export(const SysDev* sys, int nsys, int32_t* iters, double* relres, int32_t* status,
                           cudaStream_t st);
 // FP64 refinement (b: inner complex64 view; u: the caller's wavefields, one per group)
 cudaError_t launch_ir_init(const Batch& b, void* const* u, int warm, cudaStream_t st);
-cudaError_t launch_ir_rmap(const Batch& b, int nsys_total, cudaStream_t st);  // b: outer view, map filled with -1
 cudaError_t launch_ir_cold(const Batch& b, int nsys_total, cudaStream_t st);  // b: inner view
 cudaError_t launch_ir_forcing(const Batch& b, const void* q2, cudaStream_t st);
 cudaError_t launch_ir_update(const Batch& b, bool first, cudaStream_t st);  // first: x64 = dx, r64 = dr
@@ -67,6 +65,7 @@ cudaError_t launch_phase_tma(int mode, int cfg, const Batch& b, const TmaSet& T,
 
 // Chunk kernels (wri_lin.cu): stencil passes over linear chunks of the x-y plane.
 constexpr int kLinChunk = 256;  // nodes of a chunk, at most
+constexpr int kLinInlineTab = 33;  // entries of the layer table that travels with the arguments (M_APPLY)
 constexpr int kLinStages = 3;
 constexpr int kLinMaxSmem = 220 * 1024;
 struct LinWait {  // bounded waits of the copy pipelines (TmaSet)
@@ -80,6 +79,17 @@ cudaError_t launch_lin(int rbytes, int obytes, int mode, bool conj, const Batch&
                        const double* tab, int tab_n, cudaStream_t st);
 // s = S^H b of point right-hand sides (flavors SH_INIT, SH_REF) without a pass over the grid
 cudaError_t launch_init_point(int rbytes, int obytes, const Batch& b, int nsys_total, cudaStream_t st);
+// zero several device arrays (8-byte aligned, whole multiples of 8 bytes) in one launch
+struct ZeroSet {
+  void* p[3 * WRI_MAXG];
+  long long bytes[3 * WRI_MAXG];
+  int count;
+  void add(void* q, long long n) {
+    p[count] = q;
+    bytes[count++] = n;
+  }
+};
+cudaError_t launch_zero(const ZeroSet& z, cudaStream_t st);
 cudaError_t launch_point_field(int rbytes, const Batch& b, int gi, cudaStream_t st);  // r1[src] = alpha
 // x += the steps of the last b.xsteps iterations; closes systems that have stopped
 cudaError_t launch_xupdate(int rbytes, const Batch& b, cudaStream_t st);

@@ -114,6 +114,26 @@ cudaError_t launch_init_point(int rbytes, int obytes, const Batch& b, int nsys_t
   return cudaGetLastError();
 }
 
+// One array per blockIdx.y, zeroed in 16-byte stores (8-byte ones at an unaligned start and the end).
+__global__ void k_zero(const __grid_constant__ ZeroSet z) {
+  unsigned char* p = (unsigned char*)z.p[blockIdx.y];
+  const long long bytes = z.bytes[blockIdx.y];
+  const long long head = ((uintptr_t)p & 15) ? 8 : 0, mid = (bytes - head) / 16;
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+  for (long long e = t; e < mid; e += step) *(uint4*)(p + head + 16 * e) = make_uint4(0u, 0u, 0u, 0u);
+  if (t == 0 && head) *(uint2*)p = make_uint2(0u, 0u);
+  if (t == 0 && head + 16 * mid < bytes) *(uint2*)(p + head + 16 * mid) = make_uint2(0u, 0u);
+}
+
+cudaError_t launch_zero(const ZeroSet& z, cudaStream_t st) {
+  long long most = 0;
+  for (int i = 0; i < z.count; ++i) most = z.bytes[i] > most ? z.bytes[i] : most;
+  if (most <= 0) return cudaSuccess;
+  const long long blocks = (most / 16 + 1023) / 1024;  // 4 x 256 16-byte stores per block
+  k_zero<<<dim3((unsigned)(blocks < 1 ? 1 : blocks < 152 * 8 ? blocks : 152 * 8), z.count), 256, 0, st>>>(z);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_point_field(int rbytes, const Batch& b, int gi, cudaStream_t st) {
   const int grid = (b.g[gi].nsys + 127) / 128;
   if (rbytes == 8) k_point_field<double><<<grid, 128, 0, st>>>(b, gi);

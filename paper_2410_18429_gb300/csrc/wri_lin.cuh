@@ -48,8 +48,6 @@
 
 namespace wri {
 
-constexpr int kLinInlineTab = 33;  // entries of the table that travels with the kernel arguments (APPLY)
-
 struct LinSet {
   int* err;                    // set to 1 by a CTA whose copy wait timed out
   unsigned long long wait_ns;  // time limit of every wait (global timer, ns)

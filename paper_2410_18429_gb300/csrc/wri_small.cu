@@ -23,12 +23,6 @@ cudaError_t launch_setup_rhs(int dtype_bytes, int rl_bytes, const Batch& b, int 
   return cudaGetLastError();
 }
 
-cudaError_t launch_rmask(const Batch& b, int nsys_total, cudaStream_t st) {
-  if (nsys_total <= 0) return cudaSuccess;
-  k_rmask<<<nsys_total, 128, 0, st>>>(b, nsys_total);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_loop_ctl(cudaGraphConditionalHandle h, int* counters, int cap, cudaStream_t st) {
   k_loop_ctl<<<1, 1, 0, st>>>(h, counters, cap);
   return cudaGetLastError();
@@ -84,12 +78,6 @@ static int ir_blocks(const Batch& b) {
 
 cudaError_t launch_ir_init(const Batch& b, void* const* u, int warm, cudaStream_t st) {
   k_ir_init<<<1024, 256, 0, st>>>(b, ir_u(u, b.ngroups), warm);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_ir_rmap(const Batch& b, int nsys_total, cudaStream_t st) {
-  if (nsys_total <= 0) return cudaSuccess;
-  k_ir_rmap<<<nsys_total, 128, 0, st>>>(b);
   return cudaGetLastError();
 }
 

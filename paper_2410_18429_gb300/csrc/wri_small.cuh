@@ -8,7 +8,9 @@
 
 namespace wri {
 
-// lamd[k] = lambda_g d[k] and r2[k] = lamd[k] for every receiver entry (one block per system).
+// Receiver entries of a solve, one block per system: lamd[k] = lambda_g d[k] and r2[k] = lamd[k]; the receiver
+// bitmaps of the normal-residual norms (rec_col_bits; the caller zeroed them, and receivers are distinct within
+// a system, so every bit is set once); the refinement's map rmap[system][node] = receiver entry.
 template <typename DT, typename RL>
 __global__ void k_setup_rhs(const __grid_constant__ Batch b, int nsys_total) {
   const int s = blockIdx.x;
@@ -20,30 +22,19 @@ __global__ void k_setup_rhs(const __grid_constant__ Batch b, int nsys_total) {
   cx<RL>* lamd = (cx<RL>*)b.lamd;
   cx<RL>* r2 = (cx<RL>*)b.r2;
   const RL lam = RL(G.lambda);
+  uint32_t* mask = const_cast<uint32_t*>(G.rmask);
+  uint32_t* col = const_cast<uint32_t*>(G.rcol);
+  int* rmap = G.rmap ? const_cast<int*>(G.rmap) + (long long)sd.local * G.n : nullptr;
+  const long long plane = (long long)G.nx * G.ny;
   for (int k = sd.rec_begin + threadIdx.x; k < sd.rec_end; k += blockDim.x) {
     const cx<RL> v = lam * to_c(d[k - base], RL(0));
     lamd[k] = v;
     r2[k] = v;
-  }
-}
-
-// Receiver bitmaps of the normal-residual norms (rec_col_bits): one block per system; the
-// caller zeroed both maps.  Receivers are distinct within a system, so every bit is set once.
-__global__ void k_rmask(const __grid_constant__ Batch b, int nsys_total) {
-  const int s = blockIdx.x;
-  if (s >= nsys_total) return;
-  const SysDev& sd = b.sys[s];
-  const GroupDev& G = b.g[sd.group];
-  if (!G.rmask) return;
-  uint32_t* mask = const_cast<uint32_t*>(G.rmask);
-  uint32_t* col = const_cast<uint32_t*>(G.rcol);
-  const long long plane = (long long)G.nx * G.ny;
-  for (int k = sd.rec_begin + threadIdx.x; k < sd.rec_end; k += blockDim.x) {
-    const long long node = b.rec_idx[k];
-    const int z = (int)(node / plane);
-    const long long rem = node - (long long)z * plane;
-    const int y = (int)(rem / G.nx);
-    const int x = (int)(rem - (long long)y * G.nx);
+    const int node = b.rec_idx[k];
+    if (rmap) rmap[node] = k;
+    if (!mask) continue;
+    const int z = (int)(node / plane), rem = (int)(node - z * plane);
+    const int y = rem / G.nx, x = rem - y * G.nx;
     const uint32_t bit = 1u << (x & 31);
     if (G.zw) atomicOr(mask + ((long long)sd.local * plane + rem) * G.zw + (z >> 5), 1u << (z & 31));
     else atomicOr(mask + (((long long)sd.local * G.nz + z) * G.ny + y) * G.rw + (x >> 5), bit);
@@ -53,10 +44,11 @@ __global__ void k_rmask(const __grid_constant__ Batch b, int nsys_total) {
 
 // Control kernel of the device-side CG loop (the WHILE node of the iteration graph): the body runs
 // again while systems remain, no copy wait has timed out and fewer than `cap` bodies have run.
-// counters: [0] systems not done, [1] copy-wait error flag, [2] bodies run (zeroed per solve).
+// counters: [0] systems not done, [1] copy-wait error flag, [2] bodies run (0 before and after a loop).
 __global__ void k_loop_ctl(cudaGraphConditionalHandle h, int* counters, int cap) {
   const int body = ++counters[2];
   const bool go = counters[0] > 0 && counters[1] == 0 && body < cap;
+  if (!go) counters[2] = 0;  // for the next loop
   cudaGraphSetConditional(h, go ? 1u : 0u);
 }
 
@@ -246,17 +238,6 @@ struct IrU {
 };
 
 __device__ __forceinline__ int nsys_of(const Batch& b) { return b.g[b.ngroups - 1].sys0 + b.g[b.ngroups - 1].nsys; }
-
-// Receiver map of the refinement: rmap[system][node] = receiver entry (the map was filled with
-// -1 before); one block per system.
-__global__ void k_ir_rmap(const __grid_constant__ Batch b) {
-  const int s = blockIdx.x;
-  if (s >= nsys_of(b)) return;
-  const SysDev& sd = b.sys[s];
-  const GroupDev& G = b.g[sd.group];
-  int* rmap = const_cast<int*>(G.rmap) + (long long)sd.local * G.n;
-  for (int k = sd.rec_begin + threadIdx.x; k < sd.rec_end; k += blockDim.x) rmap[b.rec_idx[k]] = k;
-}
 
 // x64 = warm ? u : 0, r64 = 0, x32 = 0 on every node; r2_64 = 0 on every receiver entry.
 __global__ void k_ir_init(const __grid_constant__ Batch b, IrU U, int warm) {

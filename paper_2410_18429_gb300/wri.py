@@ -107,9 +107,11 @@ def _check(code: int, what: str):
 
 
 def _stream(stream=None):
+    if stream is not None:
+        return stream.cuda_stream
     import torch
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    # the handle of torch.cuda.current_stream(), without building a Stream object for it
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _ptr(t) -> Optional[int]:
@@ -169,6 +171,9 @@ def _device_tensor(t, what: str, dev=None, dtype=None, min_numel: Optional[int] 
     library checks what it can.  Returns the device seen so far."""
     import torch
     if not isinstance(t, torch.Tensor):
+        return dev
+    if (dev is not None and t.is_cuda and (dtype is None or t.dtype is dtype) and t.device == dev
+            and (min_numel is None or t.numel() >= min_numel) and t.is_contiguous()):
         return dev
     if not t.is_contiguous():
         raise ValueError(f"{what} must be contiguous")
@@ -263,7 +268,7 @@ def _workspace(nbytes: int, device, workspace=None):
 def apply_A(g: GroupSpec, x, adjoint: bool = False, out=None, stream=None):
     """y = A x (or A^H x) for x [nsys, n] complex on the device."""
     import torch
-    dtype = C128 if x.dtype == torch.complex128 else C64
+    dtype = C128 if x.dtype is torch.complex128 else C64
     y = torch.empty_like(x) if out is None else out
     grid = g.grid()
     nsys = x.shape[0] if x.dim() > 1 else 1
@@ -286,9 +291,9 @@ def solve(groups: Sequence[GroupSpec], opts: WriSolveOpts, workspace=None, strea
     if nbytes == 0:
         raise WriError(EINVAL, "wri_workspace_size")
     ws = _workspace(nbytes, dev, workspace)
-    iters = torch.zeros(nsys, dtype=torch.int32, device=dev)
-    relres = torch.zeros(nsys, dtype=torch.float64, device=dev)
-    status = torch.zeros(nsys, dtype=torch.int32, device=dev)
+    iters = torch.empty(nsys, dtype=torch.int32, device=dev)      # written whole by the solve
+    relres = torch.empty(nsys, dtype=torch.float64, device=dev)
+    status = torch.empty(nsys, dtype=torch.int32, device=dev)
     _check(lib.wri_solve_batch(m.arr, m.n, C.byref(opts), _ptr(iters), _ptr(relres), _ptr(status), _ptr(ws),
                                ws.numel(), _stream(stream)), "wri_solve_batch")
     return iters, relres, status
@@ -301,7 +306,7 @@ def source_estimate(groups: Sequence[GroupSpec], dtype: int, workspace=None, str
     dev = groups[0].u.device
     nsys = sum(g.nsys for g in groups)
     ws = _workspace(lib.wri_aux_workspace_size(m.arr, m.n), dev, workspace)
-    out = torch.zeros(nsys, 2, dtype=torch.float64, device=dev)
+    out = torch.empty(nsys, 2, dtype=torch.float64, device=dev)
     _check(lib.wri_source_estimate(m.arr, m.n, dtype, _ptr(out), _ptr(ws), ws.numel(), _stream(stream)),
            "wri_source_estimate")
     return torch.view_as_complex(out)
