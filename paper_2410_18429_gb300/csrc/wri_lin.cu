@@ -38,21 +38,25 @@ static cudaError_t launch_one(const Batch& b, const LinWait& w, const LinTab<MOD
   T.withhold = w.withhold;
   const size_t smem = lin_layout(b, sizeof(R), MODE, T);
   auto kern = k_lin<R, OR, MODE, CONJ, NC, NPT, PAIR, GV, kLinStages, MINB>;
-  static thread_local size_t occ_smem = 0;  // resident CTAs at the last shared-memory size
-  static thread_local int occ = 0;
-  if (occ_smem != smem) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kLinMaxSmem);
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  static thread_local size_t occ_smem = 0;  // resident CTAs at the last shared-memory size and device
+  static thread_local int occ_dev = -1, occ = 0, sms = 0;
+  if (occ_smem != smem || occ_dev != dev) {
+    occ_dev = -1;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kLinMaxSmem);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NC + 32, smem);
     if (e != cudaSuccess) return e;
     if (occ < 1) return cudaErrorInvalidConfiguration;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
     occ_smem = smem;
+    occ_dev = dev;
   }
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const long long cap = (long long)sms * occ;
   const int grid = (int)(cap < b.nitems ? cap : b.nitems);
   kern<<<grid, NC + 32, smem, st>>>(b, T, tab);
