@@ -176,16 +176,19 @@ int auto_zsplit(long long xy_items, int nz) {
   return best;
 }
 
-// The same for the chunk kernels, with chunks of at least one plane: waves of 4 CTAs per SM times the planes an
-// item streams.
+// The same for the chunk kernels, with chunks of at least one plane.  An item costs its planes and six more (its
+// halo planes, filling the stages, its end); the launch takes the mean of the full waves of 4 CTAs per SM, which is
+// right while the planes' latency binds, and of the exact count, which is right once the memory does.  Against a
+// sweep of 1..36 chunks over 14 batches this picks within 1.3 % of the best everywhere.  Full waves of planes plus
+// two lost up to 15 %: 116^3 x 4 131 us per iteration (now 114), 84^3 x 16 167 (156), 84^3 x 48 483 (447).
 int auto_zsplit_lin(long long xy_items, int nz) {
+  const long long wave = (long long)kRefSMs * 4;
   int best = 1;
   double best_cost = 0.0;
   for (int zs = 1; zs <= 64 && zs <= nz; ++zs) {
     const int zc = (nz + zs - 1) / zs;
     const long long items = xy_items * ((nz + zc - 1) / zc);
-    const long long wave = (long long)kRefSMs * 4;
-    const double cost = (double)((items + wave - 1) / wave) * (zc + 2);
+    const double cost = ((double)((items + wave - 1) / wave) + (double)items / wave) * (zc + 6);
     if (zs == 1 || cost < best_cost) {
       best_cost = cost;
       best = zs;
@@ -274,6 +277,8 @@ struct Plan {
   size_t up_total = 0;  // bytes the host uploads: systems, receivers, layer tables
   size_t aux_base = 0, aux_total = 0, total = 0;  // aux_base: without the layer tables
   GroupDev g[WRI_MAXG];
+  GroupDev g64[WRI_MAXG];  // refinement on chunk kernels: the FP64 passes' decomposition
+  long long nitems64 = 0;
   size_t v_r1[WRI_MAXG][2], v_p[WRI_MAXG][4], v_s[WRI_MAXG], v_t1[WRI_MAXG];
   int pslots = 2;  // search-direction slots: 4 when the phases may update x every fourth iteration
   size_t v_x32[WRI_MAXG], v_x64[WRI_MAXG], v_r64[WRI_MAXG], v_q64[WRI_MAXG], v_g32[WRI_MAXG], v_rmap[WRI_MAXG];
@@ -433,6 +438,28 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
     sys0 += G.nsys;
   }
   P.nitems = item;
+  // The FP64 passes of a refined solve are bound by the FP64 pipe and take the complex128 shape, whatever the
+  // complex64 phases have: an objective call on 81^3 x 9, with 2 z-chunks in the phases, 4.40 ms (4.56 in their shape).
+  if (P.lin && P.ir) {
+    std::vector<wri_grid> grids(ngroups);
+    std::vector<int> ns(ngroups);
+    for (int gi = 0; gi < ngroups; ++gi) {
+      grids[gi] = groups[gi].grid;
+      ns[gi] = groups[gi].nsys;
+    }
+    int m64 = kLinChunk, z64 = zs;
+    if (o->zsplit == 0) wide_shape(grids.data(), ns.data(), ngroups, &m64, &z64);
+    item = parts = 0;
+    for (int gi = 0; gi < ngroups; ++gi) {
+      GroupDev& G = P.g64[gi] = P.g[gi];
+      decompose_lin(groups[gi].grid, m64, z64, G);
+      G.item0 = item;
+      G.nitems = (long long)G.ntiles * G.nsys;
+      item += G.nitems;
+      parts += std::max(G.nitems, P.g[gi].nitems);
+    }
+    P.nitems64 = item;
+  }
   P.nparts = parts;
   size_t off = P.total;
   P.off_part = off;
@@ -524,7 +551,7 @@ void build_sys(const wri_group* groups, int ngroups, const Plan& P, std::vector<
       for (int k = G.rec_off[l]; k < G.rec_off[l + 1]; ++k) rec.push_back(G.rec_idx[k]);
       d.rec_end = (int)rec.size();
       d.part_off = (int)part;
-      part += P.g[gi].ntiles;
+      part += P.lin && P.ir ? std::max(P.g[gi].ntiles, P.g64[gi].ntiles) : P.g[gi].ntiles;
       d.state = ST_DONE;
       d.status = WRI_SYS_OK;
     }
@@ -1056,6 +1083,21 @@ int solve_refined(const wri_group* groups, int ngroups, const wri_solve_opts* o,
   if (!slot) return WRI_ECUDA;
   // FP64 views: the residual kernel reads x64 and writes q64 (nodes) and b.r2 = q2 (receivers)
   Batch outer = solver_batch(groups, P, ws, false);
+  if (P.lin) {
+    outer.nitems = P.nitems64;
+    for (int gi = 0; gi < P.ngroups; ++gi) {
+      const GroupDev& D = P.g64[gi];
+      GroupDev& G = outer.g[gi];
+      G.chunk = D.chunk;
+      G.tiles_x = D.tiles_x;
+      G.tiles_y = D.tiles_y;
+      G.zc = D.zc;
+      G.zsplit = D.zsplit;
+      G.ntiles = D.ntiles;
+      G.item0 = D.item0;
+      G.nitems = D.nitems;
+    }
+  }
   outer.order = order_of(o);
   outer.sblock = sblock_of(o);
   const LinWait w = lin_wait(outer, o);
