@@ -161,18 +161,25 @@ __device__ void finalize_lin(const Batch& b, const GroupDev& G, SysDev* sd, int 
   const R step = MODE == M_P2 ? R(sd->alpha * (double)lam) : R(0);
   const C* p = (MODE == M_P1 || MODE == M_P2) ? (const C*)G.p[pslot(b, sd->iter)] + off : nullptr;
   if (!(MODE == M_SH && G.rmap)) {
+    // A receiver is a few trips to the L2 that nothing else of its system is left to hide: the next index is loaded
+    // a receiver ahead and p, s and r2 together (index, then p, then s: 81^3 with 2025 receivers x 1 system 49.8 ->
+    // 44.1 us per iteration, x 9 137 -> 125).  Two receivers at a time gave 41.0 and 124, but the registers they
+    // hold spill in the plane loops: 148^3 x 4 206 -> 214.
+    int next = sd->rec_begin + tid < sd->rec_end ? b.rec_idx[sd->rec_begin + tid] : 0;
     for (int k = sd->rec_begin + tid; k < sd->rec_end; k += NT) {
-      const int node = b.rec_idx[k];
+      const int node = next;
+      if (k + NT < sd->rec_end) next = b.rec_idx[k + NT];
       if (MODE == M_P1) {
         part += (double)lam * (double)lam * (double)abs2(ldcg_c(p + node));
       } else if (MODE == M_RES) {
         r2[k] = ((const C*)b.lamd)[k] - lam * ldcg_c((const C*)G.x + off + node);
       } else {
+        OC* S = (OC*)G.s + off + node;
+        const OC s_old = ldcg_c(S);
         C r = r2[k];
         if (MODE == M_P2) r2[k] = r = r - step * ldcg_c(p + node);
-        OC* S = (OC*)G.s + off + node;
         // the stencil pass left receiver nodes out of its partial sums
-        const OC sn = to_c(to_c(ldcg_c(S), R(0)) + lam * r, OR(0));
+        const OC sn = to_c(to_c(s_old, R(0)) + lam * r, OR(0));
         *S = sn;
         part += (double)abs2(sn);
       }
