@@ -89,6 +89,33 @@ __device__ __forceinline__ cx<R> stretch_at(const AxisPml& a, R pos) {
   return mkc(R(1), CONJ ? -im : im);
 }
 
+// Not inlined: predicated off beside the common path, the conversion would still take its slots.
+static __device__ __noinline__ double widen_cvt(float v) { return (double)v; }
+
+// float to double, exactly, by rebiasing the exponent in integer arithmetic: a conversion instruction runs on
+// the narrow FP64 pipe.  Zeros too; subnormals, infinities and NaN take the instruction.
+__device__ __forceinline__ double widen(float v) {
+  const uint32_t b = __float_as_uint(v), a = b & 0x7fffffffu;
+  if (a - 0x00800000u >= 0x7f000000u && a != 0u) return widen_cvt(v);
+  const uint32_t hi = (a >> 3) + (a ? 0x38000000u : 0u);
+  return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double v) { return v; }
+
+// double to float, rounded to nearest even, the same way: the exponent rebiased and the 29 dropped bits rounded in
+// integers.  Zeros too; results near or beyond the ends of the float range, infinities and NaN take the instruction.
+static __device__ __noinline__ float narrow_cvt(double v) { return (float)v; }
+__device__ __forceinline__ float narrow(double v) {
+  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v), a = hi & 0x7fffffffu;
+  if (a - (923u << 20) >= (226u << 20)) {  // not 2^-100 <= |v| < 2^126
+    if ((a | lo) != 0u) return narrow_cvt(v);
+    return __uint_as_float(hi);
+  }
+  const uint32_t t = __funnelshift_l(lo, a, 3) - (896u << 23);
+  return __uint_as_float((hi & 0x80000000u) | (t + (((lo & 0x1fffffffu) + 0x0fffffffu + (t & 1u)) >> 29)));
+}
+
+
 // ------------------------------------------------------------------ kernel modes
 enum Mode : int {
   M_APPLY = 0,  // y = A x (or A^H x); no reduction

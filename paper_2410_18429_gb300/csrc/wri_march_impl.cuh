@@ -212,19 +212,6 @@ __device__ void finalize(const Batch& b, const GroupDev& G, SysDev* sd, int sl, 
   }
 }
 
-// Not inlined: predicated off beside the common path, the conversion would still take its slots.
-static __device__ __noinline__ double widen_cvt(float v) { return (double)v; }
-
-// float to double, exactly, by rebiasing the exponent in integer arithmetic: a conversion instruction runs on
-// the narrow FP64 pipe.  Zeros too; subnormals, infinities and NaN take the instruction.
-__device__ __forceinline__ double widen(float v) {
-  const uint32_t b = __float_as_uint(v), a = b & 0x7fffffffu;
-  if (a - 0x00800000u >= 0x7f000000u && a != 0u) return widen_cvt(v);
-  const uint32_t hi = (a >> 3) + (a ? 0x38000000u : 0u);
-  return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
-}
-__device__ __forceinline__ double widen(double v) { return v; }
-
 // Re(conj(a) b), its rounding spelled out: the gradient must not depend on how an instantiation contracts it.
 __device__ __forceinline__ float re_dot(float2 a, float2 b) { return __fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)); }
 __device__ __forceinline__ double re_dot(double2 a, double2 b) { return __fma_rn(a.x, b.x, __dmul_rn(a.y, b.y)); }
