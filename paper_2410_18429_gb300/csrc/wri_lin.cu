@@ -30,14 +30,15 @@ size_t lin_smem(const Batch& b, int rbytes, int mode) {
   return lin_layout(b, rbytes, mode, T);
 }
 
-template <typename R, typename OR, int MODE, bool CONJ, int NC, int NPT, bool PAIR, bool GV, int MINB>
+template <typename R, typename OR, int MODE, bool CONJ, int NC, int NPT, bool PAIR, bool GV, int MINB,
+          bool XO = (sizeof(R) == 8)>
 static cudaError_t launch_one(const Batch& b, const LinWait& w, const LinTab<MODE>& tab, cudaStream_t st) {
   LinSet T;
   T.err = w.err;
   T.wait_ns = w.wait_ns;
   T.withhold = w.withhold;
   const size_t smem = lin_layout(b, sizeof(R), MODE, T);
-  auto kern = k_lin<R, OR, MODE, CONJ, NC, NPT, PAIR, GV, kLinStages, MINB>;
+  auto kern = k_lin<R, OR, MODE, CONJ, NC, NPT, PAIR, GV, kLinStages, MINB, XO>;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -61,6 +62,13 @@ static cudaError_t launch_one(const Batch& b, const LinWait& w, const LinTab<MOD
   const int grid = (int)(cap < b.nitems ? cap : b.nitems);
   kern<<<grid, NC + 32, smem, st>>>(b, T, tab);
   return cudaGetLastError();
+}
+
+// planes of the batch's longest items
+static int longest(const Batch& b) {
+  int zc = 0;
+  for (int g = 0; g < b.ngroups; ++g) zc = b.g[g].zc > zc ? b.g[g].zc : zc;
+  return zc;
 }
 
 cudaError_t launch_lin(int rbytes, int obytes, int mode, bool conj, const Batch& b, const LinWait& w,
@@ -97,8 +105,15 @@ cudaError_t launch_lin(int rbytes, int obytes, int mode, bool conj, const Batch&
     }
   } else {
     switch (mode) {
-      case M_P1: WRI_LIN(M_P1, false, double, double, 256, 1, false, false, 2)
-      case M_P2: WRI_LIN(M_P2, true, double, double, 256, 1, false, false, 2)
+      // long items: a kind of loop more (see the kernel's step)
+      case M_P1:
+        if (longest(b) < 8)
+          return launch_one<double, double, M_P1, false, 256, 1, false, false, 2, false>(b, w, LinTab<M_P1>(), st);
+        WRI_LIN(M_P1, false, double, double, 256, 1, false, false, 2)
+      case M_P2:
+        if (longest(b) < 8)
+          return launch_one<double, double, M_P2, true, 256, 1, false, false, 2, false>(b, w, LinTab<M_P2>(), st);
+        WRI_LIN(M_P2, true, double, double, 256, 1, false, false, 2)
       case M_SH:
         if (obytes == 4) WRI_LIN(M_SH, true, double, float, 256, 1, false, false, 2)
         WRI_LIN(M_SH, true, double, double, 256, 1, false, false, 2)

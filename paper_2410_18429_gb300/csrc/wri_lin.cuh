@@ -196,8 +196,9 @@ __device__ void finalize_lin(const Batch& b, const GroupDev& G, SysDev* sd, int 
 
 // R: arithmetic; OR: type of the stencil's output vector; MODE: M_APPLY, M_SH, M_RES, M_P1, M_P2 or M_GRAD; NC
 // consumer threads of NPT nodes each; GV: phase 2 adds S^H r64 (gvec); PAIR: a thread's two nodes are adjacent (16-byte accesses: nx even
-// and every pointer aligned), otherwise they lie NC apart; S stages.
-template <typename R, typename OR, int MODE, bool CONJ, int NC, int NPT, bool PAIR, bool GV, int S, int MINB>
+// and every pointer aligned), otherwise they lie NC apart; S stages; XO:
+// warps outside the y layers have loops of their own.
+template <typename R, typename OR, int MODE, bool CONJ, int NC, int NPT, bool PAIR, bool GV, int S, int MINB, bool XO>
 __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ Batch b, const __grid_constant__ LinSet T,
                                                          const __grid_constant__ LinTab<MODE> tab_in) {
   typedef cx<R> C;
@@ -375,7 +376,8 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
     int ni[NPT], nj[NPT];
     uint32_t rcb = 0;      // the thread's columns that hold receivers of this system
     uint32_t rz[NPT] = {};  // their receivers at the current 32 planes
-    bool gen = false;  // a stretched axis or a neighbour outside the grid
+    bool gen = false;   // a stretched axis or a neighbour outside the grid
+    bool geny = false;  // the y axis too
 #pragma unroll
     for (int r = 0; r < NPT; ++r) {
       own[r] = e0 + r * RS < c1;
@@ -383,12 +385,14 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
       nj[r] = ee / nx;
       ni[r] = ee - nj[r] * nx;
       const int w = npml > 0 ? npml + 1 : 1;
-      gen = gen || (own[r] && !(ni[r] >= w && ni[r] < nx - w && nj[r] >= w && nj[r] < ny - w));
+      geny = geny || (own[r] && !(nj[r] >= w && nj[r] < ny - w));
+      gen = gen || geny || (own[r] && !(ni[r] >= w && ni[r] < nx - w));
       if (NORM && G.rmask && own[r]) {
         if ((__ldg(G.rcol + ((long long)sl * ny + nj[r]) * G.rw + (ni[r] >> 5)) >> (ni[r] & 31)) & 1u) rcb |= 1u << r;
       }
     }
     gen = __any_sync(0xffffffffu, gen);
+    if (XO) geny = __any_sync(0xffffffffu, geny);
     const bool idle = !__any_sync(0xffffffffu, own[0]);  // the warp lies past the chunk's end
 
     const R coef = MODE == M_P1 ? (iter > 0 ? R(sd->beta) : R(0)) : MODE == M_P2 ? -R(sd->alpha) : R(0);
@@ -610,9 +614,13 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
       }
     }
     // One plane of the item: its F, the z + 1 term of plane k - 1, and its own stencil without that term.
-    // gen_c: the x and y coefficients are general; zg_c: plane k lies in a z layer.
+    // gen_c: 1 the x coefficients are general, 2 those of x and y; zg_c: plane k lies in a z layer.  XO (FP64)
+    // has a kind of its own for x alone, with the same roundings and 6 FP64 instructions of 31 less: rows of 116
+    // nodes leave half of the warps with an x layer and most of these outside the y layers.  A^H on 81^3 x 9 285
+    // -> 264 us, gradient on 148^3 x 16 2883 -> 2766.  The phases take it for items of 8 planes and more: 148^3 x 1
+    // 521 -> 505 us per iteration, 81^3 x 9 835 -> 804, but 36^3 x 1, with items of 3 planes, 38.8 -> 40.1.
     auto step = [&](auto gen_c, auto zg_c, int k) -> bool {
-      constexpr bool GEN = decltype(gen_c)::value, ZG = decltype(zg_c)::value;
+      constexpr bool GEN = decltype(gen_c)::value > 0, GY = decltype(gen_c)::value == 2, ZG = decltype(zg_c)::value;
       if (!wait()) return false;
       const C* A = reinterpret_cast<const C*>(base + da) + o;
       const C* B = HASB ? reinterpret_cast<const C*>(base + db + T.off_b) + o : nullptr;
@@ -679,7 +687,8 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         for (int r = 0; r < NPT; ++r) {
           const C d = DIFF ? v[r] - fc[r] : v[r];
           t[r] = ZG ? cfma(hz, d, q[r]) : rfma(ih2, d, q[r]);
-          if (GEN && !GRAD) t[r] = smul(sy_[PAIR ? 0 : r], smul(sx_[r], t[r]));
+          if (GEN && !GRAD) t[r] = smul(sx_[r], t[r]);
+          if (GY && !GRAD) t[r] = smul(sy_[PAIR ? 0 : r], t[r]);
         }
         if constexpr (GRAD) {
           accum(k - 1, t, GEN, ZG);
@@ -732,8 +741,8 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         if (GEN) {
           acc = cfma(am[r], l[r], acc);
           acc = cfma(ap[r], rgt[r], acc);
-          acc = cfma(bm[PAIR ? 0 : r], ym[r], acc);
-          acc = cfma(bp[PAIR ? 0 : r], yp[r], acc);
+          acc = GY ? cfma(bm[PAIR ? 0 : r], ym[r], acc) : rfma(ih2, ym[r], acc);
+          acc = GY ? cfma(bp[PAIR ? 0 : r], yp[r], acc) : rfma(ih2, yp[r], acc);
           acc = ZG ? cfma(cz.am, zm, acc) : rfma(ih2, zm, acc);
         } else {
           C sum = (l[r] + rgt[r]) + (ym[r] + yp[r]);
@@ -802,7 +811,15 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
           dead = !wait();
           if (!dead) release();
         }
-      } else if (!dead) dead = gen ? !planes(std::true_type()) : !planes(std::false_type());
+      } else if (!dead) {
+        if (!gen) {
+          dead = !planes(std::integral_constant<int, 0>());
+        } else if (XO && !geny) {
+          if constexpr (XO) dead = !planes(std::integral_constant<int, 1>());
+        } else {
+          dead = !planes(std::integral_constant<int, 2>());
+        }
+      }
       if (!dead) {
         // the plane above completes the last one
         C v[NPT];
