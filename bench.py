@@ -36,6 +36,8 @@ BYTES_PER_NODE_SYS = 80.0  # one CGLS iteration, per node and system: phase 1 48
 # grouped-update configurations: x read and written every m-th iteration, with m - 1 extra p reads
 # then: phase 1 (m 32 + 16 + 8 (m - 1)) / m = 44 B (m = 2) or 42 B (m = 4)
 XSTEPS = {22: 2, 23: 2, 24: 4}
+CHUNK_CONFIGS = (18, 22, 24)  # the chunk kernels; 24 is the automatic choice
+CHUNK_DEFAULT = 24
 MODEL_BYTES = 8.0          # m (float32) read by both phases, per node of a group, shared by its systems
 K_POLL = 2                 # CG iterations per body of the iteration graph's device-side loop
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "cg_iteration_traffic.json")
@@ -102,7 +104,9 @@ def phase_kernel_name(opts):
     k = int(opts.kernel)
     if k == 1:
         return "k_march"
-    cfg = k - 2 if k >= 2 else 8
+    cfg = k - 2 if k >= 2 else CHUNK_DEFAULT
+    if cfg in CHUNK_CONFIGS:
+        return "k_lin + k_xupdate"
     return "k_phase_tma" if cfg <= 3 else "k_phase_tma2" if cfg <= 8 else "k_phase_ws"
 
 
@@ -249,7 +253,7 @@ def run_reference(args, ws, rank):
 # ---------------------------------------------------------------- grouping sweep
 def run_group_sweep(args):
     """Grouping (Eq. Mmatrix2): one CGLS iteration of n_b systems of the largest grid advanced by
-    one batched call, for every n_b of ``--group-sweep`` (the default TMA configuration and
+    one batched call, for every n_b of ``--group-sweep`` (the automatic configuration and
     order unless ``--kernel`` / ``--order`` say otherwise; no autotuning, so every n_b runs the
     same kernel).  The per-iteration time is the difference of two solves of 20 and 80
     iterations (tol = 0, CUDA events on the launching stream, best of two each), which removes
@@ -299,7 +303,8 @@ def run_group_sweep(args):
         ta = min(timed(20) for _ in range(2))
         tb = min(timed(80) for _ in range(2))
         t_iter = (tb - ta) / 60.0
-        alg = n * (bytes_per_node_sys(base) * nb + MODEL_BYTES)
+        eff = base if base.kernel else wri.make_opts(kernel=2 + CHUNK_DEFAULT)  # what the automatic choice runs
+        alg = n * (bytes_per_node_sys(eff) * nb + MODEL_BYTES)
         print(json.dumps({"group_sweep": nb, "grid": f"{g0.spec.nx}x{g0.spec.ny}x{g0.spec.nz}",
                           "ms_per_iter": t_iter * 1e3, "us_per_system_iter": t_iter / nb * 1e6,
                           "gpt_iter_s": nb * n / t_iter / 1e9, "hbm_gbs": alg / t_iter / 1e9,
@@ -315,8 +320,8 @@ def run_camembert_shape(args):
     """One misfit + gradient evaluation on the shape of the paper's timing case (Sec. "Evaluation of
     GPU Acceleration Efficiency", Table CMPTime: a 3 km cube at h = 50 m, 61^3 nodes, 9 sources,
     2025 receivers, 5 Hz, relative residual 1e-6), with synthetic model and data on a 10-cell
-    absorbing layer (81^3 computational nodes), and on the nearest cube whose x extent the TMA phases
-    take (60^3 + layer, 80^3).  Certified precision configuration, refined to an
+    absorbing layer (81^3 computational nodes), and on the nearest cube of even extents
+    (60^3 + layer, 80^3).  Certified precision configuration, refined to an
     FP64 normal-equation residual of 1e-6 (every system must end with status OK).  The 9 systems
     are evaluated in batched calls of n_b systems (9, 4 and 1, so 1, 3 and 9 calls), each call a
     solve, a source estimate and a gradient, after one untimed evaluation; CUDA events on the
@@ -335,8 +340,7 @@ def run_camembert_shape(args):
 
 
 def camembert_case(args, G, dev, stream):
-    """The evaluations of run_camembert_shape on one grid (61^3 physical: x extent 81, z-march
-    kernels; 60^3: x extent 80, TMA phases)."""
+    """The evaluations of run_camembert_shape on one grid (61^3 or 60^3 physical)."""
     import torch
 
     import synth
@@ -396,7 +400,7 @@ def camembert_case(args, G, dev, stream):
     print(json.dumps({"camembert_shape": {
         "grid": f"{g.nx}x{g.ny}x{g.nz} computational nodes ({g.nx - 2 * g.npml}^3 physical + {g.npml}-cell layer), "
                 f"h = {g.h} m",
-        "phase_kernels": "TMA" if g.nx % 4 == 0 else "z-march (x extent not a multiple of 4)",
+        "phase_kernels": "linear chunks (k_lin)",
         "freq_hz": G.freq, "systems": int(G.nsys), "receivers_per_system": int(G.rec_off[1] - G.rec_off[0]),
         "precision": "complex64 CGLS inside FP64 iterative refinement to an FP64 normal-equation residual of 1e-6; "
                      "FP64 source estimate and gradient from the refinement's residual",
@@ -420,17 +424,17 @@ def solve_opts(wri, args, certified=True, iters=None, **kw):
 
 
 def step_launches(iters, k, certified, ngroups):
-    """Kernels of libwri in one step (the claim of the bench line).  Both configurations: the
-    receiver bitmaps, the z tables, the right-hand sides, the initial S^H b, the loop of phase 1 +
-    phase 2 in bodies of K iterations with one control kernel each (the P1 after the last iteration
-    is the x-only pass), the export and the source estimate.  Certified: the refinement's receiver
-    map, init and cold start (r2), its update, one FP64 residual step of 3 kernels (residual,
-    forcing, S^H), the final rounding, and the gradient from that residual (one kernel per group).
+    """Kernels of libwri in one step on the chunk kernels (the claim of the bench line).  Both
+    configurations: the vectors' zeroing, the right-hand sides with the receiver bitmaps, the initial
+    S^H b, the loop of phase 1 + phase 2 in bodies of K iterations with an iterate update after every
+    fourth and at a body's end and one control kernel each, the export and the source estimate.
+    Certified: the refinement's cold start, its update (nodes and receivers), one FP64 residual step
+    (residual, S^H), the final rounding, and the gradient from that residual (one kernel per group).
     Unrefined: the gradient's z tables, gradient kernel and data term."""
     bodies = -(-(iters + 1) // k)
-    loop = bodies * (2 * k + 1)
-    fixed = 1 + 1 + 1 + 1 + 1 + 1
-    fixed += (1 + 1 + 1 + 1 + 3 + 1 + ngroups) if certified else 3
+    loop = bodies * (2 * k + -(-k // 4) + 1)
+    fixed = 5
+    fixed += (1 + 2 + 2 + 1 + ngroups) if certified else 3
     return loop + fixed
 
 

@@ -102,7 +102,8 @@ typedef struct {
   void* u;                  /* device [nsys][n] complex (dtype): in = x0 if warm_start, out = u */
   void* u64;                /* WRI_C64 only, optional: device [nsys][n] complex128 (16-byte aligned)
                                or NULL.  wri_solve_batch also writes the solution here, in FP64
-                               (the refinement's FP64 master; without refinement, u widened), and
+                               (the refinement's FP64 master, which it keeps here while it runs;
+                               without refinement, u widened), and
                                wri_source_estimate / wri_gradient then read it instead of u and use
                                FP64 stencils: the gradient needs the PDE residual A u - a e, which
                                rounding u to complex64 would swamp.  In one call either every
@@ -129,16 +130,19 @@ typedef struct {
                           its control kernel (0 = library default, about 300 us of work) */
   int32_t tile;        /* tile configuration (0 = autotuned / default, see wri_tile_count) */
   int32_t zsplit;      /* z-chunks per tile column (0 = chosen from the batch size) */
-  int32_t kernel;      /* 0 = automatic (TMA-pipelined phases when the batch allows them),
-                          1 = z-march kernels only, 2 + c = TMA configuration c (0..24; 9..24
-                          are the warp-specialised kernels; 22 and 23 update the
-                          iterate every second iteration, 24 every fourth); see wri_autotune */
-  int32_t order;       /* TMA phases: 0 = automatic (6), 1 = tiles of a system consecutive,
+  int32_t kernel;      /* 0 = automatic (the chunk kernels, as configuration 24), 1 = z-march
+                          kernels only, 2 + c = configuration c (0..24).  18, 22 and 24 are the
+                          chunk kernels (any x extent, both dtypes; 18 and 22 update the iterate
+                          every second iteration, 24 every fourth in complex64), the others the
+                          TMA box phases (9..24 warp-specialised; 23 updates the iterate every
+                          second iteration); see wri_autotune.  An explicit `tile` with a batch
+                          the boxes cannot take runs on the z-march kernels. */
+  int32_t order;       /* chunk and TMA phases: 0 = automatic (6), 1 = tiles of a system consecutive,
                           2 = systems of a tile consecutive, 3 = z-chunk slowest,
                           4 / 5 / 6 = blocks of 4 / 8 / 16 systems, tiles in order */
   int32_t l2_promotion; /* TMA copies: L2 fill size on a miss, 0 = automatic, 1 = none,
                            2 = 64 B, 3 = 128 B, 4 = 256 B */
-  int32_t wait_limit_us; /* TMA phases: time limit of every wait of the copy pipelines, in
+  int32_t wait_limit_us; /* chunk and TMA phases: time limit of every wait of the copy pipelines, in
                             microseconds (0 = 2 s).  A wait that runs out stops the solve:
                             wri_solve_batch returns WRI_ECUDA and the context stays usable. */
   int32_t host_loop;     /* 1: the host replays a graph of poll_every iterations and reads the
@@ -146,8 +150,8 @@ typedef struct {
                             WHILE node).  Kernel profilers cannot see kernels inside conditional
                             graph nodes; this keeps the phase kernels visible to them.  The
                             environment variable WRI_HOST_LOOP=1 sets it for every solve. */
-  int32_t test_withhold; /* test hook of the bounded waits, 0 = off.  k > 0: in the warp-specialised
-                            TMA phases the copy warp of block 0 never issues its (k-1)-th plane
+  int32_t test_withhold; /* test hook of the bounded waits, 0 = off.  k > 0: in the chunk and the
+                            warp-specialised TMA phases the copy warp of block 0 never issues its (k-1)-th plane
                             fill, so the wait for it runs out after wait_limit_us.  Nothing
                             faults or hangs; the call returns WRI_ECUDA. */
 } wri_solve_opts;
@@ -163,7 +167,7 @@ WRI_API int wri_apply_AH(const wri_grid* grid, int dtype, const void* m, int nsy
 
 /* Bytes of device workspace wri_solve_batch needs for these groups and options
  * (0 on invalid arguments).  The workspace must be 256-byte aligned.  With opts->kernel = 0
- * (automatic) it also covers the four search-direction vectors per system of TMA configuration
+ * (automatic) it also covers the four search-direction vectors per system of configuration
  * 24, so that a workspace sized before wri_autotune fits every configuration it may choose. */
 WRI_API size_t wri_workspace_size(const wri_group* groups, int ngroups, const wri_solve_opts* opts);
 
@@ -269,8 +273,7 @@ WRI_API int wri_gradient_noalloc(const wri_group* groups, int ngroups, int dtype
 
 /* Autotuner of the batched solve (an interface outside the paper, which prescribes no
  * kernel configuration).  For a complex64 batch it times `trial_iters` CGLS iterations (>= 2)
- * of every candidate pair (TMA configuration 8, 9, 12, 13, 17, 18, 22 or 24 x work-item order 2, 5
- * or 6)
+ * of every candidate pair (configuration 8, 9, 12, 13, 17, 18, 22 or 24 x work-item order 2, 5 or 6)
  * on the caller's own batch, on `stream`, and writes the fastest into opts->kernel and
  * opts->order (other fields unchanged).  With refinement (max_refine > 0) the candidates are
  * the warp-specialised configurations (9, 12, 13, 17, 18, 22, 24), which run its inner solves, and the
@@ -279,7 +282,7 @@ WRI_API int wri_gradient_noalloc(const wri_group* groups, int ngroups, int dtype
  *   - The choice is cached for the process, keyed by the device, the grids, the system counts
  *     and the receiver counts: a repeated call for the same batch shape returns the cached
  *     choice without timing anything (and without touching u).
- *   - Batches the TMA phases cannot take (complex128, the unfused baseline, an x extent that is
+ *   - Batches the TMA box phases cannot take (complex128, the unfused baseline, an x extent that is
  *     not a multiple of 4) keep opts unchanged and return WRI_OK.
  *   - Synchronises `stream` (it reads event timings on the host). */
 WRI_API int wri_autotune(const wri_group* groups, int ngroups, wri_solve_opts* opts, int trial_iters,
