@@ -31,9 +31,9 @@
 // issue utilisation, 270 warp instructions per 64 nodes and plane (320 in the boxes, 374 before the warps
 // without stretched nodes and the z layers got loops of their own).  Running addresses in the copy warp, no
 // plane or lane checks in the main loop and one set of y coefficients per pair: 148^3 x 32 46.8 -> 45.8 us
-// per system and iteration, 84^3 x 64 9.0 -> 8.7.  Chunks of 512 nodes (half the halo) are slower: 47.8
-// and 9.4, 276 x 276 x 180 x 4 181 against 173.  Stages beyond three are slower (the
-// plane streams alone: 749 against 550 us with six).  complex128 passes are bound by the FP64 pipe (86-90 %
+// per system and iteration (41.7 with the shorter end of a phase), 84^3 x 64 9.0 -> 8.7.  Chunks of 512 nodes
+// (half the halo) are slower: 47.8 and 9.4, 276 x 276 x 180 x 4 181 against 173.  Stages beyond three are slower
+// (the plane streams alone: 749 against 550 us with six).  complex128 passes are bound by the FP64 pipe (86-90 %
 // busy).
 //
 // All waits are bounded as in wri_tma.cuh: a time-out raises the CTA's abort flag and the launch's error
