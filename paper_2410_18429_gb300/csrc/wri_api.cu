@@ -275,8 +275,7 @@ struct Plan {
   size_t off_r2_64 = 0, off_r2_in = 0;  // refinement: FP64 receiver residual master, complex64 inner r2
   size_t off_ltab32[WRI_MAXG], off_ltab64[WRI_MAXG];  // layer tables of the chunk kernels
   size_t zero_total = 0;  // bytes from off_rem that a solve starts with zeroed
-  size_t up_total = 0;  // bytes the host uploads: systems, receivers, layer tables
-  size_t aux_base = 0, aux_total = 0, total = 0;  // aux_base: without the layer tables
+  size_t aux_base = 0, aux_total = 0, total = 0;  // aux_base: without the layer tables, which come last
   GroupDev g[WRI_MAXG];
   GroupDev g64[WRI_MAXG];  // refinement on chunk kernels: the FP64 passes' decomposition
   long long nitems64 = 0;
@@ -299,26 +298,26 @@ void plan_aux(const wri_group* groups, int ngroups, Plan& P) {
     P.nnz_total += groups[gi].rec_off[groups[gi].nsys];
   }
   size_t off = 0;
-  P.off_sys = off;
-  off += align_up(sizeof(SysDev) * (size_t)P.nsys_total);
-  P.off_rec = off;
-  off += align_up(sizeof(int) * (size_t)std::max(P.nnz_total, 1));
-  const size_t tabs = off;
-  for (int gi = 0; gi < ngroups; ++gi) {  // layer tables of the chunk kernels (one upload with the above)
-    const size_t e = (size_t)kLayerTab * (groups[gi].grid.npml + 1);
-    P.off_ltab32[gi] = off;
-    off += align_up(sizeof(float) * e);
-    P.off_ltab64[gi] = off;
-    off += align_up(sizeof(double) * e);
-  }
-  P.up_total = off;
   for (int gi = 0; gi < ngroups; ++gi) {  // [2][nz][3] complex coefficients in FP32 and FP64
     P.off_ztab[gi] = off;
     off += align_up(sizeof(float) * 2 * 2 * 3 * (size_t)groups[gi].grid.nz);
     P.off_ztab64[gi] = off;
     off += align_up(sizeof(double) * 2 * 2 * 3 * (size_t)groups[gi].grid.nz);
   }
-  P.aux_base = off - (P.up_total - tabs);
+  P.off_sys = off;
+  off += align_up(sizeof(SysDev) * (size_t)P.nsys_total);
+  P.off_rec = off;
+  off += align_up(sizeof(int) * (size_t)std::max(P.nnz_total, 1));
+  P.aux_base = off;
+  // Layer tables of the chunk kernels (one upload with the systems and receivers).  Last, so that a call on
+  // the z-march kernels, which has none, stays within aux_base.
+  for (int gi = 0; gi < ngroups; ++gi) {
+    const size_t e = (size_t)kLayerTab * (groups[gi].grid.npml + 1);
+    P.off_ltab32[gi] = off;
+    off += align_up(sizeof(float) * e);
+    P.off_ltab64[gi] = off;
+    off += align_up(sizeof(double) * e);
+  }
   P.aux_total = off;
   P.total = off;
 }
@@ -994,16 +993,18 @@ int upload(const wri_group* groups, int ngroups, const Plan& P, char* ws, cudaSt
   std::vector<SysDev> sys;
   std::vector<int> rec;
   build_sys(groups, ngroups, P, sys, rec);
-  std::vector<char> up(P.lin ? P.up_total : P.off_rec + sizeof(int) * rec.size());  // one copy
-  std::memcpy(up.data() + P.off_sys, sys.data(), sizeof(SysDev) * sys.size());
-  std::memcpy(up.data() + P.off_rec, rec.data(), sizeof(int) * rec.size());
+  // one copy, from the systems on: the receivers follow, then the layer tables where they are used
+  std::vector<char> up((P.lin ? P.aux_total : P.off_rec + sizeof(int) * rec.size()) - P.off_sys);
+  auto at = [&](size_t off) { return up.data() + (off - P.off_sys); };
+  std::memcpy(at(P.off_sys), sys.data(), sizeof(SysDev) * sys.size());
+  std::memcpy(at(P.off_rec), rec.data(), sizeof(int) * rec.size());
   if (P.lin) {
     std::vector<double> t;
     for (int gi = 0; gi < ngroups; ++gi) {
       layer_table(groups[gi].grid, t);
-      float* p32 = (float*)(up.data() + P.off_ltab32[gi]);
+      float* p32 = (float*)at(P.off_ltab32[gi]);
       for (size_t i = 0; i < t.size(); ++i) p32[i] = (float)t[i];
-      std::memcpy(up.data() + P.off_ltab64[gi], t.data(), sizeof(double) * t.size());
+      std::memcpy(at(P.off_ltab64[gi]), t.data(), sizeof(double) * t.size());
     }
   }
   WRI_CK(cudaMemcpyAsync(ws + P.off_sys, up.data(), up.size(), cudaMemcpyHostToDevice, st));

@@ -1,0 +1,72 @@
+"""Device-memory layout of the host code, checked without a GPU: a probe that includes the host source
+reports the byte ranges that a call touches."""
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from test_abi_cpu import W, _spec  # noqa: F401  (W: fixture)
+
+PROBE = r"""
+#include "wri_api.cu"
+
+// Ends of the byte ranges that wri_gradient_noalloc writes in its static array: out[0] without the layer
+// tables (z-march kernels: z tables, systems, receivers), out[1] with them (chunk kernels); out[2] and out[3]
+// the sizes that it compares with its limit and with the array's for the two, out[4] the array's.
+extern "C" __attribute__((visibility("default"))) void noalloc_ranges(const wri_group* groups, int ngroups,
+                                                                      long long* out) {
+  Plan P;
+  plan_aux(groups, ngroups, P);
+  size_t z = P.off_rec + sizeof(int) * (size_t)P.nnz_total;
+  z = std::max(z, P.off_sys + sizeof(SysDev) * (size_t)P.nsys_total);
+  size_t l = z;
+  for (int gi = 0; gi < ngroups; ++gi) {
+    const size_t nz = groups[gi].grid.nz, e = (size_t)kLayerTab * (groups[gi].grid.npml + 1);
+    z = std::max(z, std::max(P.off_ztab[gi] + 48 * nz, P.off_ztab64[gi] + 96 * nz));
+    l = std::max(l, std::max(P.off_ltab32[gi] + 4 * e, P.off_ltab64[gi] + 8 * e));
+  }
+  out[0] = (long long)z;
+  out[1] = (long long)std::max(l, z);
+  out[2] = (long long)P.aux_base;
+  out[3] = (long long)P.aux_total;
+  out[4] = (long long)sizeof(g_noalloc_scratch);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def probe(W, tmp_path_factory):  # noqa: F811
+    from paper_2410_18429_gb300 import build as B
+    d = tmp_path_factory.mktemp("probe")
+    src, lib = str(d / "probe.cu"), str(d / "probe.so")
+    with open(src, "w") as f:
+        f.write(PROBE)
+    objs = [os.path.join(B.BUILD, s.replace(".cu", ".o")) for s in B.SOURCES if s != "wri_api.cu"]
+    subprocess.run([B.nvcc(), "-std=c++17", "-O1", "-Xcompiler", "-fPIC,-fvisibility=hidden", *B.ARCH, "-shared",
+                    "-I", B.CSRC, "-o", lib, src, *objs], check=True, capture_output=True, text=True)
+    return C.CDLL(lib)
+
+
+@pytest.mark.parametrize("ngroups,npml", [(1, 10), (8, 20), (8, 226), (8, 300)])
+def test_noalloc_gradient_stays_inside_its_array(W, probe, ngroups, npml):  # noqa: F811
+    """The largest geometry that the limit of wri_gradient_noalloc accepts: the bytes that a call
+    without layer tables touches end within the size compared with the limit, and those of a call with them
+    within the size compared with the array's (npml = 300: 344 KB of tables, more than the array has for them)."""
+    def ranges(nnz):
+        specs = [_spec(W, nx=2 * npml + 1, ny=2 * npml + 1, nz=2 * npml + 1, npml=npml, src=np.array([0]),
+                       rec_off=np.array([0, nnz]), rec_idx=np.arange(nnz, dtype=np.int32)) for _ in range(ngroups)]
+        m = W._Marshal(specs)
+        out = (C.c_longlong * 5)()
+        probe.noalloc_ranges(m.arr, m.n, out)
+        return list(out)
+
+    limit = W.NOALLOC_SCRATCH_BYTES
+    lo, hi = 1, limit // 4 // ngroups  # receivers per group
+    while hi - lo > 1:
+        mid = (lo + hi) // 2
+        lo, hi = (mid, hi) if ranges(mid)[2] <= limit else (lo, mid)
+    plain, tables, base, total, size = ranges(lo)
+    assert limit - 256 * ngroups < base <= limit < ranges(hi)[2]
+    assert plain <= base and tables <= total and limit <= size
