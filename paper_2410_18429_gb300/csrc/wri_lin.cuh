@@ -337,11 +337,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         }
       }
     }
-    if (stop) {
-      // wait (bounded) until every copy issued into the ring has landed
-      const unsigned first = fills > (unsigned)S ? fills - S : 0u;
-      for (unsigned u = first; u < fills; ++u) mbar_wait(&full[u % S], (u / S) & 1u, T.wait_ns);
-    }
+    drain_copies<S>(full, fills, T.withhold);
     return;
   }
 

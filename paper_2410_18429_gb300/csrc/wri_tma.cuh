@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(WRI_TX* BY, MINB) k_phase_tma(const __grid_con
         // a copy never completed: record it, drain the copies this CTA issued (bounded), stop
         if (tid == 0) {
           atomicExch(T.err, 1);
-          for (int qq = q_fail; qq < issued; ++qq) mbar_wait(&bar[(uses + qq) % S], ((uses + qq) / S) & 1u, T.wait_ns);
+          for (int qq = q_fail; qq < issued; ++qq) mbar_wait(&bar[(uses + qq) % S], ((uses + qq) / S) & 1u, kWaitLimitNs);
         }
         __syncthreads();
         return;
@@ -686,7 +686,7 @@ __global__ void __launch_bounds__(16 * BY, MINB) k_phase_tma2(const __grid_const
       if (q_fail >= 0) {
         if (tid == 0) {
           atomicExch(T.err, 1);
-          for (int qq = q_fail; qq < issued; ++qq) mbar_wait(&bar[(uses + qq) % S], ((uses + qq) / S) & 1u, T.wait_ns);
+          for (int qq = q_fail; qq < issued; ++qq) mbar_wait(&bar[(uses + qq) % S], ((uses + qq) / S) & 1u, kWaitLimitNs);
         }
         __syncthreads();
         return;
@@ -768,6 +768,17 @@ __device__ __forceinline__ bool first_threads_any(bool v) {
       : "r"((uint32_t)v), "n"(NC)
       : "memory");
   return r != 0;
+}
+
+// Waits (bounded) until the last copies of a ring of S stages have landed, `fills` fills after the kernel's
+// start, and is called by the thread that issued them before it leaves, whether or not it was told to stop:
+// consumers that gave up leave without waiting, and the CTA's shared memory must not be handed on under a
+// copy.  The limit is the library's and not the caller's, which may be shorter than a copy takes.  CTA 0 skips
+// the fill that the test hook withheld.
+template <int S>
+__device__ __forceinline__ void drain_copies(uint64_t* full, unsigned fills, int withheld) {
+  for (unsigned u = fills > (unsigned)S ? fills - S : 0u; u < fills; ++u)
+    if (!(blockIdx.x == 0 && (int)u == withheld)) mbar_wait(&full[u % S], (u / S) & 1u, kWaitLimitNs);
 }
 
 __device__ __forceinline__ float2 fma_c(float c, float2 b, float2 a) {
@@ -895,11 +906,7 @@ __global__ void __launch_bounds__(16 * BY + (PW ? 32 : 0), MINB) k_phase_ws(cons
         tma_load_3d(base + L::OFF_M, &T.map[gi][TM_M], x0, y0, kq, &full[st]);
       }
     }
-    if (stop) {
-      // wait (bounded) until every copy issued into the ring has landed
-      const unsigned first = fills > (unsigned)S ? fills - S : 0u;
-      for (unsigned u = first; u < fills; ++u) mbar_wait(&full[u % S], (u / S) & 1u, T.wait_ns);
-    }
+    drain_copies<S>(full, fills, T.withhold);
     return;
   }
 
@@ -1359,9 +1366,7 @@ __global__ void __launch_bounds__(16 * BY + (PW ? 32 : 0), MINB) k_phase_ws(cons
     if (s_last) finalize<float, float, MODE, NC, CSync>(b, G, sd, sl, xonly, red, &bcast);
   }
   if (!PW && tid == 0 && s_abort) {
-    // stopped early: wait (bounded) until every copy thread 0 issued has landed
-    const unsigned first = issued > (unsigned)S ? issued - S : 0u;
-    for (unsigned u = first; u < issued; ++u) mbar_wait(&full[u % S], (u / S) & 1u, T.wait_ns);
+    drain_copies<S>(full, issued, -1);  // stopped early
   }
 }
 
