@@ -235,6 +235,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], NCW);
     }
+    mbar_init_done();
     s_abort = 0;
   }
   if constexpr (MODE == M_APPLY)

@@ -46,6 +46,10 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
 }
 
+// Makes initialised barriers visible to the copies, which signal them through the async proxy; by the thread
+// that initialised them, before the CTA's barrier.
+__device__ __forceinline__ void mbar_init_done() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
                : "memory");
@@ -178,6 +182,7 @@ __global__ void __launch_bounds__(WRI_TX* BY, MINB) k_phase_tma(const __grid_con
 
   if (tid == 0) {
     for (int s = 0; s < S; ++s) mbar_init(&bar[s], 1);
+    mbar_init_done();
     s_abort = 0;
   }
   __syncthreads();
@@ -446,6 +451,7 @@ __global__ void __launch_bounds__(16 * BY, MINB) k_phase_tma2(const __grid_const
 
   if (tid == 0) {
     for (int s = 0; s < S; ++s) mbar_init(&bar[s], 1);
+    mbar_init_done();
     s_abort = 0;
   }
   __syncthreads();
@@ -843,6 +849,7 @@ __global__ void __launch_bounds__(16 * BY + (PW ? 32 : 0), MINB) k_phase_ws(cons
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], NCW);
     }
+    mbar_init_done();
     // a copy wait of an earlier launch of this solve timed out: the solve is being stopped, and
     // this launch does nothing (read once here so that the whole CTA takes the same decision)
     s_abort = (*(volatile const int*)T.err != 0) ? 1 : 0;

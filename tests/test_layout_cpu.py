@@ -70,3 +70,18 @@ def test_noalloc_gradient_stays_inside_its_array(W, probe, ngroups, npml):  # no
     plain, tables, base, total, size = ranges(lo)
     assert limit - 256 * ngroups < base <= limit < ranges(hi)[2]
     assert plain <= base and tables <= total and limit <= size
+
+
+def test_initialised_barriers_are_fenced_before_copies_signal_them(W):  # noqa: F811
+    """Every kernel that initialises mbarriers fences them for the async proxy, by the same thread, before the
+    CTA's barrier (a CTA barrier alone does not order the two proxies; no run can be relied on to show it)."""
+    from paper_2410_18429_gb300 import build as B
+    kernels = 0
+    for name in ("wri_tma.cuh", "wri_lin.cuh"):
+        with open(os.path.join(B.CSRC, name)) as f:
+            for part in f.read().split("__global__")[1:]:
+                if "mbar_init(" in part:
+                    kernels += 1
+                    after = part[part.rindex("mbar_init("):]
+                    assert 0 <= after.find("mbar_init_done();") < after.index("__syncthreads();"), (name, part[:120])
+    assert kernels == 4
