@@ -1167,8 +1167,9 @@ int solve_refined(const wri_group* groups, int ngroups, const wri_solve_opts* o,
     } else {
       WRI_CK(stencil_pass(P, 4, 4, M_SH, r, w, st));
     }
-    WRI_CK(cudaMemcpyAsync(slot, inner.remaining, sizeof(int), cudaMemcpyDeviceToHost, st));
+    WRI_CK(cudaMemcpyAsync(slot, inner.remaining, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
     WRI_CK(cudaStreamSynchronize(st));
+    if (slot[1] != 0) return WRI_ECUDA;                            // a bounded copy wait timed out
     if (*slot > 0) {
       Batch in = inner;
       for (int gi = 0; gi < P.ngroups; ++gi) in.g[gi].gvec = nullptr;  // r64 = 0: no g'
@@ -1183,7 +1184,7 @@ int solve_refined(const wri_group* groups, int ngroups, const wri_solve_opts* o,
     first_outer = 1;
   }
   for (int outer_k = first_outer;; ++outer_k) {
-    WRI_CK(cudaMemsetAsync(outer.remaining, 0, 3 * sizeof(int), st));
+    WRI_CK(cudaMemsetAsync(outer.remaining, 0, sizeof(int), st));  // the error flag beside it stays
     Batch r = outer;
     r.outer = outer_k;
     r.flavor = SH_REFINE;

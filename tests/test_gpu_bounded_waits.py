@@ -29,3 +29,31 @@ def test_time_out_of_items_shorter_than_the_ring(W, dtype, cfg, limit_us):  # no
         it, _, _ = W.solve([again], W.make_opts(**kw))
         assert it.cpu().tolist() == [k] * 3
         assert torch.equal(again.u, ref.u)
+
+
+def test_time_out_of_a_refined_solve_in_its_first_pass(W):  # noqa: F811
+    """A general right-hand side under refinement, one system, 24 x 43 x 43: the complex64 pass that forms S^H b
+    has two planes per work item and the FP64 passes one, so of all passes before the first iteration only
+    this one reaches the third fill of block 0.  Its system never starts, and the call must not report it as
+    solved: WRI_ECUDA, and the next solve is unharmed."""
+    G = case(nphys=(18, 37, 37), npml=3, nsys=1)
+    g = torch.Generator().manual_seed(3)
+    q = torch.randn(1, G.spec.n, dtype=torch.complex64, generator=g)
+    kw = dict(tol=1e-3, max_iter=12, dtype=0, max_refine=1, refine_tol=1e-12, inner_tol=1e-3)
+
+    def spec():
+        s = _spec(W, G, 0)
+        s.q = q.cuda()
+        s.u64 = torch.zeros(1, G.spec.n, dtype=torch.complex128, device="cuda")
+        return s
+
+    ref = spec()
+    it, _, _ = W.solve([ref], W.make_opts(**kw))
+    assert it.cpu().tolist() == [12]
+    with pytest.raises(W.WriError) as e:
+        W.solve([spec()], W.make_opts(wait_limit_us=1000, test_withhold=3, **kw))
+    assert e.value.code == W.ECUDA
+    torch.cuda.synchronize()
+    again = spec()
+    W.solve([again], W.make_opts(**kw))
+    assert torch.equal(again.u64, ref.u64)
