@@ -73,10 +73,14 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
 
 __device__ __forceinline__ float fma_r(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_r(double a, double b, double c) { return __fma_rn(a, b, c); }
-// acc + a b (complex a), acc + s b (real s)
+// acc + a b and a b (complex a), acc + s b (real s)
 template <typename C>
 __device__ __forceinline__ C cfma(C a, C b, C acc) {
   return mkc(fma_r(a.x, b.x, fma_r(-a.y, b.y, acc.x)), fma_r(a.x, b.y, fma_r(a.y, b.x, acc.y)));
+}
+template <typename C>
+__device__ __forceinline__ C cmul(C a, C b) {
+  return mkc(fma_r(a.x, b.x, -(a.y * b.y)), fma_r(a.x, b.y, a.y * b.x));
 }
 template <typename R, typename C>
 __device__ __forceinline__ C rfma(R s, C b, C acc) {
@@ -210,8 +214,11 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
   constexpr bool NORM = (MODE == M_P1 || MODE == M_P2 || MODE == M_SH);
   constexpr int NCW = NC / 32;
   constexpr bool GRAD = MODE == M_GRAD;
-  // complex64 forms the stencil from differences to the node, which are exact or nearly so for a resolved
-  // field; complex128 from the values, with the diagonal in one coefficient (up to 12 FP64 instructions less)
+  // The stencil is formed from differences to the node, which are exact or nearly so for a resolved field, so
+  // that the rounding of a coefficient acts on a difference.  complex128 takes the unstretched axes together,
+  // as the sum of their neighbours minus 6 (or 4, 2) u: fewer FP64 instructions.  The diagonal in one coefficient
+  // would save 2 (interior) to 8 (x and y layer) of 17 to 37 more (A^H on 81^3 x 9 297 -> 264 us), but its
+  // error is up to four times as large (A u of plane waves, 116 x 60 x 80 with 10 cells: 4.0e-15 against 1.1e-15).
   constexpr bool DIFF = sizeof(R) == 4;
   // complex64: the first step of an item finishes a plane below it all the same (no check in the loop) and
   // its result is overwritten; complex128 saves the FP64 instructions
@@ -422,9 +429,8 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
 
     // coefficients of the thread's nodes (only warps with a stretched or boundary node)
     constexpr int NY = PAIR ? 1 : NPT;  // rows of the thread's nodes (a pair lies in one row)
-    C am[NPT], ap[NPT], bm[NY], bp[NY], cc[NPT];
+    C am[NPT], ap[NPT], bm[NY], bp[NY];
     R sx_[NPT], sy_[NY];
-    R cc0[NPT];   // Re cc with the z axis unstretched
     R w2xy[NPT];  // gradient: |s_x s_y|^2
 
     double accd = 0.0;
@@ -604,18 +610,16 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
           bp[r] = cy_.ap;
           sy_[r] = cy_.im;
         }
-        cc[r] = cx_.a0 + cy_.a0;
-        cc0[r] = cc[r].x - R(2) * ih2;
         w2xy[r] = fma_r(cx_.im, cx_.im, R(1)) * fma_r(cy_.im, cy_.im, R(1));
         sx_[r] = cx_.im;
       }
     }
     // One plane of the item: its F, the z + 1 term of plane k - 1, and its own stencil without that term.
     // gen_c: 1 the x coefficients are general, 2 those of x and y; zg_c: plane k lies in a z layer.  XO (FP64)
-    // has a kind of its own for x alone, with the same roundings and 6 FP64 instructions of 31 less: rows of 116
-    // nodes leave half of the warps with an x layer and most of these outside the y layers.  A^H on 81^3 x 9 285
-    // -> 264 us, gradient on 148^3 x 16 2883 -> 2766.  The phases take it for items of 8 planes and more: 148^3 x 1
-    // 521 -> 505 us per iteration, 81^3 x 9 835 -> 804, but 36^3 x 1, with items of 3 planes, 38.8 -> 40.1.
+    // has a kind of its own for x alone, with 10 FP64 instructions of 37 less (the phases 6: their kernels with
+    // and without it round alike): of the warps of 81^3 two thirds have an x layer, of 148^3 a third, most of
+    // them outside the y layers.  The phases take it for items of 8 planes and more: with items of 3 planes
+    // (36^3 x 1) the additional loops cost 3 % of the iteration, with 17 to 50 (81^3 x 9, 148^3 x 1) they gave 3 to 4 %.
     auto step = [&](auto gen_c, auto zg_c, int k) -> bool {
       constexpr bool GEN = decltype(gen_c)::value > 0, GY = decltype(gen_c)::value == 2, ZG = decltype(zg_c)::value;
       if (!wait()) return false;
@@ -682,8 +686,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         C t[NPT];
 #pragma unroll
         for (int r = 0; r < NPT; ++r) {
-          const C d = DIFF ? v[r] - fc[r] : v[r];
-          t[r] = ZG ? cfma(hz, d, q[r]) : rfma(ih2, d, q[r]);
+          t[r] = ZG ? cfma(hz, v[r] - fc[r], q[r]) : rfma(ih2, DIFF ? v[r] - fc[r] : v[r], q[r]);
           if (GEN && !GRAD) t[r] = smul(sx_[r], t[r]);
           if (GY && !GRAD) t[r] = smul(sy_[PAIR ? 0 : r], t[r]);
         }
@@ -719,33 +722,44 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
           ym[r] = ym[r] - v[r];
           yp[r] = yp[r] - v[r];
         }
-        const C zm = DIFF ? fc[r] - v[r] : fc[r];
-        C acc;  // the diagonal, then the neighbours
+        const R c = om2 * mk[r];
+        C acc;
         if (DIFF) {
-          const R c = om2 * mk[r];
+          const C zm = fc[r] - v[r];
           acc = mkc(c * v[r].x, c * v[r].y);
-        } else if (GEN) {
-          const C c = ZG ? mkc(fma_r(om2, mk[r], cc[r].x) + cz.a0.x, cc[r].y + cz.a0.y)
-                         : mkc(fma_r(om2, mk[r], cc0[r]), cc[r].y);
-          acc = mkc(fma_r(c.x, v[r].x, -c.y * v[r].y), fma_r(c.x, v[r].y, c.y * v[r].x));
-        } else if (ZG) {
-          const C c = mkc(fma_r(om2, mk[r], R(-4) * ih2) + cz.a0.x, cz.a0.y);
-          acc = mkc(fma_r(c.x, v[r].x, -c.y * v[r].y), fma_r(c.x, v[r].y, c.y * v[r].x));
+          if (GEN) {
+            acc = cfma(am[r], l[r], acc);
+            acc = cfma(ap[r], rgt[r], acc);
+            acc = GY ? cfma(bm[PAIR ? 0 : r], ym[r], acc) : rfma(ih2, ym[r], acc);
+            acc = GY ? cfma(bp[PAIR ? 0 : r], yp[r], acc) : rfma(ih2, yp[r], acc);
+            acc = ZG ? cfma(cz.am, zm, acc) : rfma(ih2, zm, acc);
+          } else {
+            C sum = (l[r] + rgt[r]) + (ym[r] + yp[r]);
+            if (!ZG) sum = sum + zm;
+            acc = rfma(ih2, sum, acc);
+            if (ZG) acc = cfma(cz.am, zm, acc);
+          }
         } else {
-          const R c = fma_r(om2, mk[r], R(-6) * ih2);
-          acc = mkc(c * v[r].x, c * v[r].y);
-        }
-        if (GEN) {
-          acc = cfma(am[r], l[r], acc);
-          acc = cfma(ap[r], rgt[r], acc);
-          acc = GY ? cfma(bm[PAIR ? 0 : r], ym[r], acc) : rfma(ih2, ym[r], acc);
-          acc = GY ? cfma(bp[PAIR ? 0 : r], yp[r], acc) : rfma(ih2, yp[r], acc);
-          acc = ZG ? cfma(cz.am, zm, acc) : rfma(ih2, zm, acc);
-        } else {
-          C sum = (l[r] + rgt[r]) + (ym[r] + yp[r]);
-          if (!ZG) sum = sum + zm;
-          acc = rfma(ih2, sum, acc);
-          if (ZG) acc = cfma(cz.am, zm, acc);
+          // In a z layer every term but omega^2 m u is a difference: these first, then that one in one rounding.
+          // The phases have kernels with and without the loops for x alone (XO), which have to round alike.
+          constexpr bool YD = GY || (GEN && HASB);
+          constexpr int axes = 6 - (GEN ? 2 : 0) - (YD ? 2 : 0) - (ZG ? 2 : 0);
+          acc = ZG ? cmul(cz.am, fc[r] - v[r]) : mkc(c * v[r].x, c * v[r].y);
+          C sum = fc[r];  // neighbours on the unstretched axes but for z + 1
+          if (GEN) {
+            acc = cfma(am[r], l[r] - v[r], acc);
+            acc = cfma(ap[r], rgt[r] - v[r], acc);
+          }
+          if (YD) {
+            acc = GY ? cfma(bm[PAIR ? 0 : r], ym[r] - v[r], acc) : rfma(ih2, ym[r] - v[r], acc);
+            acc = GY ? cfma(bp[PAIR ? 0 : r], yp[r] - v[r], acc) : rfma(ih2, yp[r] - v[r], acc);
+          } else {
+            sum = ym[r] + yp[r];
+            if (!GEN) sum = (l[r] + rgt[r]) + sum;
+            if (!ZG) sum = sum + fc[r];
+          }
+          if (axes > 0) acc = rfma(ih2, rfma(R(-axes), v[r], sum), acc);
+          if (ZG) acc = rfma(c, v[r], acc);
         }
         q[r] = ZG && !GRAD ? smul(cz.im, acc) : acc;
         fc[r] = v[r];
@@ -765,11 +779,20 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
       for (; k < za; ++k)
         if (!step(gen_c, std::true_type(), k)) return false;
       const int kl = k;
+      // complex128: the z + 1 term of an interior plane lacks -u / h^2, which its q holds
+      if (!DIFF && k < zb) {
+#pragma unroll
+        for (int r = 0; r < NPT; ++r) q[r] = rfma(-ih2, fc[r], q[r]);
+      }
       for (; k < zb; ++k)
         if (!step(gen_c, std::false_type(), k)) return false;
       if (k > kl) {  // the pending plane is an interior one
         hz = mkc(ih2, R(0));
         hs = R(0);
+        if (!DIFF) {
+#pragma unroll
+          for (int r = 0; r < NPT; ++r) q[r] = rfma(ih2, fc[r], q[r]);
+        }
       }
       for (; k < z1; ++k)
         if (!step(gen_c, std::true_type(), k)) return false;
@@ -835,7 +858,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
           C t[NPT];
 #pragma unroll
           for (int r = 0; r < NPT; ++r) {
-            t[r] = cfma(hz, DIFF ? v[r] - fc[r] : v[r], q[r]);
+            t[r] = cfma(hz, v[r] - fc[r], q[r]);
             if (gen && !GRAD) t[r] = smul(sy_[PAIR ? 0 : r], smul(sx_[r], t[r]));
           }
           if constexpr (GRAD) accum(z1 - 1, t, gen, true);

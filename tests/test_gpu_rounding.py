@@ -1,0 +1,47 @@
+"""Rounding of the FP64 stencils: how exactly they see a field without curvature."""
+import numpy as np
+import pytest
+
+import oracle as O
+from test_gpu_parity import W, _spec  # noqa: F401  (W: fixture)
+from wri_cases import case
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+U = 2.0 ** -53
+
+
+@pytest.mark.parametrize("nphys,npml,nsys", [((41, 23, 30), 5, 2), ((108, 40, 28), 4, 1), ((30, 9, 8), 0, 2),
+                                             ((40, 40, 70), 3, 40)])
+def test_constant_field_fp64(W, nphys, npml, nsys):  # noqa: F811
+    """A u of a constant field is s_x s_y s_z omega^2 m u off the faces: every difference vanishes, and about two
+    roundings of terms as large as u / h^2 are left (the sum of neighbours minus 6 u, and the z + 1 neighbour that is
+    added last).  h = 8 makes 1 / h^2 exact, and 1 Hz makes omega^2 m a thousandth of it, so a rounding of the
+    diagonal -6 / h^2 or of its product with u (up to 4 / h^2 each) exceeds the bound.  A, A^H and the gradient,
+    whose residual is the same stencil; u = 1 + i / 2, so the sums themselves are exact."""
+    G = case(nphys=nphys, npml=npml, h=8.0, freq=1.0, nsys=nsys, with_data=False)
+    nz, ny, nx = G.spec.shape
+    m = 1.0 / np.random.default_rng(5).uniform(1500.0, 3300.0, G.spec.n) ** 2
+    spec = _spec(W, G, 1)
+    spec.m = torch.from_numpy(m).cuda()
+    u = np.full((nsys, G.spec.n), 1.0 + 0.5j)
+    om2, ih2 = G.omega ** 2, 1.0 / 64.0
+    w = O.stretch_weight(G.spec.shape, 8.0, G.omega, npml, G.v_max, G.pml_R)
+    inner = np.zeros(G.spec.shape, bool)
+    inner[1:-1, 1:-1, 1:-1] = True
+    inner = inner.ravel()
+    ut = torch.from_numpy(u).cuda()
+    for adjoint in (False, True):
+        y = W.apply_A(spec, ut, adjoint=adjoint).cpu().numpy()
+        ref = (w.conj() if adjoint else w) * (om2 * m * u[0])
+        bound = U * np.abs(w) * abs(u[0, 0]) * (2.5 * ih2 + 16 * om2 * m)
+        err = np.abs(y - ref)[:, inner] / bound[inner]
+        assert err.max() <= 1.0, (adjoint, err.max())
+    spec.u = ut
+    spec.d = torch.zeros(len(G.rec_idx), dtype=torch.complex128, device="cuda")
+    g, _ = W.gradient([spec], 1, torch.zeros(nsys, dtype=torch.complex128, device="cuda"))
+    g = g[0].cpu().numpy().ravel()
+    ref = nsys * om2 * np.abs(w) ** 2 * om2 * m * abs(u[0, 0]) ** 2
+    bound = U * nsys * om2 * np.abs(w) ** 2 * abs(u[0, 0]) ** 2 * (2.5 * ih2 + (16 + nsys) * om2 * m)
+    err = np.abs(g - ref)[inner] / bound[inner]
+    assert err.max() <= 1.0, err.max()
