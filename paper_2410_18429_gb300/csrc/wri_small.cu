@@ -132,7 +132,8 @@ cudaError_t launch_tv(const double* m, int nx, int ny, int nz, double beta, doub
   zs = zs > nz / 8 ? nz / 8 : zs;
   zs = zs < 1 ? 1 : zs;
   const int zc = (nz + zs - 1) / zs;
-  k_tv<<<dim3(bx, by, (nz + zc - 1) / zc), dim3(kTvX, kTvY), 0, st>>>(m, nx, ny, nz, zc, beta, gamma, tv, grad);
+  const long long blocks = ((long long)bx * by * ((nz + zc - 1) / zc) + kTvCluster - 1) / kTvCluster * kTvCluster;
+  k_tv<<<(unsigned)blocks, dim3(kTvX, kTvY), 0, st>>>(m, nx, ny, nz, bx, by, zc, beta, gamma, tv, grad);
   return cudaGetLastError();
 }
 

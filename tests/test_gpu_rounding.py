@@ -1,4 +1,6 @@
-"""Rounding of the FP64 stencils: how exactly they see a field without curvature."""
+"""Rounding of the FP64 kernels where every term of a kind is equal: flat fields and models."""
+import math
+
 import numpy as np
 import pytest
 
@@ -45,3 +47,21 @@ def test_constant_field_fp64(W, nphys, npml, nsys):  # noqa: F811
     bound = U * nsys * om2 * np.abs(w) ** 2 * abs(u[0, 0]) ** 2 * (2.5 * ih2 + (16 + nsys) * om2 * m)
     err = np.abs(g - ref)[inner] / bound[inner]
     assert err.max() <= 1.0, err.max()
+
+
+@pytest.mark.parametrize("slope", [925311, 571099, 616179])
+def test_total_variation_of_equal_cells(W, slope):  # noqa: F811
+    """A model with one slope in x, y and z (exact in FP64): all cells and with them nearly all block sums are
+    equal, so their additions to the result may all round the same way.  128^3 has 720 blocks; 180 additions
+    are off by half a unit of the growing sum each at the most, 90 U in all, and 10 U are left for the sums
+    inside.  (An addition per block is off by 115 to 140 U for these slopes.)"""
+    n, a, beta = 128, slope * 2.0 ** -50, 1e-9
+    i = np.arange(n, dtype=np.float64)
+    m = a * (i[:, None, None] + i[None, :, None] + i[None, None, :])
+    last = np.ones(n)
+    last[-1] = 0.0
+    q = np.sqrt(a * a * (last[:, None, None] + last[None, :, None] + last[None, None, :]) + beta * beta)
+    ref = math.fsum(q.ravel())
+    spec = W.GroupSpec(n, n, n, 0, 10.0, 60.0, 3000.0, None, None, None, None, None, 1.0, None)
+    tv, _ = W.tv(spec, torch.from_numpy(m).cuda(), beta)
+    assert abs(tv.item() - ref) <= 100 * U * ref, (tv.item() - ref) / ref / U
