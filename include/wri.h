@@ -132,8 +132,8 @@ typedef struct {
   int32_t zsplit;      /* z-chunks per tile column (0 = chosen from the batch size) */
   int32_t kernel;      /* 0 = automatic (the chunk kernels, as configuration 24), 1 = z-march
                           kernels only, 2 + c = configuration c (0..24).  18, 22 and 24 are the
-                          chunk kernels (any x extent, both dtypes; 18 and 22 update the iterate
-                          every second iteration, 24 every fourth in complex64), the others the
+                          chunk kernels (any x extent, both dtypes; 18 updates the iterate in every
+                          iteration, 22 every second, 24 every fourth in complex64), the others the
                           TMA box phases (9..24 warp-specialised; 23 updates the iterate every
                           second iteration); see wri_autotune.  An explicit `tile` with a batch
                           the boxes cannot take runs on the z-march kernels. */

@@ -330,8 +330,8 @@ bool host_loop_forced() {
   return forced;
 }
 
-// TMA configurations whose phases are the chunk kernels: 18 and 22 (two direction slots, x updated every
-// second iteration) and 24, the automatic choice (four slots, every fourth iteration).  Complex128 batches
+// TMA configurations whose phases are the chunk kernels: 18 (x updated in every iteration), 22 (every second, two
+// direction slots) and 24, the automatic choice (every fourth, four slots).  Complex128 batches
 // and x extents that are not multiples of 4, which the TMA boxes cannot take, run on them too unless
 // z-march kernels or a z-march tile are asked for.  Microseconds per system and iteration against the
 // boxes of configuration 9 (and of 24): 148^3 x 32 systems 41.7 (58.6, 52.5), 116^3 x 32 20.9 (31.4, 28.7),
@@ -374,7 +374,7 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
   if (P.lin) {
     // complex128 keeps two direction slots: the same bytes per iteration as an update in every one
     P.pslots = (o->dtype == WRI_C64 && cfg == 24) ? 4 : 2;
-    P.xsteps = P.pslots;
+    P.xsteps = cfg == 18 ? 1 : P.pslots;
   } else if (boxes) {
     P.tma_cfg = o->kernel >= 2 ? o->kernel - 2 : kBoxTmaCfg;
     // the refinement's inner phase 2 adds S^H r64, which only the warp-specialised kernels do

@@ -230,8 +230,9 @@ struct Batch {
                         // 3 = blocks of sblock systems, tiles in order, systems fastest in a block
   int sblock;           // systems per block of order 3
   int pair;             // chunk kernels, complex64: a thread's two nodes are adjacent (nx even, arrays aligned)
-  int xsteps;           // m: phase 1 adds the steps of m iterations to x every m-th iteration (m = 2, 4:
-                        // the warp-specialised grouped-update configurations; 0 or 1: every iteration)
+  int xsteps;           // m: the steps of m iterations are added to x every m-th iteration (m = 2, 4: the
+                        // grouped-update configurations; 0 or 1: every iteration), by phase 1 of the boxes
+                        // and by k_xupdate of the chunk kernels
   double tol;           // tolerance of a cold-start solve
   double refine_tol, inner_tol;
   int outer, max_refine, warm;

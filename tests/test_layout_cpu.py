@@ -33,6 +33,16 @@ extern "C" __attribute__((visibility("default"))) void noalloc_ranges(const wri_
   out[3] = (long long)P.aux_total;
   out[4] = (long long)sizeof(g_noalloc_scratch);
 }
+
+// Of a solve's plan: chunk kernels or not, iterations per iterate update, direction slots.
+extern "C" __attribute__((visibility("default"))) void plan_of(const wri_group* groups, int ngroups,
+                                                               const wri_solve_opts* opts, long long* out) {
+  Plan P;
+  plan_solve(groups, ngroups, opts, P);
+  out[0] = P.lin ? 1 : 0;
+  out[1] = P.xsteps;
+  out[2] = P.pslots;
+}
 """
 
 
@@ -85,3 +95,20 @@ def test_initialised_barriers_are_fenced_before_copies_signal_them(W):  # noqa: 
                     after = part[part.rindex("mbar_init("):]
                     assert 0 <= after.find("mbar_init_done();") < after.index("__syncthreads();"), (name, part[:120])
     assert kernels == 4
+
+
+def _plan(W, probe, spec, **kw):  # noqa: F811
+    m = W._Marshal([spec])
+    out = (C.c_longlong * 3)()
+    probe.plan_of(m.arr, m.n, C.byref(W.make_opts(**kw)), out)
+    return tuple(out)
+
+
+@pytest.mark.parametrize("dtype,grouped", [(0, 4), (1, 2)])
+def test_iterations_per_iterate_update_of_the_chunk_configurations(W, probe, dtype, grouped):  # noqa: F811
+    """18: every iteration (what the grouped configurations are compared with, bit for bit); 22: every second; 24 and
+    the automatic choice: as many as there are direction slots."""
+    for cfg, m in ((18, 1), (22, 2), (24, grouped)):
+        lin, xsteps, slots = _plan(W, probe, _spec(W), dtype=dtype, kernel=W.KERNEL_TMA(cfg))
+        assert (lin, xsteps) == (1, m) and slots == max(2, m), cfg
+    assert _plan(W, probe, _spec(W), dtype=dtype, kernel=0)[:2] == (1, grouped)
