@@ -133,7 +133,8 @@ typedef struct {
   int32_t kernel;      /* 0 = automatic (the chunk kernels, as configuration 24), 1 = z-march
                           kernels only, 2 + c = configuration c (0..24).  18, 22 and 24 are the
                           chunk kernels (any x extent, both dtypes; 18 updates the iterate in every
-                          iteration, 22 every second, 24 every fourth in complex64), the others the
+                          iteration, 22 every second, 24 every fourth in complex64 where the
+                          workspace has the directions for it), the others the
                           TMA box phases (9..24 warp-specialised; 23 updates the iterate every
                           second iteration); see wri_autotune.  An explicit `tile` with a batch
                           the boxes cannot take runs on the z-march kernels. */
@@ -167,8 +168,8 @@ WRI_API int wri_apply_AH(const wri_grid* grid, int dtype, const void* m, int nsy
 
 /* Bytes of device workspace wri_solve_batch needs for these groups and options
  * (0 on invalid arguments).  The workspace must be 256-byte aligned.  With opts->kernel = 0
- * (automatic) it also covers the four search-direction vectors per system of configuration
- * 24, so that a workspace sized before wri_autotune fits every configuration it may choose. */
+ * (automatic) and a batch that wri_autotune takes it also covers the four search-direction vectors
+ * per system of configuration 24, so that a workspace sized before tuning fits every choice. */
 WRI_API size_t wri_workspace_size(const wri_group* groups, int ngroups, const wri_solve_opts* opts);
 
 /* Solve every system of every group (the LSQR/CG solve of Eq. SimpObj, Algorithm 1

@@ -281,6 +281,7 @@ struct Plan {
   long long nitems64 = 0;
   size_t v_r1[WRI_MAXG][2], v_p[WRI_MAXG][4], v_s[WRI_MAXG], v_t1[WRI_MAXG];
   int pslots = 2;  // search-direction slots: 4 when the phases may update x every fourth iteration
+  bool ring_in_x64 = false;  // slots 2 and 3 in the place of the refinement's unused FP64 solution (v_x64)
   size_t v_x32[WRI_MAXG], v_x64[WRI_MAXG], v_r64[WRI_MAXG], v_q64[WRI_MAXG], v_g32[WRI_MAXG], v_rmap[WRI_MAXG];
   size_t off_ztab[WRI_MAXG], off_ztab64[WRI_MAXG];  // z-coefficient tables (FP32, FP64) per group
   size_t off_rmask[WRI_MAXG], off_rcol[WRI_MAXG], rmask_bytes[WRI_MAXG], rcol_bytes[WRI_MAXG];
@@ -372,8 +373,13 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
     P.lin = P.lin && lin_smem(probe, (o->dtype == WRI_C128 || P.ir) ? 8 : 4, M_P1) <= (size_t)kLinMaxSmem;
   }
   if (P.lin) {
-    // complex128 keeps two direction slots: the same bytes per iteration as an update in every one
-    P.pslots = (o->dtype == WRI_C64 && cfg == 24) ? 4 : 2;
+    // complex128 keeps two direction slots: the same bytes per iteration as an update in every one.  So do complex64
+    // batches the boxes cannot take, whose workspace has no room for four; a refined solve with an FP64 array of
+    // the caller's for every group leaves that of its own master (two complex64 vectors) for the other two.
+    bool wide_out = P.ir;
+    for (int gi = 0; gi < ngroups; ++gi) wide_out = wide_out && groups[gi].u64;
+    P.ring_in_x64 = !boxes && wide_out;
+    P.pslots = (o->dtype == WRI_C64 && cfg == 24 && (boxes || wide_out)) ? 4 : 2;
     P.xsteps = cfg == 18 ? 1 : P.pslots;
   } else if (boxes) {
     P.tma_cfg = o->kernel >= 2 ? o->kernel - 2 : kBoxTmaCfg;
@@ -494,7 +500,7 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
     P.v_p[gi][0] = off; off += vb;
     P.v_p[gi][1] = off; off += vb;
     P.v_p[gi][2] = P.v_p[gi][3] = 0;
-    if (P.pslots == 4) {
+    if (P.pslots == 4 && !P.ring_in_x64) {
       P.v_p[gi][2] = off; off += vb;
       P.v_p[gi][3] = off; off += vb;
     }
@@ -509,6 +515,10 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
       P.v_q64[gi] = off; off += align_up(16 * nn);
       P.v_g32[gi] = off; off += align_up(8 * nn);
       P.v_rmap[gi] = off; off += align_up(4 * nn);
+      if (P.pslots == 4 && P.ring_in_x64) {
+        P.v_p[gi][2] = P.v_x64[gi];
+        P.v_p[gi][3] = P.v_x64[gi] + 8 * nn;
+      }
     }
   }
   P.total = off;

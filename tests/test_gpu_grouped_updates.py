@@ -31,3 +31,21 @@ def test_grouped_updates_equal_single_updates(W, nphys, dtype):  # noqa: F811
             for a, b in zip(run(cfg, **kw), single):
                 assert np.array_equal(a, b), (cfg, kw)
     assert single[3].tolist() == [W.SYS_OK] * 3 and len(set((single[1] % 4).tolist())) > 1, single[1]
+
+
+def test_grouped_updates_of_refined_solves_on_an_odd_extent(W):  # noqa: F811
+    """With an FP64 array of the caller's the slots of two of the four directions lie in the workspace of the
+    refinement's own FP64 solution, which is then unused: the same wavefields, bit for bit, as with two slots in
+    the solve without such an array and as with single updates, over several outer steps."""
+    G = case(nphys=(29, 12, 11), npml=4, nsys=3, seed=12)
+    out = []
+    for cfg, wide in ((18, True), (24, True), (22, False), (24, False)):
+        spec = _spec(W, G, 0)
+        if wide:
+            spec.u64 = torch.zeros(G.nsys, G.spec.n, dtype=torch.complex128, device="cuda")
+        it, rr, st = W.solve([spec], W.make_opts(dtype=0, tol=1e-3, max_iter=37, max_refine=3, refine_tol=1e-12,
+                                                 inner_tol=1e-12, kernel=W.KERNEL_TMA(cfg)))
+        assert it.cpu().tolist() == [3 * 37] * 3, it
+        out.append([spec.u.clone(), rr, it])
+    for o in out[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(o, out[0]))
