@@ -917,6 +917,8 @@ int run_loop(const Plan& P, const Batch& b1_in, const Batch& b2_in, int mode2, i
   const int xs = P.lin ? P.xsteps : use_tma ? tma_config_xsteps(P.tma_cfg) : 1;
   if (xs == 4 && !b1.g[0].p[2]) return WRI_EINVAL;
   b1.xsteps = b2.xsteps = xs;
+  // the iterations use no FP64 solution: its address (the caller's array, where there is one) is no part of the graph
+  for (int gi = 0; gi < P.ngroups; ++gi) b1.g[gi].x64 = b2.g[gi].x64 = nullptr;
   // chunk kernels: the iterate-update pass follows every xs-th iteration of a body and its last one, so a
   // body holds a multiple of xs iterations or all of them
   if (P.lin) K = K >= max_iter ? max_iter : (K + xs - 1) / xs * xs;
