@@ -26,6 +26,7 @@ import statistics
 import subprocess
 import sys
 import time
+import types
 
 ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
@@ -33,8 +34,8 @@ sys.path.insert(0, ROOT)
 METRIC = "WRI gradient src·freq/s at 128³ (GPt·iter/s, % HBM roofline) vs plain path"
 UNIT = "src·freq/s"
 BYTES_PER_NODE_SYS = 80.0  # one CGLS iteration, per node and system: phase 1 48 B + phase 2 32 B (c64)
-# grouped-update configurations: x read and written every m-th iteration, with m - 1 extra p reads
-# then: phase 1 (m 32 + 16 + 8 (m - 1)) / m = 44 B (m = 2) or 42 B (m = 4)
+# grouped-update configurations (18 updates x in every iteration): x read and written every m-th iteration,
+# with m - 1 extra p reads then: phase 1 (m 32 + 16 + 8 (m - 1)) / m = 44 B (m = 2) or 42 B (m = 4)
 XSTEPS = {22: 2, 23: 2, 24: 4}
 CHUNK_CONFIGS = (18, 22, 24)  # the chunk kernels; 24 is the automatic choice
 CHUNK_DEFAULT = 24
@@ -97,6 +98,12 @@ def bytes_per_node_sys(opts):
     k = int(opts.kernel)
     m = XSTEPS.get(k - 2, 1) if k >= 2 else 1
     return BYTES_PER_NODE_SYS - 16.0 + (16.0 + 8.0 * (m - 1)) / m
+
+
+def algorithmic_bytes(opts):
+    """The same for the kernels that run under opts: the automatic choice runs as its configuration."""
+    k = int(opts.kernel)
+    return bytes_per_node_sys(types.SimpleNamespace(kernel=k if k else 2 + CHUNK_DEFAULT))
 
 
 def phase_kernel_name(opts):
@@ -303,8 +310,7 @@ def run_group_sweep(args):
         ta = min(timed(20) for _ in range(2))
         tb = min(timed(80) for _ in range(2))
         t_iter = (tb - ta) / 60.0
-        eff = base if base.kernel else wri.make_opts(kernel=2 + CHUNK_DEFAULT)  # what the automatic choice runs
-        alg = n * (bytes_per_node_sys(eff) * nb + MODEL_BYTES)
+        alg = n * (algorithmic_bytes(base) * nb + MODEL_BYTES)
         print(json.dumps({"group_sweep": nb, "grid": f"{g0.spec.nx}x{g0.spec.ny}x{g0.spec.nz}",
                           "ms_per_iter": t_iter * 1e3, "us_per_system_iter": t_iter / nb * 1e6,
                           "gpt_iter_s": nb * n / t_iter / 1e9, "hbm_gbs": alg / t_iter / 1e9,
@@ -603,7 +609,7 @@ def main():
     t_hi = min(timed_solve(iters_done) for _ in range(2))
     t_lo = min(timed_solve(lo_iters) for _ in range(2))
     t_iter = (t_hi - t_lo) / (iters_done - lo_iters)
-    alg_bytes = node_sys * bytes_per_node_sys(opts) + sum(g.spec.n for g in groups) * MODEL_BYTES
+    alg_bytes = node_sys * algorithmic_bytes(opts) + sum(g.spec.n for g in groups) * MODEL_BYTES
     peaks = {}
     try:
         peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
