@@ -38,6 +38,10 @@ constexpr int kDefaultOrder = 6;
 constexpr int kDefaultPromotion = 2;
 constexpr int kGradPlanes = 16;  // planes of a z-chunk of the gradient, at most (its sums: 32 KB of shared memory)
 constexpr size_t kAlign = 256;
+// Bytes that direction slots 2 and 3 may take in a batch the boxes cannot take, which had two slots before it ran on
+// the chunk kernels: 0.4 % of the device, so that a batch near its size still fits (81^3 x 9 takes 77 MB, and
+// 14.0 us per system and iteration with four slots, 14.7 with two; the traffic of large batches differs by 3 %).
+constexpr double kRingRoom = 1 << 30;
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
@@ -281,7 +285,6 @@ struct Plan {
   long long nitems64 = 0;
   size_t v_r1[WRI_MAXG][2], v_p[WRI_MAXG][4], v_s[WRI_MAXG], v_t1[WRI_MAXG];
   int pslots = 2;  // search-direction slots: 4 when the phases may update x every fourth iteration
-  bool ring_in_x64 = false;  // slots 2 and 3 in the place of the refinement's unused FP64 solution (v_x64)
   size_t v_x32[WRI_MAXG], v_x64[WRI_MAXG], v_r64[WRI_MAXG], v_q64[WRI_MAXG], v_g32[WRI_MAXG], v_rmap[WRI_MAXG];
   size_t off_ztab[WRI_MAXG], off_ztab64[WRI_MAXG];  // z-coefficient tables (FP32, FP64) per group
   size_t off_rmask[WRI_MAXG], off_rcol[WRI_MAXG], rmask_bytes[WRI_MAXG], rcol_bytes[WRI_MAXG];
@@ -373,13 +376,11 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
     P.lin = P.lin && lin_smem(probe, (o->dtype == WRI_C128 || P.ir) ? 8 : 4, M_P1) <= (size_t)kLinMaxSmem;
   }
   if (P.lin) {
-    // complex128 keeps two direction slots: the same bytes per iteration as an update in every one.  So do complex64
-    // batches the boxes cannot take, whose workspace has no room for four; a refined solve with an FP64 array of
-    // the caller's for every group leaves that of its own master (two complex64 vectors) for the other two.
-    bool wide_out = P.ir;
-    for (int gi = 0; gi < ngroups; ++gi) wide_out = wide_out && groups[gi].u64;
-    P.ring_in_x64 = !boxes && wide_out;
-    P.pslots = (o->dtype == WRI_C64 && cfg == 24 && (boxes || wide_out)) ? 4 : 2;
+    // complex128 keeps two direction slots: the same bytes per iteration as an update in every one.  So do large complex64
+    // batches the boxes cannot take, whose workspace never had room for four (kRingRoom).
+    double ring = 0.0;
+    for (int gi = 0; gi < ngroups; ++gi) ring += 16.0 * groups[gi].nsys * (double)grid_n(groups[gi].grid);
+    P.pslots = (o->dtype == WRI_C64 && cfg == 24 && (boxes || ring <= kRingRoom)) ? 4 : 2;
     P.xsteps = cfg == 18 ? 1 : P.pslots;
   } else if (boxes) {
     P.tma_cfg = o->kernel >= 2 ? o->kernel - 2 : kBoxTmaCfg;
@@ -500,7 +501,7 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
     P.v_p[gi][0] = off; off += vb;
     P.v_p[gi][1] = off; off += vb;
     P.v_p[gi][2] = P.v_p[gi][3] = 0;
-    if (P.pslots == 4 && !P.ring_in_x64) {
+    if (P.pslots == 4) {
       P.v_p[gi][2] = off; off += vb;
       P.v_p[gi][3] = off; off += vb;
     }
@@ -515,10 +516,6 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
       P.v_q64[gi] = off; off += align_up(16 * nn);
       P.v_g32[gi] = off; off += align_up(8 * nn);
       P.v_rmap[gi] = off; off += align_up(4 * nn);
-      if (P.pslots == 4 && P.ring_in_x64) {
-        P.v_p[gi][2] = P.v_x64[gi];
-        P.v_p[gi][3] = P.v_x64[gi] + 8 * nn;
-      }
     }
   }
   P.total = off;

@@ -34,9 +34,7 @@ def test_grouped_updates_equal_single_updates(W, nphys, dtype):  # noqa: F811
 
 
 def test_grouped_updates_of_refined_solves_on_an_odd_extent(W):  # noqa: F811
-    """With an FP64 array of the caller's the slots of two of the four directions lie in the workspace of the
-    refinement's own FP64 solution, which is then unused: the same wavefields, bit for bit, as with two slots in
-    the solve without such an array and as with single updates, over several outer steps."""
+    """The same over several outer steps of a refined solve, with and without an FP64 array of the caller's."""
     G = case(nphys=(29, 12, 11), npml=4, nsys=3, seed=12)
     out = []
     for cfg, wide in ((18, True), (24, True), (22, False), (24, False)):

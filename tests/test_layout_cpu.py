@@ -7,7 +7,7 @@ import subprocess
 import numpy as np
 import pytest
 
-from test_abi_cpu import W, _FakeTensor, _spec  # noqa: F401  (W: fixture)
+from test_abi_cpu import W, _spec  # noqa: F401  (W: fixture)
 
 PROBE = r"""
 #include "wri_api.cu"
@@ -115,19 +115,18 @@ def test_iterations_per_iterate_update_of_the_chunk_configurations(W, probe, dty
 
 
 def test_workspace_of_batches_that_the_boxes_cannot_take(W, probe):  # noqa: F811
-    """An x extent that is not a multiple of 4: two direction slots, as on the z-march kernels, so that what fitted
-    the device there fits it on the chunk kernels too (but for layer tables and the shape of the receiver bits).  A
-    refined solve into an FP64 array of the caller's has four, in the same bytes."""
-    n, nsys = 21 * 18 * 16, 2
-    refined = dict(max_refine=2, refine_tol=1e-8, inner_tol=1e-2)
-    for dtype in (0, 1):
-        march = W.workspace_size([_spec(W, nx=21)], W.make_opts(dtype=dtype, kernel=W.KERNEL_MARCH))
-        for kernel in (0, W.KERNEL_TMA(24)):
-            assert _plan(W, probe, _spec(W, nx=21), dtype=dtype, kernel=kernel) == (1, 2, 2)
-            assert W.workspace_size([_spec(W, nx=21)], W.make_opts(dtype=dtype, kernel=kernel)) < march + n * nsys
-    for u64, slots in ((None, 2), (_FakeTensor(0x20000), 4)):
-        spec = _spec(W, nx=21, u64=u64)
-        assert _plan(W, probe, spec, **refined) == (1, slots, slots)
-        assert (W.workspace_size([spec], W.make_opts(**refined))
-                == W.workspace_size([_spec(W, nx=21)], W.make_opts(**refined)))
-    assert _plan(W, probe, _spec(W), kernel=0) == (1, 4, 4)
+    """An x extent that is not a multiple of 4: large batches have two direction slots, as on the z-march kernels, so
+    that what fitted the device there fits it on the chunk kernels too (but for layer tables and the shape of the
+    receiver bits); the two slots more of the others take at most 1 GiB."""
+    def vectors(spec, **kw):  # complex64 vectors beyond the z-march workspace, in bytes per node and system
+        n = spec.nx * spec.ny * spec.nz * len(spec.src)
+        march = W.workspace_size([spec], W.make_opts(kernel=W.KERNEL_MARCH, **kw))
+        return [round((W.workspace_size([spec], W.make_opts(kernel=k, **kw)) - march) / n) for k in (0, W.KERNEL_TMA(24))]
+
+    for kw in (dict(), dict(max_refine=2, refine_tol=1e-8, inner_tol=1e-2)):
+        for nx, ny, nz, slots in ((81, 80, 80, 4), (405, 408, 406, 4), (407, 410, 406, 2), (801, 400, 400, 2)):
+            spec = _spec(W, nx=nx, ny=ny, nz=nz, src=np.array([0]), rec_off=np.array([0, 5]))
+            assert _plan(W, probe, spec, kernel=0, **kw) == (1, slots, slots), nx
+            assert vectors(spec, **kw) == [16 if slots == 4 else 0] * 2, nx
+    assert _plan(W, probe, _spec(W, nx=21), dtype=1, kernel=0) == (1, 2, 2)
+    assert _plan(W, probe, _spec(W, nx=800, ny=400, nz=400), kernel=0) == (1, 4, 4)
