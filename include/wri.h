@@ -127,7 +127,8 @@ typedef struct {
   int32_t plain;       /* 1: unbatched, unfused baseline (one system at a time, separate
                           BLAS-1 kernels, scalars read back by the host every iteration) */
   int32_t poll_every;  /* CG iterations per body of the device-side loop, between two runs of
-                          its control kernel (0 = library default, about 300 us of work) */
+                          its control kernel (0 = library default, about 300 us of work); the chunk
+                          kernels round it up to a multiple of the iterations per iterate update */
   int32_t tile;        /* tile configuration (0 = autotuned / default, see wri_tile_count) */
   int32_t zsplit;      /* z-chunks per tile column (0 = chosen from the batch size) */
   int32_t kernel;      /* 0 = automatic (the chunk kernels, as configuration 24), 1 = z-march
@@ -145,7 +146,10 @@ typedef struct {
                            2 = 64 B, 3 = 128 B, 4 = 256 B */
   int32_t wait_limit_us; /* chunk and TMA phases: time limit of every wait of the copy pipelines, in
                             microseconds (0 = 2 s).  A wait that runs out stops the solve:
-                            wri_solve_batch returns WRI_ECUDA and the context stays usable. */
+                            wri_solve_batch returns WRI_ECUDA and the context stays usable.  The calls
+                            that only enqueue work (wri_apply_A, wri_apply_AH, wri_gradient and its
+                            variant without allocation) wait 2 s and cannot return it: y holds NaN where
+                            such a wait ran out and is otherwise undefined, or *f is NaN and grad undefined. */
   int32_t host_loop;     /* 1: the host replays a graph of poll_every iterations and reads the
                             counters after each replay, instead of the device-side loop (a graph
                             WHILE node).  Kernel profilers cannot see kernels inside conditional

@@ -205,9 +205,9 @@ int auto_zsplit_lin(long long xy_items, int nz) {
 // fullest SM: two items at a time, a plane of one item takes 1.3 us and 0.0063 us per node on its own, two items
 // the FP64 pipe's 0.0245 us per node, and an item 0.7 planes more than it has.  Chunks below 256 nodes only while
 // an SM has at most two items (with more, the fuller CTAs win: 81^3 x 9 883 us per iteration against 890-1010).
-// The sweep over both that set these (the pipe has a little less to do now: 36^3 x 1 38.8, 81^3 x 9 804) gave,
-// in us per iteration: 36^3 x 1 39 (whole columns of 256 nodes: 228), 48^3 x 4 118 (337),
-// 81^3 x 9 883 (1057), 116^3 x 4 1031 (1358).
+// The sweep over both that set the constants covered the four batches below and nothing else; the rule extrapolates
+// to other sizes.  It gave, in us per iteration, 36^3 x 1 39 (whole columns of 256 nodes: 228), 48^3 x 4 118
+// (337), 81^3 x 9 883 (1057), 116^3 x 4 1031 (1358); now 41, 128, 871 and 1115.
 void wide_shape(const wri_grid* grids, const int* nsys, int ngroups, int* most, int* zsplit) {
   double best_cost = 0.0;
   int nz = 0;
@@ -340,7 +340,7 @@ bool host_loop_forced() {
 // z-march kernels or a z-march tile are asked for.  Microseconds per system and iteration against the
 // boxes of configuration 9 (and of 24): 148^3 x 32 systems 41.7 (58.6, 52.5), 116^3 x 32 20.9 (31.4, 28.7),
 // 84^3 x 48 9.3 (84^3 x 64: 12.3, 11.2), one 148^3 71 (92, 86); against the z-march kernels on 81^3 x 9 with
-// 2025 receivers: 13.6 (41) in complex64.
+// 2025 receivers: 14.0 (41) in complex64.
 bool lin_config(int cfg) { return cfg == 18 || cfg == 22 || cfg == 24; }
 
 void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, Plan& P) {
@@ -1382,7 +1382,7 @@ int apply_common(const wri_grid* grid, int dtype, const void* m, int nsys, const
   b.nitems = G.nitems;
   const int rb = dtype == WRI_C128 ? 8 : 4;
   // The chunk kernel, where the layer table fits its arguments and the arrays have their natural alignment
-  // (complex128, A^H on 81^3 x 9: 264 us against the z-march kernel's 1387; a single complex64 36^3 is bound
+  // (complex128, A^H on 81^3 x 9: 297 us against the z-march kernel's 1387; a single complex64 36^3 is bound
   // by the call).
   if (grid->npml < kLinInlineTab && (long long)grid->nx * grid->ny < (1LL << 28) && (uintptr_t)m % rb == 0 &&
       ((uintptr_t)x | (uintptr_t)y) % vb == 0 && lin_smem(b, rb, M_APPLY) <= (size_t)kLinMaxSmem) {

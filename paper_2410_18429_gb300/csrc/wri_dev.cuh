@@ -19,7 +19,7 @@ constexpr int kXupdNodes = 4096;  // nodes of a work item of the iterate-update 
 
 // z-chunk of the gradient kernel (its FP64 accumulator tile lives in shared memory: 16 KB at 8 rows, so that
 // registers and not shared memory decide how many CTAs an SM holds)
-__host__ __device__ constexpr int grad_zc(int by) { return by >= 16 ? 8 : 8; }
+__host__ __device__ constexpr int grad_zc(int) { return 8; }
 
 // squared slowness at a node, in the precision of the caller's model array (double only under FP64 stencils)
 template <typename R>

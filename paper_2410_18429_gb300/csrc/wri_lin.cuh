@@ -27,14 +27,10 @@
 // is its own new value), computes plane k's without the z + 1 term and hands the stage back, so S - 1
 // planes stay in flight.
 //
-// What binds: complex64 phases move 32 bytes per node and reach 5.4 TB/s in phase 1 (148^3 x 16, ncu) at 50 %
-// issue utilisation, 270 warp instructions per 64 nodes and plane (320 in the boxes, 374 before the warps
-// without stretched nodes and the z layers got loops of their own).  Running addresses in the copy warp, no
-// plane or lane checks in the main loop and one set of y coefficients per pair: 148^3 x 32 46.8 -> 45.8 us
-// per system and iteration (41.7 with the shorter end of a phase), 84^3 x 64 9.0 -> 8.7.  Chunks of 512 nodes
-// (half the halo) are slower: 47.8 and 9.4, 276 x 276 x 180 x 4 181 against 173.  Stages beyond three are slower
-// (the plane streams alone: 749 against 550 us with six).  complex128 passes are bound by the FP64 pipe (86-90 %
-// busy).
+// What binds: the complex64 phases run at 5.5 TB/s of DRAM traffic (148^3 x 16) with half of the issue slots
+// used, 253 (phase 1) and 262 (phase 2) warp instructions per 64 nodes and plane; FP64 passes run the FP64 pipe at
+// 87-89 %.  Chunks of 512 nodes (half the halo) are slower (148^3 x 32 45.8 -> 47.8 us per system and iteration,
+// 276 x 276 x 180 x 4 173 -> 181), and so are stages beyond three (the plane streams alone 550 -> 749 us with six).
 //
 // All waits are bounded as in wri_tma.cuh: a time-out raises the CTA's abort flag and the launch's error
 // flag, the consumers leave on a barrier-reduced copy of it, and the copy warp waits for its own copies.
@@ -199,9 +195,9 @@ __device__ void finalize_lin(const Batch& b, const GroupDev& G, SysDev* sd, int 
 }
 
 // R: arithmetic; OR: type of the stencil's output vector; MODE: M_APPLY, M_SH, M_RES, M_P1, M_P2 or M_GRAD; NC
-// consumer threads of NPT nodes each; GV: phase 2 adds S^H r64 (gvec); PAIR: a thread's two nodes are adjacent (16-byte accesses: nx even
-// and every pointer aligned), otherwise they lie NC apart; S stages; XO:
-// warps outside the y layers have loops of their own.
+// consumer threads of NPT nodes each; GV: phase 2 adds S^H r64 (gvec); PAIR: a thread's two nodes are adjacent
+// (16-byte accesses: nx even and every pointer aligned), otherwise they lie NC apart; S stages; XO: warps outside
+// the y layers have loops of their own.
 template <typename R, typename OR, int MODE, bool CONJ, int NC, int NPT, bool PAIR, bool GV, int S, int MINB, bool XO>
 __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ Batch b, const __grid_constant__ LinSet T,
                                                          const __grid_constant__ LinTab<MODE> tab_in) {
@@ -489,8 +485,8 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
     // gradient: the finished plane kp, accumulated over the systems.  t is the stencil without the node factor
     // w = s_x s_y s_z, which leaves the sums: with A u - c = w t', t' = t - c / w,
     //   Re(conj(w u) w t') = |w|^2 Re(conj(u) t'),  |w t'|^2 = |w|^2 |t'|^2,
-    // and |w|^2 enters the gradient once, after the last system (9 to 12 FP64 instructions less per node and
-    // system in the layer: 148^3 x 16 3.82 -> 2.99 ms).
+    // and |w|^2 enters the gradient once, after the last system: 9 to 12 FP64 instructions less per node and
+    // system in the layer, 22 % of the time on 148^3 x 16.
     auto accum = [&](int kp, C (&t)[NPT], bool g, bool z) {
 #pragma unroll
       for (int r = 0; r < NPT; ++r) {
@@ -579,7 +575,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
       }
       pO += plane;
       // FP64: straight into the sum (three additions of zero less).  With the model and the complex64 output
-      // converted in integers: 116^3 x 32 M_SH 3016 -> 2686 us, M_RES 2639 -> 2531.
+      // converted in integers this took 11 % off M_SH and 4 % off M_RES (116^3 x 32).
       if (NORM && sizeof(R) == 8) {
 #pragma unroll
         for (int r = 0; r < NPT; ++r)
@@ -618,8 +614,10 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
     // gen_c: 1 the x coefficients are general, 2 those of x and y; zg_c: plane k lies in a z layer.  XO (FP64)
     // has a kind of its own for x alone, with 10 FP64 instructions of 37 less (the phases 6: their kernels with
     // and without it round alike): of the warps of 81^3 two thirds have an x layer, of 148^3 a third, most of
-    // them outside the y layers.  The phases take it for items of 8 planes and more: with items of 3 planes
-    // (36^3 x 1) the additional loops cost 3 % of the iteration, with 17 to 50 (81^3 x 9, 148^3 x 1) they gave 3 to 4 %.
+    // them outside the y layers.  The phases take it for items of 8 planes and more, where the additional loops
+    // pay: us per iteration without and with it, items of 2 and 3 planes 40.6 / 41.4 (36^3 x 1) and 128.0 / 125.8
+    // (48^3 x 4), of 9 to 50 planes 912 / 871 (81^3 x 9), 485 / 475 (84^3 x 4), 1155 / 1115 (116^3 x 4), 602 / 584
+    // (148^3 x 1) and 140.4 / 141.7 (81^3 x 1).  Nothing between 3 and 9 planes was measured.
     auto step = [&](auto gen_c, auto zg_c, int k) -> bool {
       constexpr bool GEN = decltype(gen_c)::value > 0, GY = decltype(gen_c)::value == 2, ZG = decltype(zg_c)::value;
       if (!wait()) return false;
