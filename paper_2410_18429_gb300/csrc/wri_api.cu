@@ -5,7 +5,6 @@
 
 #include <algorithm>
 #include <cmath>
-#include <complex>
 #include <cstdlib>
 #include <cstring>
 #include <memory>
@@ -112,23 +111,62 @@ void fill_geom(GroupDev& G, const wri_grid& g) {
   G.n = grid_n(g);
 }
 
+// Real numbers as unevaluated sums of two doubles (about 100 bits), for coefficients that are rounded once.
+struct Dbl2 {
+  double hi, lo;
+  explicit operator double() const { return hi; }
+};
+Dbl2 sum2(double a, double b) {  // Knuth's exact sum
+  const double s = a + b, bb = s - a;
+  return {s, (a - (s - bb)) + (b - bb)};
+}
+Dbl2 operator+(Dbl2 a, Dbl2 b) {
+  const Dbl2 s = sum2(a.hi, b.hi);
+  return sum2(s.hi, s.lo + (a.lo + b.lo));
+}
+Dbl2 operator-(Dbl2 a) { return {-a.hi, -a.lo}; }
+Dbl2 operator*(Dbl2 a, Dbl2 b) {
+  const double p = a.hi * b.hi;
+  return sum2(p, std::fma(a.hi, b.hi, -p) + (a.hi * b.lo + a.lo * b.hi));
+}
+Dbl2 operator/(Dbl2 a, Dbl2 b) {
+  const double q = a.hi / b.hi;
+  const Dbl2 r = a + -(b * Dbl2{q, 0.0});
+  return sum2(q, (r.hi + r.lo) / b.hi);
+}
+
 // Layer table of the chunk kernels (kLayerTab): entries for nodes 0 .. npml cells inside the layer, in FP64.
 // The same entries serve the three axes and both faces, since the profile depends on the distance alone.
+// With s = 1 + i t at the node and 1 + i r at the half point, alpha = (1 - i t) (1 - i r) / (|s|^2 |s(half)|^2 h^2).
+// Every entry is rounded once: in plain FP64 (complex divisions) the coefficients carried most of the error of the
+// complex128 stencils in the layer, 7.0 units (2^-53 u / h^2, root mean square) where one axis is stretched and 18.2
+// where all three are, against 5.5 and 12.9 now (864 damped waves on four grids; z-march kernels 6.1 and 16.3).
+// Takes less than 1 us of host time per call.
 void layer_table(const wri_grid& g, std::vector<double>& t) {
-  typedef std::complex<double> Z;
   t.assign((size_t)(g.npml + 1) * kLayerTab, 0.0);
-  const AxisPml a = axis(g.nx, g);
-  auto stretch = [&](double cells) -> Z {
-    const double q = std::max(cells, 0.0) * a.h * a.invL;
-    return Z(1.0, a.smax * q * q * a.inv_omega);
-  };
+  const Dbl2 one = {1.0, 0.0}, h2 = Dbl2{g.h, 0.0} * Dbl2{g.h, 0.0};
+  Dbl2 unit = {0.0, 0.0};  // Im s one cell inside the layer
+  if (g.npml > 0)
+    unit = Dbl2{axis(g.nx, g).smax, 0.0} / (Dbl2{(double)g.npml * g.npml, 0.0} * Dbl2{g.omega, 0.0});
+  auto imag = [&](double cells) { return unit * Dbl2{cells * cells, 0.0}; };
+  // the nearer (0) and the farther (1) half point: Im s, 1 / (|s|^2 h^2)
+  Dbl2 r[2] = {{0.0, 0.0}, {0.0, 0.0}}, w[2] = {one / h2, one / h2};
   for (int d = 0; d <= g.npml; ++d) {
-    const Z s = stretch(d), ih2 = Z(1.0 / (g.h * g.h), 0.0);
-    const Z near_ = ih2 / stretch(d - 0.5), far_ = ih2 / stretch(d + 0.5);
-    const Z an = near_ / s, af = far_ / s, a0 = -(an + af);
-    const double e[kLayerTab] = {an.real(), an.imag(), af.real(), af.imag(), a0.real(), a0.imag(), s.imag(), 0.0,
-                                 near_.real(), near_.imag(), far_.real(), far_.imag()};
-    std::copy(e, e + kLayerTab, t.begin() + (size_t)d * kLayerTab);
+    r[1] = imag(d + 0.5);
+    w[1] = one / ((one + r[1] * r[1]) * h2);
+    const Dbl2 s = imag(d), is2 = one / (one + s * s);
+    Dbl2 alpha[2][2];  // [nearer, farther][real, imaginary]
+    for (int f = 0; f < 2; ++f) {
+      const Dbl2 ws = w[f] * is2;
+      alpha[f][0] = (one + -(r[f] * s)) * ws;
+      alpha[f][1] = -((r[f] + s) * ws);
+    }
+    const Dbl2 e[kLayerTab] = {alpha[0][0], alpha[0][1], alpha[1][0], alpha[1][1],
+                               -(alpha[0][0] + alpha[1][0]), -(alpha[0][1] + alpha[1][1]), s, {0.0, 0.0},
+                               w[0], -(r[0] * w[0]), w[1], -(r[1] * w[1])};
+    for (int i = 0; i < kLayerTab; ++i) t[(size_t)d * kLayerTab + i] = (double)e[i];
+    r[0] = r[1];
+    w[0] = w[1];
   }
 }
 
