@@ -245,7 +245,7 @@ int auto_zsplit_lin(long long xy_items, int nz) {
 // an SM has at most two items (with more, the fuller CTAs win: 81^3 x 9 883 us per iteration against 890-1010).
 // The sweep over both that set the constants covered the four batches below and nothing else; the rule extrapolates
 // to other sizes.  It gave, in us per iteration, 36^3 x 1 39 (whole columns of 256 nodes: 228), 48^3 x 4 118
-// (337), 81^3 x 9 883 (1057), 116^3 x 4 1031 (1358); now 41, 128, 871 and 1115.
+// (337), 81^3 x 9 883 (1057), 116^3 x 4 1031 (1358); now 39, 127, 877 and 1140.
 void wide_shape(const wri_grid* grids, const int* nsys, int ngroups, int* most, int* zsplit) {
   double best_cost = 0.0;
   int nz = 0;
@@ -1420,7 +1420,7 @@ int apply_common(const wri_grid* grid, int dtype, const void* m, int nsys, const
   b.nitems = G.nitems;
   const int rb = dtype == WRI_C128 ? 8 : 4;
   // The chunk kernel, where the layer table fits its arguments and the arrays have their natural alignment
-  // (complex128, A^H on 81^3 x 9: 297 us against the z-march kernel's 1387; a single complex64 36^3 is bound
+  // (complex128, A^H on 81^3 x 9: 305 us against the z-march kernel's 1387; a single complex64 36^3 is bound
   // by the call).
   if (grid->npml < kLinInlineTab && (long long)grid->nx * grid->ny < (1LL << 28) && (uintptr_t)m % rb == 0 &&
       ((uintptr_t)x | (uintptr_t)y) % vb == 0 && lin_smem(b, rb, M_APPLY) <= (size_t)kLinMaxSmem) {

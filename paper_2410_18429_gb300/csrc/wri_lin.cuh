@@ -211,10 +211,13 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
   constexpr int NCW = NC / 32;
   constexpr bool GRAD = MODE == M_GRAD;
   // The stencil is formed from differences to the node, which are exact or nearly so for a resolved field, so
-  // that the rounding of a coefficient acts on a difference.  complex128 takes the unstretched axes together,
-  // as the sum of their neighbours minus 6 (or 4, 2) u: fewer FP64 instructions.  The diagonal in one coefficient
-  // would save 2 (interior) to 8 (x and y layer) of 17 to 37 more (A^H on 81^3 x 9 297 -> 264 us), but its
-  // error is up to four times as large (A u of plane waves, 116 x 60 x 80 with 10 cells: 4.0e-15 against 1.1e-15).
+  // that the rounding of a coefficient acts on a difference.  complex128 takes an unstretched axis as the sum of
+  // its two neighbours minus 2 u (fewer FP64 instructions), and x and y together as four minus 4 u where both are.
+  // Its root mean square error is 1.8 units (2^-53 u / h^2) off the layers, 2.9 at a source, 5.4 where one axis is
+  // stretched and 12.9 where all are (damped outgoing waves, 864 on four grids; z-march kernels 1.9, 3.2, 6.1, 16.3).
+  // Cheaper forms lose: five neighbours in one sum saves 2 FP64 instructions of 19 off the layers (A^H on 81^3 x 9
+  // 305 -> 297 us) but has 2.3 units there and 3.4 at a source, and the diagonal in one coefficient saves 4 of 19 to
+  // 8 of 37 (264 us) at up to four times the error.
   constexpr bool DIFF = sizeof(R) == 4;
   // complex64: the first step of an item finishes a plane below it all the same (no check in the loop) and
   // its result is overwritten; complex128 saves the FP64 instructions
@@ -433,8 +436,9 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
     // sum of |output|^2: FP32 over 4 planes, then FP64 (pairs past the chunk's end are left out at the end)
     R accf = R(0);
     C fc[NPT], q[NPT];
+    C zm[NPT];  // complex128: the z - 1 neighbour of a pending plane off the z layers
 #pragma unroll
-    for (int r = 0; r < NPT; ++r) fc[r] = q[r] = czero<R>();
+    for (int r = 0; r < NPT; ++r) fc[r] = q[r] = zm[r] = czero<R>();
     C hz = mkc(ih2, R(0));  // weight of the z + 1 neighbour of the pending plane
     R hs = R(0);            // gradient: Im s_z of the pending plane
     if constexpr (GRAD)
@@ -612,12 +616,12 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
     }
     // One plane of the item: its F, the z + 1 term of plane k - 1, and its own stencil without that term.
     // gen_c: 1 the x coefficients are general, 2 those of x and y; zg_c: plane k lies in a z layer.  XO (FP64)
-    // has a kind of its own for x alone, with 10 FP64 instructions of 37 less (the phases 6: their kernels with
+    // has a kind of its own for x alone, with 8 FP64 instructions of 37 less (the phases 6: their kernels with
     // and without it round alike): of the warps of 81^3 two thirds have an x layer, of 148^3 a third, most of
     // them outside the y layers.  The phases take it for items of 8 planes and more, where the additional loops
-    // pay: us per iteration without and with it, items of 2 and 3 planes 40.6 / 41.4 (36^3 x 1) and 128.0 / 125.8
-    // (48^3 x 4), of 9 to 50 planes 912 / 871 (81^3 x 9), 485 / 475 (84^3 x 4), 1155 / 1115 (116^3 x 4), 602 / 584
-    // (148^3 x 1) and 140.4 / 141.7 (81^3 x 1).  Nothing between 3 and 9 planes was measured.
+    // pay: us per iteration without and with it, items of 2 and 3 planes 39.3 / 40.7 (36^3 x 1) and 127.0 / 125.2
+    // (48^3 x 4), of 9 to 50 planes 923 / 878 (81^3 x 9), 493 / 479 (84^3 x 4), 1181 / 1141 (116^3 x 4), 609 / 589
+    // (148^3 x 1) and 141.4 / 142.4 (81^3 x 1).  Nothing between 3 and 9 planes was measured.
     auto step = [&](auto gen_c, auto zg_c, int k) -> bool {
       constexpr bool GEN = decltype(gen_c)::value > 0, GY = decltype(gen_c)::value == 2, ZG = decltype(zg_c)::value;
       if (!wait()) return false;
@@ -684,7 +688,8 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         C t[NPT];
 #pragma unroll
         for (int r = 0; r < NPT; ++r) {
-          t[r] = ZG ? cfma(hz, v[r] - fc[r], q[r]) : rfma(ih2, DIFF ? v[r] - fc[r] : v[r], q[r]);
+          if (ZG) t[r] = cfma(hz, v[r] - fc[r], q[r]);
+          else t[r] = rfma(ih2, DIFF ? v[r] - fc[r] : rfma(R(-2), fc[r], zm[r] + v[r]), q[r]);
           if (GEN && !GRAD) t[r] = smul(sx_[r], t[r]);
           if (GY && !GRAD) t[r] = smul(sy_[PAIR ? 0 : r], t[r]);
         }
@@ -723,41 +728,36 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         const R c = om2 * mk[r];
         C acc;
         if (DIFF) {
-          const C zm = fc[r] - v[r];
+          const C dz = fc[r] - v[r];
           acc = mkc(c * v[r].x, c * v[r].y);
           if (GEN) {
             acc = cfma(am[r], l[r], acc);
             acc = cfma(ap[r], rgt[r], acc);
             acc = GY ? cfma(bm[PAIR ? 0 : r], ym[r], acc) : rfma(ih2, ym[r], acc);
             acc = GY ? cfma(bp[PAIR ? 0 : r], yp[r], acc) : rfma(ih2, yp[r], acc);
-            acc = ZG ? cfma(cz.am, zm, acc) : rfma(ih2, zm, acc);
+            acc = ZG ? cfma(cz.am, dz, acc) : rfma(ih2, dz, acc);
           } else {
             C sum = (l[r] + rgt[r]) + (ym[r] + yp[r]);
-            if (!ZG) sum = sum + zm;
+            if (!ZG) sum = sum + dz;
             acc = rfma(ih2, sum, acc);
-            if (ZG) acc = cfma(cz.am, zm, acc);
+            if (ZG) acc = cfma(cz.am, dz, acc);
           }
         } else {
           // In a z layer every term but omega^2 m u is a difference: these first, then that one in one rounding.
           // The phases have kernels with and without the loops for x alone (XO), which have to round alike.
           constexpr bool YD = GY || (GEN && HASB);
-          constexpr int axes = 6 - (GEN ? 2 : 0) - (YD ? 2 : 0) - (ZG ? 2 : 0);
           acc = ZG ? cmul(cz.am, fc[r] - v[r]) : mkc(c * v[r].x, c * v[r].y);
-          C sum = fc[r];  // neighbours on the unstretched axes but for z + 1
-          if (GEN) {
-            acc = cfma(am[r], l[r] - v[r], acc);
-            acc = cfma(ap[r], rgt[r] - v[r], acc);
-          }
-          if (YD) {
-            acc = GY ? cfma(bm[PAIR ? 0 : r], ym[r] - v[r], acc) : rfma(ih2, ym[r] - v[r], acc);
-            acc = GY ? cfma(bp[PAIR ? 0 : r], yp[r] - v[r], acc) : rfma(ih2, yp[r] - v[r], acc);
+          if (!GEN && !ZG) {
+            acc = rfma(ih2, rfma(R(-4), v[r], (l[r] + rgt[r]) + (ym[r] + yp[r])), acc);
           } else {
-            sum = ym[r] + yp[r];
-            if (!GEN) sum = (l[r] + rgt[r]) + sum;
-            if (!ZG) sum = sum + fc[r];
+            if (GEN) acc = cfma(ap[r], rgt[r] - v[r], cfma(am[r], l[r] - v[r], acc));
+            else acc = rfma(ih2, rfma(R(-2), v[r], l[r] + rgt[r]), acc);
+            if (GY) acc = cfma(bp[r], yp[r] - v[r], cfma(bm[r], ym[r] - v[r], acc));
+            else if (YD) acc = rfma(ih2, yp[r] - v[r], rfma(ih2, ym[r] - v[r], acc));
+            else acc = rfma(ih2, rfma(R(-2), v[r], ym[r] + yp[r]), acc);
           }
-          if (axes > 0) acc = rfma(ih2, rfma(R(-axes), v[r], sum), acc);
           if (ZG) acc = rfma(c, v[r], acc);
+          zm[r] = fc[r];
         }
         q[r] = ZG && !GRAD ? smul(cz.im, acc) : acc;
         fc[r] = v[r];
@@ -777,10 +777,10 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
       for (; k < za; ++k)
         if (!step(gen_c, std::true_type(), k)) return false;
       const int kl = k;
-      // complex128: the z + 1 term of an interior plane lacks -u / h^2, which its q holds
+      // complex128: a pending plane of the layer (where 1 / s(half) = 1) lacks (up - u) / h^2 alone
       if (!DIFF && k < zb) {
 #pragma unroll
-        for (int r = 0; r < NPT; ++r) q[r] = rfma(-ih2, fc[r], q[r]);
+        for (int r = 0; r < NPT; ++r) zm[r] = fc[r];
       }
       for (; k < zb; ++k)
         if (!step(gen_c, std::false_type(), k)) return false;
@@ -789,7 +789,7 @@ __global__ void __launch_bounds__(NC + 32, MINB) k_lin(const __grid_constant__ B
         hs = R(0);
         if (!DIFF) {
 #pragma unroll
-          for (int r = 0; r < NPT; ++r) q[r] = rfma(ih2, fc[r], q[r]);
+          for (int r = 0; r < NPT; ++r) q[r] = rfma(ih2, zm[r] - fc[r], q[r]);
         }
       }
       for (; k < z1; ++k)

@@ -65,3 +65,32 @@ def test_total_variation_of_equal_cells(W, slope):  # noqa: F811
     spec = W.GroupSpec(n, n, n, 0, 10.0, 60.0, 3000.0, None, None, None, None, None, 1.0, None)
     tv, _ = W.tv(spec, torch.from_numpy(m).cuda(), beta)
     assert abs(tv.item() - ref) <= 100 * U * ref, (tv.item() - ref) / ref / U
+
+
+@pytest.mark.parametrize("nphys,npml", [((150, 21, 20), 0), ((141, 20, 21), 4), ((33, 31, 40), 0)])
+def test_sums_of_neighbours_fp64(W, nphys, npml):  # noqa: F811
+    """A u and A^H u off the layers for u = 0.9 (1 + i) with random last bits: h = 8 makes 1 / h^2 exact and the exact
+    sums are integers.  What rounds are sums of two neighbours below 2 (by 2^-53 at the most, three axes) and of four
+    below 4 (by 2^-52); the differences that follow are below 2^-10, so everything else rounds by less than
+    2^-8 2^-53 together.  The error of a component is therefore at most 5 2^-53 / h^2 and that.  (Five neighbours in
+    one sum round by up to 2^-51 more.)"""
+    G = case(nphys=nphys, npml=npml, h=8.0, freq=0.5, nsys=2, with_data=False)
+    shape = G.spec.shape
+    rng = np.random.default_rng(9)
+    ints = np.int64(0.9 * 2 ** 53) + rng.integers(0, 2 ** 40, (2, 2, *shape))  # [system, component, z, y, x]
+    spec = _spec(W, G, 1)
+    spec.m = torch.full((G.spec.n,), 1.0 / 3000.0 ** 2, dtype=torch.float64, device="cuda")
+    vals = ints * 2.0 ** -53
+    u = torch.from_numpy(vals[:, 0] + 1j * vals[:, 1]).reshape(2, -1).cuda()
+    lap = -6 * ints[..., 1:-1, 1:-1, 1:-1]
+    for a in range(3):
+        for o in (0, 2):
+            cut = [slice(1, -1)] * 3
+            cut[a] = slice(o, o + shape[a] - 2)
+            lap = lap + ints[(..., *cut)]
+    ref = lap * 2.0 ** -59 + G.omega ** 2 / 3000.0 ** 2 * vals[..., 1:-1, 1:-1, 1:-1]
+    inner = (..., *[slice(npml, n - 2 - npml) for n in shape])  # nodes npml + 1 .. n - 2 - npml of an axis
+    for adjoint in (False, True):
+        y = W.apply_A(spec, u, adjoint=adjoint).cpu().numpy().reshape(2, *shape)[..., 1:-1, 1:-1, 1:-1]
+        err = np.abs((np.stack([y.real, y.imag], 1) - ref)[inner]).max() * 2.0 ** 59
+        assert err <= 5 + 2.0 ** -8, (adjoint, err)
