@@ -27,10 +27,11 @@
 // is its own new value), computes plane k's without the z + 1 term and hands the stage back, so S - 1
 // planes stay in flight.
 //
-// What binds: the complex64 phases run at 5.5 TB/s of DRAM traffic (148^3 x 16) with half of the issue slots
+// What binds: the complex64 phases run at 5.3 TB/s of DRAM traffic (148^3 x 16) with 55 to 57 % of the issue slots
 // used, 253 (phase 1) and 262 (phase 2) warp instructions per 64 nodes and plane; FP64 passes run the FP64 pipe at
-// 87-89 %.  Chunks of 512 nodes (half the halo) are slower (148^3 x 32 45.8 -> 47.8 us per system and iteration,
-// 276 x 276 x 180 x 4 173 -> 181), and so are stages beyond three (the plane streams alone 550 -> 749 us with six).
+// 87-89 % of its rate.  Chunks of 512 nodes (half the halo) are slower (148^3 x 32 45.8 -> 47.8 us per system and
+// iteration, 276 x 276 x 180 x 4 173 -> 181), and so are stages beyond three (the plane streams alone 550 -> 749 us
+// with six).
 //
 // All waits are bounded as in wri_tma.cuh: a time-out raises the CTA's abort flag and the launch's error
 // flag, the consumers leave on a barrier-reduced copy of it, and the copy warp waits for its own copies.
