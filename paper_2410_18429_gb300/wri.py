@@ -110,8 +110,9 @@ def _stream(stream=None):
     if stream is not None:
         return stream.cuda_stream
     import torch
-    # the handle of torch.cuda.current_stream(), without building a Stream object for it
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    # the handle of torch.cuda.current_stream(), without building a Stream object where PyTorch has the call for it
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return torch.cuda.current_stream().cuda_stream if raw is None else raw(torch.cuda.current_device())
 
 
 def _ptr(t) -> Optional[int]:
