@@ -218,13 +218,19 @@ int auto_zsplit(long long xy_items, int nz) {
   return best;
 }
 
+// CTAs of a complex64 chunk kernel that an SM holds: four by its registers, fewer where long rows of x (nx nodes on
+// either side of a chunk) make the stages large: from 424 nodes three, from 632 two, from 1032 one.
+int lin_resident(size_t smem) { return (int)std::min<size_t>(4, (228 << 10) / (smem + 1024 + 128)); }
+
 // The same for the chunk kernels, with chunks of at least one plane.  An item costs its planes and six more (its
-// halo planes, filling the stages, its end); the launch takes the mean of the full waves of 4 CTAs per SM, which is
+// halo planes, filling the stages, its end); the launch takes the mean of the full waves of resident CTAs, which is
 // right while the planes' latency binds, and of the exact count, which is right once the memory does.  Against a
-// sweep of 1..36 chunks over 14 batches this picks within 1.3 % of the best everywhere.  Full waves of planes plus
-// two lost up to 15 %: 116^3 x 4 131 us per iteration (now 114), 84^3 x 16 167 (156), 84^3 x 48 483 (447).
-int auto_zsplit_lin(long long xy_items, int nz) {
-  const long long wave = (long long)kRefSMs * 4;
+// sweep of 1..36 chunks over 14 batches with four CTAs this picks within 1.3 % of the best everywhere.  Full waves of
+// planes plus two lost up to 15 %: 116^3 x 4 131 us per iteration (now 114), 84^3 x 16 167 (156), 84^3 x 48 483 (447).
+// Counting four CTAs where long rows leave three lost up to 30 % on small batches (ps per node, system and iteration:
+// 448 x 40 x 40 x 1 66.8, now 51.2; 512 x 120 x 120 x 1 24.7, now 20.8).
+int auto_zsplit_lin(long long xy_items, int nz, int resident) {
+  const long long wave = (long long)kRefSMs * resident;
   int best = 1;
   double best_cost = 0.0;
   for (int zs = 1; zs <= 64 && zs <= nz; ++zs) {
@@ -394,6 +400,7 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
   for (int gi = 0; gi < ngroups; ++gi)
     boxes = boxes && (groups[gi].grid.nx % 4 == 0) && (P.ir || (uintptr_t)groups[gi].u % 16 == 0);
   const int cfg = o->kernel >= 2 ? o->kernel - 2 : kDefaultTmaCfg;
+  int resident = 4;
   if (!o->plain && o->kernel != 1 && lin_config(cfg) && (boxes || o->tile == 0)) {
     P.lin = true;
     P.pair = o->dtype == WRI_C64 ? 1 : 0;
@@ -412,6 +419,7 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
       probe.g[gi].m_double = o->dtype == WRI_C128 ? 1 : 0;
     }
     P.lin = P.lin && lin_smem(probe, (o->dtype == WRI_C128 || P.ir) ? 8 : 4, M_P1) <= (size_t)kLinMaxSmem;
+    resident = lin_resident(lin_smem(probe, 4, M_P1));
   }
   if (P.lin) {
     // complex128 keeps two direction slots: the same bytes per iteration as an update in every one.  So do large complex64
@@ -461,7 +469,7 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
     }
   }
   const int zs = o->zsplit > 0 ? o->zsplit
-                 : P.lin       ? auto_zsplit_lin(xy_items, nz_max)
+                 : P.lin       ? auto_zsplit_lin(xy_items, nz_max, resident)
                                : auto_zsplit(o->plain ? xy_items / std::max(1, P.nsys_total) : xy_items, nz_max);
   long long item = 0, parts = 0;
   int sys0 = 0;
@@ -1429,7 +1437,7 @@ int apply_common(const wri_grid* grid, int dtype, const void* m, int nsys, const
     b.sblock = 16;
     int most = kLinChunk, zs = 1;
     if (rb == 8) wide_shape(grid, &nsys, 1, &most, &zs);
-    else zs = auto_zsplit_lin((long long)nsys * lin_chunks(*grid), grid->nz);
+    else zs = auto_zsplit_lin((long long)nsys * lin_chunks(*grid), grid->nz, lin_resident(lin_smem(b, rb, M_APPLY)));
     decompose_lin(*grid, most, zs, G);
     G.nitems = (long long)G.ntiles * nsys;
     b.nitems = G.nitems;
