@@ -137,7 +137,9 @@ typedef struct {
                           iteration, 22 every second, 24 every fourth in complex64 where the
                           workspace has the directions for it), the others the
                           TMA box phases (9..24 warp-specialised; 23 updates the iterate every
-                          second iteration); see wri_autotune.  An explicit `tile` with a batch
+                          second iteration).  Complex64 batches with x extents of 632 and more that
+                          the boxes can take run on boxes in 18, 22 and 24 too, and on those of 9
+                          when automatic; see wri_autotune.  An explicit `tile` with a batch
                           the boxes cannot take runs on the z-march kernels. */
   int32_t order;       /* chunk and TMA phases: 0 = automatic (6), 1 = tiles of a system consecutive,
                           2 = systems of a tile consecutive, 3 = z-chunk slowest,

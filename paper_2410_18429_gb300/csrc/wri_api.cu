@@ -32,6 +32,7 @@ constexpr int kRefSMs = 152;  // SMs of a GB300; sets the z-split of small batch
 // wri_autotune refines the choice per batch.
 constexpr int kDefaultTmaCfg = 24;
 constexpr int kBoxTmaCfg = 9;   // where the chunk kernels cannot run (see plan_solve)
+constexpr int kLinResident = 3;  // CTAs per SM below which the boxes are faster (see plan_solve)
 constexpr int kFirstWsCfg = 9;  // configurations from here on are the warp-specialised kernels
 constexpr int kDefaultOrder = 6;
 constexpr int kDefaultPromotion = 2;
@@ -385,6 +386,11 @@ bool host_loop_forced() {
 // boxes of configuration 9 (and of 24): 148^3 x 32 systems 41.7 (58.6, 52.5), 116^3 x 32 20.9 (31.4, 28.7),
 // 84^3 x 48 9.3 (84^3 x 64: 12.3, 11.2), one 148^3 71 (92, 86); against the z-march kernels on 81^3 x 9 with
 // 2025 receivers: 14.0 (41) in complex64.
+// Batches the boxes can take with rows of 632 nodes and more, where the stages leave an SM fewer than kLinResident
+// CTAs, run on the boxes (of the same configuration if one is asked for).  ps per node, system and iteration, chunks
+// (boxes of configuration 9): 628 x 120 x 120 x 16 14.9 (17.1), 640 17.2 (15.7), 768 18.0 (16.7), 992 18.0 (16.7),
+// 1100 28.4 (17.6); 628 x 40 x 40 x 2 27.5 (31.6), 640 35.2 (30.7).  Refined solves too: over 200 iterations they gain
+// 5 to 8 % there, more than the z-march kernels take longer for the two FP64 passes (at 24 they lose 10 %).
 bool lin_config(int cfg) { return cfg == 18 || cfg == 22 || cfg == 24; }
 
 void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, Plan& P) {
@@ -420,6 +426,7 @@ void plan_solve(const wri_group* groups, int ngroups, const wri_solve_opts* o, P
     }
     P.lin = P.lin && lin_smem(probe, (o->dtype == WRI_C128 || P.ir) ? 8 : 4, M_P1) <= (size_t)kLinMaxSmem;
     resident = lin_resident(lin_smem(probe, 4, M_P1));
+    if (boxes && resident < kLinResident) P.lin = false;
   }
   if (P.lin) {
     // complex128 keeps two direction slots: the same bytes per iteration as an update in every one.  So do large complex64

@@ -67,3 +67,16 @@ def test_z_chunks_count_the_resident_ctas(plan, nx, ny, nsys):
     best = min(cost(-(-ny // zs)) for zs in range(1, min(ny, 64) + 1))
     zc = -(-ny // (items // columns))
     assert items % columns == 0 and cost(zc) <= best * (1 + 1e-12), (items, wave)
+
+
+@pytest.mark.parametrize("refined", [{}, dict(max_refine=1, refine_tol=1e-8, inner_tol=1e-2)])
+def test_long_rows_run_on_the_boxes(plan, refined):
+    """Below three CTAs per SM (rows of 632 nodes) the boxes are faster where they can take the batch: x extents that
+    are multiples of 4, complex64."""
+    assert plan(628, 40, 40, kernel=0, **refined)[0] == 1
+    for nx in (632, 768, 1600):
+        assert plan(nx, 40, 40, kernel=0, **refined)[:2] == (0, 9), nx
+        for cfg in (18, 22, 24):
+            assert plan(nx, 40, 40, kernel=2 + cfg, **refined)[:2] == (0, cfg), nx
+    assert plan(630, 40, 40, kernel=0, **refined)[0] == plan(770, 40, 40, kernel=0, **refined)[0] == 1
+    assert plan(768, 40, 40, kernel=0, dtype=1)[0] == 1
