@@ -129,4 +129,4 @@ def test_workspace_of_batches_that_the_boxes_cannot_take(W, probe):  # noqa: F81
             assert _plan(W, probe, spec, kernel=0, **kw) == (1, slots, slots), nx
             assert vectors(spec, **kw) == [16 if slots == 4 else 0] * 2, nx
     assert _plan(W, probe, _spec(W, nx=21), dtype=1, kernel=0) == (1, 2, 2)
-    assert _plan(W, probe, _spec(W, nx=800, ny=400, nz=400), kernel=0) == (1, 4, 4)
+    assert _plan(W, probe, _spec(W, nx=400, ny=800, nz=400), kernel=0) == (1, 4, 4)
